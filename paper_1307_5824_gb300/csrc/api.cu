@@ -171,6 +171,7 @@ size_t layout_workspace(const firm_params& p, char* base, Workspace& w) {
     w.cursor = c.take<uint32_t>(nb3);
     w.work = c.take<int4>(max_work);
     w.wmax_item = c.take<float>(max_work);
+    w.rec_item = c.take<int4>(max_work);
     w.scan_part = c.take<unsigned long long>(2 * (nb3 / kScanSpan + 1));
     w.item_part = c.take<double>(2 * max_work);
     w.counters = c.take<int>(8);
@@ -190,14 +191,28 @@ size_t layout_workspace(const firm_params& p, char* base, Workspace& w) {
     const size_t ids_bytes = (M * nH * sizeof(uint32_t) + 255) & ~(size_t)255;
     const size_t cls_bytes = (M * nH + 255) & ~(size_t)255;
     const size_t smp_bytes = (M * nH * sizeof(float2) + 255) & ~(size_t)255;
-    const size_t pay_bytes = ids_bytes + cls_bytes + smp_bytes + M * nH * sizeof(uint16_t);
-    const size_t u_bytes = std::max({M * N * N * esz, pay_bytes, (fx1 + fx2) * sizeof(float2) + 256});
+    const size_t pay_bytes = (ids_bytes + cls_bytes + smp_bytes + M * nH * sizeof(uint16_t) + 255) & ~(size_t)255;
+    // tensor-core spreading: 4 words a record slot for the kernel channel, 5 for A*b, 6 fused
+    const int nb_k = (int)nbk, nb_r = (int)(Gr / kBrick);
+    const bool mma_k = mma_rule(p, M * nH, nb_k, 1) || (fused && mma_rule(p, M * nH, nb_k, 3));
+    const size_t slots_k = mma_k ? mma_slots(M * nH, nb_k) : 0;
+    const size_t slots_r = mma_rule(p, M * nH, nb_r, 2) ? mma_slots(M * nH, nb_r) : 0;
+    const size_t rec_words = std::max(slots_k * (fused ? 6 : 4), slots_r * 5);
+    const size_t pts_bytes = (slots_k || slots_r) ? M * nH * (sizeof(uint4) + sizeof(float2)) : 0;
+    const size_t in_bytes = std::max(pay_bytes, (pts_bytes + 255) & ~(size_t)255);
+    const size_t rec_bytes = (rec_words * sizeof(uint32_t) + 255) & ~(size_t)255;
+    const size_t u_bytes = std::max({M * N * N * esz, in_bytes + rec_bytes + std::max(slots_k, slots_r) / 16,
+                                     (fx1 + fx2) * sizeof(float2) + 256});
     char* u = c.take<char>(u_bytes);
     w.images = u;
     w.payload = reinterpret_cast<uint32_t*>(u);
     w.cls = u ? reinterpret_cast<uint8_t*>(u + ids_bytes) : nullptr;
     w.samples_b = u ? reinterpret_cast<float2*>(u + ids_bytes + cls_bytes) : nullptr;
     w.perm = u ? reinterpret_cast<uint16_t*>(u + ids_bytes + cls_bytes + smp_bytes) : nullptr;
+    w.pts = reinterpret_cast<uint4*>(u);
+    w.pts_w = u ? reinterpret_cast<float2*>(u + M * nH * sizeof(uint4)) : nullptr;
+    w.rec = u ? reinterpret_cast<uint32_t*>(u + in_bytes) : nullptr;
+    w.rec_cls = u ? reinterpret_cast<uint8_t*>(u + in_bytes + rec_bytes) : nullptr;
     w.fx1 = reinterpret_cast<float2*>(u);
     w.fx2 = u ? reinterpret_cast<float2*>(u + ((fx1 * sizeof(float2) + 255) & ~(size_t)255)) : nullptr;
     w.ker = c.take<float>(H3);
@@ -613,7 +628,7 @@ int firm_kernel(firm_plan_t plan, int M, const double* R, const int32_t* group, 
     tm.start(0);
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
-    FIRM_CK(launch_bin(P, M, true));
+    FIRM_CK(launch_bin(P, M, true, true));
     tm.stop();
     tm.start(1);
     FIRM_CK(launch_spread(P, M, true));
@@ -672,7 +687,7 @@ int firm_backproject(firm_plan_t plan, int M, const void* images, const double* 
     if (from_stage) FIRM_CK(cudaEventRecord(P.ev_stage_read, P.stream));   // staging free again
     tm.stop();
     tm.start(5);
-    FIRM_CK(launch_bin(P, M, false));
+    FIRM_CK(launch_bin(P, M, false, true));
     tm.stop();
     tm.start(6);
     FIRM_CK(launch_spread(P, M, false));
@@ -701,19 +716,20 @@ int firm_kernel_backproject(firm_plan_t plan, int M, const void* images, const d
     FIRM_CK(e);
     P.ev_used[5] = P.ev_used[6] = false;      // no separate A*b binning or spreading stage here
     const bool staged = M > 0 && P.staged_host == images && P.staged_M == M;
-    // host images not staged ahead are copied into the workspace region the point ids
-    // use, so they are transformed before the binning; otherwise the binning (poses
-    // only) goes first, beside a staged upload
+    // the points are counted first (poses only, beside a staged upload).  Their ids are
+    // placed before the image DFT too, unless the tensor-core form places the A*b weights
+    // with them, or host images not staged ahead are copied into the workspace region the
+    // ids use
     const bool host_copy = M > 0 && !staged && !is_device(images);
     if (staged) FIRM_CK(start_stage(P));
     P.bin_M = -1;
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
-    if (!host_copy) {
-        tm.start(0);
-        FIRM_CK(launch_bin(P, M, true));
-        tm.stop();
-    }
+    tm.start(0);
+    FIRM_CK(launch_bin_count(P, M, 3, true));
+    const bool place_first = !host_copy && !P.bin_mma;
+    if (place_first) FIRM_CK(launch_bin_place(P, M, 3));
+    tm.stop();
     if (staged) {
         FIRM_CK(cudaStreamWaitEvent(P.stream, P.ev_staged, 0));     // the upload has landed
         P.cur_images = P.staged_dev;
@@ -729,12 +745,8 @@ int firm_kernel_backproject(firm_plan_t plan, int M, const void* images, const d
     FIRM_CK(launch_image_dft(P, M, P.cur_images, P.cur_shifts, P.cur_gid));
     if (staged) FIRM_CK(cudaEventRecord(P.ev_stage_read, P.stream));   // staging free again
     tm.stop();
-    if (host_copy) {
-        tm.start(0);
-        FIRM_CK(launch_bin(P, M, true));
-        tm.stop();
-    }
     tm.start(10);
+    if (!place_first) FIRM_CK(launch_bin_place(P, M, 3));
     FIRM_CK(launch_fused_gather(P, M));
     tm.stop();
     tm.start(1);
@@ -832,7 +844,7 @@ int firm_forward(firm_plan_t plan, int M, const float* V, const double* R, const
     FIRM_CK(stage_forward_inputs(P, M, V, R, group, Vd));
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += 1;
-    FIRM_CK(launch_bin(P, M, false));
+    FIRM_CK(launch_bin(P, M, false, false));
     float2* ghat = reinterpret_cast<float2*>(w.grid);
     FIRM_CK(launch_fwd_transform(P, Vd, ghat));
     const bool odev = is_device(out);
@@ -869,7 +881,7 @@ int firm_data_residual(firm_plan_t plan, int M, const float* V, const void* imag
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += 1;
     FIRM_CK(launch_image_dft(P, M, img, sh, P.cur_gid, true));    // b itself into samples
-    FIRM_CK(launch_bin(P, M, false));                                // b copied in scatter order
+    FIRM_CK(launch_bin(P, M, false, false));                                // b copied in scatter order
     float2* ghat = reinterpret_cast<float2*>(w.grid);
     FIRM_CK(launch_fwd_transform(P, Vd, ghat));
     FIRM_CK(launch_interp(P, M, ghat, nullptr, w.item_part, w.red_a));
@@ -1159,7 +1171,7 @@ int firm_bin(firm_plan_t plan, int M, const double* R, int channel) {
     FIRM_CK(e);
     FIRM_CK(launch_geom(Rd, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
-    FIRM_CK(launch_bin(P, M, channel == 0));
+    FIRM_CK(launch_bin(P, M, channel == 0, false));
     P.bin_M = M;
     P.bin_kc = channel == 0;
     P.have_kernel = P.have_rhs = false;      // the ids share memory with the other stages' buffers

@@ -33,8 +33,8 @@ struct firm_batch_s {
     // device workspace (caller's)
     char* desc_k = nullptr;                 // n spreading descriptors, kernel channel
     char* desc_r = nullptr;                 // n spreading descriptors, A*b channel
-    int* item_off = nullptr;                // 2 x (n + 1)
-    int* queue = nullptr;                   // 2
+    int* item_off = nullptr;                // per channel 2 x (n + 1) (spreading form)
+    int* queue = nullptr;                   // per channel 2
     // graph
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -75,7 +75,7 @@ size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 // [descriptors, kernel channel | descriptors, A*b channel | item offsets | queues |
 //  network inputs | network outputs | MLP scratch | CG state pointers | not-done count]
 size_t desc_region(int n) { return round256(desc_stride() * (size_t)n); }
-size_t off_region(int n) { return round256(2 * (size_t)(n + 1) * sizeof(int)); }
+size_t off_region(int n) { return round256(4 * (size_t)(n + 1) * sizeof(int)); }
 size_t net_region(int n) { return round256((size_t)n * 1024 * sizeof(float)); }
 size_t mlp_region(int n) { return round256(firm_mlp_work_floats(n) * sizeof(float)); }
 size_t ptr_region(int n) { return round256((size_t)n * sizeof(CgState*)); }
@@ -110,6 +110,13 @@ bool same_items(const std::vector<firm_batch_item>& a, const firm_batch_item* b,
         if (e_ != cudaSuccess) return e_;         \
     } while (0)
 
+// Plans of the batch whose points are spread in the tensor-core form.
+int count_mma(const firm_batch_s& b, const firm_batch_item* items, bool kc) {
+    int c = 0;
+    for (int i = 0; i < b.n; ++i) c += spread_uses_mma(b.plans[i]->P, items[i].M, kc ? 1 : 2) ? 1 : 0;
+    return c;
+}
+
 // Everything up to (not including) the kernel-channel spreading, for one plan.
 cudaError_t plan_front(Plan& P, const firm_batch_item& it, bool spread_here) {
     Workspace& w = P.ws;
@@ -123,7 +130,7 @@ cudaError_t plan_front(Plan& P, const firm_batch_item& it, bool spread_here) {
     BCK(cudaMemsetAsync(w.counters + 2, 0, sizeof(int), P.stream));
     BCK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
-    BCK(launch_bin(P, M, true));
+    BCK(launch_bin(P, M, true, true));
     BCK(launch_spread_clear(P, true));
     if (spread_here) BCK(launch_spread_only(P, M, true));
     P.last_M = M;
@@ -139,7 +146,7 @@ cudaError_t plan_middle(Plan& P, const firm_batch_item& it, bool spread_here) {
     BCK(launch_lam_eff(P));
     BCK(launch_damping(P));
     BCK(launch_image_dft(P, M, P.cur_images, P.cur_shifts, P.cur_gid));
-    BCK(launch_bin(P, M, false));
+    BCK(launch_bin(P, M, false, true));
     BCK(launch_spread_clear(P, false));
     if (spread_here) BCK(launch_spread_only(P, M, false));
     return cudaSuccess;
@@ -245,17 +252,18 @@ cudaError_t enqueue_body(firm_batch_s& b, const firm_batch_item* items, int iter
     }
     if (persistent) {
         BCK(join(b));
-        BCK(launch_spread_batch(b.n, true, b.W, b.poly, b.desc_k, b.item_off, b.queue, b.num_sms, b.main));
-        own += 2;
+        const int mk = count_mma(b, items, true), mr = count_mma(b, items, false);
+        BCK(launch_spread_batch(b.n, mk, true, b.W, b.poly, b.desc_k, b.item_off, b.queue, b.num_sms, b.main));
+        own += 2 * ((mk > 0) + (mk < b.n));
         BCK(fork(b));
         for (int k = 0; k < b.n; ++k) {
             const int i = b.order[k];
             BCK(plan_middle(b.plans[i]->P, items[i], false));
         }
         BCK(join(b));
-        BCK(launch_spread_batch(b.n, false, b.W, b.poly, b.desc_r, b.item_off + b.n + 1, b.queue + 1, b.num_sms,
-                                b.main));
-        own += 2;
+        BCK(launch_spread_batch(b.n, mr, false, b.W, b.poly, b.desc_r, b.item_off + 2 * (b.n + 1), b.queue + 2,
+                                b.num_sms, b.main));
+        own += 2 * ((mr > 0) + (mr < b.n));
         BCK(fork(b));
     }
     if (!solve) {
@@ -299,8 +307,8 @@ cudaError_t write_desc(firm_batch_s& b, const firm_batch_item* items) {
     for (int i = 0; i < b.n; ++i) {
         Plan& P = b.plans[i]->P;
         P.cur_gid = items[i].group ? items[i].group : P.ws.gid;
-        spread_batch_fill_desc(P, true, hk.data() + st * i);
-        spread_batch_fill_desc(P, false, hr.data() + st * i);
+        spread_batch_fill_desc(P, items[i].M, true, hk.data() + st * i);
+        spread_batch_fill_desc(P, items[i].M, false, hr.data() + st * i);
     }
     BCK(cudaMemcpyAsync(b.desc_k, hk.data(), hk.size(), cudaMemcpyHostToDevice, b.main));
     BCK(cudaMemcpyAsync(b.desc_r, hr.data(), hr.size(), cudaMemcpyHostToDevice, b.main));

@@ -18,6 +18,11 @@ constexpr int kKbDeg = 7;             // degree of the per-tap window polynomial
 constexpr int kMaxW = 8;              // widest Kaiser-Bessel window supported
 constexpr int kChunk = 8192;          // most points one spreading work item takes
 constexpr int kMinChunk = 1024;       // smallest work-item size a plan may be tuned to
+// Tensor-core spreading (spread_mma.cu): most points of one work item (a block sorts
+// them in shared memory), and the padding its classes can need: 15 points for each of
+// 27 classes, an item's records starting at a multiple of 16 slots.
+constexpr int kMmaChunk = 4096;
+constexpr int kMmaPad = 27 * 15 + 15;
 constexpr int kMaxBatch = 1024;       // most plans one batch holds
 constexpr int kTBits = 13;            // point id = m << kTBits | t (t < 8192)
 constexpr int kMaxHist = 20001;       // residual history capacity (iterations + 1)
@@ -31,11 +36,12 @@ struct KbPoly {
 };
 
 // Per-image slice geometry: rows 0 and 1 of R_m (the in-plane axes u, v of the slice,
-// xi = w1 u + w2 v) split into float hi + lo parts so that positions on the fine
-// grid are formed to ~1e-7 cells.
-struct ImgGeom {
-    float uh[3], ul[3], vh[3], vl[3];
+// xi = w1 u + w2 v) in fixed point, round(u 2^41) as high part * 2^16 + low part, so that
+// k1 u + k2 v is formed exactly in 32-bit integer arithmetic (spread.cuh).
+struct __align__(16) ImgGeom {
+    int32_t uh[3], vh[3], ul[3], vl[3];
 };
+constexpr int kGeomBits = 41;
 
 // CG state on the device (FP64 scalars; Section 3.3).
 struct CgState {
@@ -89,9 +95,15 @@ struct Workspace {
     uint16_t* perm = nullptr;       // per payload position: index in scatter order within its piece
     int4* work = nullptr;           // (brick, start, count, -)
     float* wmax_item = nullptr;     // fused form: per work item, the largest |h b| of its points
+    uint4* pts = nullptr;           // tensor-core form: placed points, x, y, z coordinate words and a weight
+    float2* pts_w = nullptr;        //   (h^2; A*b: its real part), and the other weights
+    uint32_t* rec = nullptr;        //   sorted, padded point records
+    uint8_t* rec_cls = nullptr;     //   the class of every 16 slots
+    int4* rec_item = nullptr;       //   per work item: (brick, first slot, groups, scales)
     unsigned long long* scan_part = nullptr;   // brick scan: per-block (points, items) totals
     double* item_part = nullptr;    // per work item: two FP64 partial sums (data residual)
-    int* counters = nullptr;        // [0] work items, [1] work cursor, [2] error flag
+    int* counters = nullptr;        // [0] work items, [1] work cursor, [2] error flag, [3] sort cursor,
+                                    // [4] record slots taken (in 16s)
     double* grid = nullptr;         // fine grid, FP64 (real for Ker, complex for A*b)
     float2* fx1 = nullptr;          // FFT intermediates
     float2* fx2 = nullptr;
@@ -152,6 +164,7 @@ struct Plan {
     long long launches = 0;         // kernels launched by this plan
     int pc_mode = 0;                // FIRM_PRECOND_*
     bool pc_ready = false;          // pc_diag built for the current K-hat and mode
+    bool bin_mma = false;           // the binned points are ordered for the tensor-core form
     int last_M = 0;                 // images of the last firm_kernel
     int bin_M = -1;                 // images of the last firm_bin (its ids and items still held); -1 none
     bool bin_kc = true;             // channel of the last firm_bin (true: kernel, 4N grid)
@@ -184,7 +197,23 @@ double ctf_value(const firm_ctf_group& g, double r_invA);
 
 // ---- launchers (spread.cu) ----
 cudaError_t launch_geom(const double* R, int M, ImgGeom* geom, cudaStream_t s);
-cudaError_t launch_bin(Plan& P, int M, bool kernel_channel);
+// Binning in two steps: the count of points per brick and the work items (poses only),
+// then the points in the items' order.  ch: 1 kernel channel, 2 A*b, 3 both on the 4N
+// grid.  spread: the points will be spread, in the tensor-core form where spread_uses_mma
+// says so; otherwise (interpolation, inspection) they are ordered round-robin over bank
+// classes.  The tensor-core form places the A*b weights with the points: the image DFT
+// comes before launch_bin_place then.
+cudaError_t launch_bin_count(Plan& P, int M, int ch, bool spread);
+cudaError_t launch_bin_place(Plan& P, int M, int ch);
+inline cudaError_t launch_bin(Plan& P, int M, bool kernel_channel, bool spread) {
+    const cudaError_t e = launch_bin_count(P, M, kernel_channel ? 1 : 2, spread);
+    return e != cudaSuccess ? e : launch_bin_place(P, M, kernel_channel ? 1 : 2);
+}
+// Whether M images of a plan are spread in the tensor-core form (points: all of them, on a
+// grid of nb bricks per axis), and the record slots that can take.
+bool mma_rule(const firm_params& p, size_t points, int nb, int ch);
+size_t mma_slots(size_t points, int nb);
+bool spread_uses_mma(const Plan& P, int M, int ch);
 cudaError_t launch_spread(Plan& P, int M, bool kernel_channel);        // clear + spread
 cudaError_t launch_spread_clear(Plan& P, bool kernel_channel);          // zero the fine grid
 cudaError_t launch_spread_only(Plan& P, int M, bool kernel_channel);    // spread (grid cleared)
@@ -199,8 +228,10 @@ cudaError_t launch_fused_gather(Plan& P, int M);
 // fine grids; each plan's grid cleared and its points binned beforehand.  args: device
 // array of n per-plan descriptors; item_off: device (n + 1) ints; queue: device int.
 size_t spread_batch_desc_bytes();
-void spread_batch_fill_desc(Plan& P, bool kernel_channel, void* host_desc);
-cudaError_t launch_spread_batch(int n, bool kernel_channel, int W, const KbPoly& poly, const void* dev_desc,
+void spread_batch_fill_desc(Plan& P, int M, bool kernel_channel, void* host_desc);
+// n_mma of the plans are binned for the tensor-core form: their items go in a launch of
+// their own.  item_off: 2 (n + 1) ints, queue: 2 ints.
+cudaError_t launch_spread_batch(int n, int n_mma, bool kernel_channel, int W, const KbPoly& poly, const void* dev_desc,
                                 int* item_off, int* queue, int num_sms, cudaStream_t s);
 
 // ---- launchers (fft_passes.cu) ----

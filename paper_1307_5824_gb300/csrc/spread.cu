@@ -21,7 +21,10 @@
 // transformed grid and gathers the W^3 taps of each point, with no atomics.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "firm_internal.h"
+#include "spread.cuh"
 
 namespace firm {
 
@@ -35,12 +38,15 @@ __global__ void k_geom(const double* __restrict__ R, int M, ImgGeom* __restrict_
     ImgGeom o;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        double u = r[d], v = r[3 + d];
-        float uh = (float)u, vh = (float)v;
-        o.uh[d] = uh;
-        o.ul[d] = (float)(u - (double)uh);
-        o.vh[d] = vh;
-        o.vl[d] = (float)(v - (double)vh);
+        // a column of R longer than 1.3 (never a rotation; NaN too) would leave the grid by
+        // more than the arithmetic holds: it is dropped, so that no point leaves the bricks
+        const bool ok = r[d] * r[d] + r[3 + d] * r[3 + d] <= 1.69;
+        const long long u = ok ? __double2ll_rn(r[d] * (double)(1ll << kGeomBits)) : 0;
+        const long long v = ok ? __double2ll_rn(r[3 + d] * (double)(1ll << kGeomBits)) : 0;
+        o.uh[d] = (int)(u >> 16);
+        o.ul[d] = (int)(u & 0xffff);
+        o.vh[d] = (int)(v >> 16);
+        o.vl[d] = (int)(v & 0xffff);
     }
     g[m] = o;
 }
@@ -49,122 +55,6 @@ cudaError_t launch_geom(const double* R, int M, ImgGeom* geom, cudaStream_t s) {
     if (M <= 0) return cudaSuccess;
     k_geom<<<(M + 255) / 256, 256, 0, s>>>(R, M, geom);
     return cudaGetLastError();
-}
-
-// Integer cell I in [0, G) and fraction f in [0, 1) of the coordinate
-// y = G/2 + sk1 * u + sk2 * v along one axis, with sk1 = (G/N) k1 and sk2 = (G/N) k2
-// exact small integers.  The products are split exactly (FMA error terms) and the
-// integer parts removed before the fractions are summed, so y is formed to ~1e-7.
-__device__ __forceinline__ void cell_coord(float sk1, float sk2, float uh, float ul, float vh, float vl,
-                                           int halfG, int G, int& I, float& f) {
-    // explicit rounding intrinsics: no contraction, so every kernel that calls this
-    // (binning and spreading) gets bit-identical cells.  Round-to-nearest integers by
-    // adding 1.5 * 2^23 (|a|, |b| <= G/2 < 2^22); the bit pattern then holds the integer.
-    constexpr float kMagic = 12582912.0f;
-    constexpr int kMagicBits = 0x4B400000;
-    const float a = __fmul_rn(sk1, uh), ea = fmaf(sk1, uh, -a);
-    const float b = __fmul_rn(sk2, vh), eb = fmaf(sk2, vh, -b);
-    const float ma = __fadd_rn(a, kMagic), mb = __fadd_rn(b, kMagic);
-    const float ra = __fsub_rn(ma, kMagic), rb = __fsub_rn(mb, kMagic);
-    const float lo = __fadd_rn(__fadd_rn(ea, eb), fmaf(sk1, ul, __fmul_rn(sk2, vl)));
-    const float fr = __fadd_rn(__fadd_rn(__fsub_rn(a, ra), __fsub_rn(b, rb)), lo);
-    const float fl = floorf(fr);
-    float ff = __fsub_rn(fr, fl);
-    int ii = (__float_as_int(ma) - kMagicBits) + (__float_as_int(mb) - kMagicBits) +
-             (__float_as_int(__fadd_rn(fl, kMagic)) - kMagicBits) + halfG;
-    if (ff >= 1.0f) { ff = 0.0f; ii += 1; }
-    // |k1 u + k2 v| <= |k| <= N/2 (u, v: parts of a unit column of R), so ii lies in
-    // [-1, G + 1]: one wrap either way is the periodic index
-    if (ii >= G) ii -= G;
-    else if (ii < 0) ii += G;
-    I = ii;
-    f = ff;
-}
-
-struct PointPos {
-    int I[3];
-    float f[3];
-};
-
-__device__ __forceinline__ PointPos point_pos(const ImgGeom& g, int32_t kk, float scale, int halfG, int G) {
-    const float k1 = (float)(int16_t)(kk & 0xffff), k2 = (float)(kk >> 16);
-    const float sk1 = scale * k1, sk2 = scale * k2;
-    PointPos p;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) cell_coord(sk1, sk2, g.uh[d], g.ul[d], g.vh[d], g.vl[d], halfG, G, p.I[d], p.f[d]);
-    return p;
-}
-
-// ---------------------------------------------------------------------------
-// Window taps and the region base of a point
-// ---------------------------------------------------------------------------
-template <int W>
-__device__ __forceinline__ int tap_shift(float f) {
-    // first tap offset u = c - (f - h) in [0, 1), h = 1/2 for odd W, 0 for even W
-    constexpr float h = (W & 1) ? 0.5f : 0.0f;
-    return (int)ceilf(f - h);
-}
-
-template <int W>
-__device__ __forceinline__ void window_taps(const KbPoly& P, float f, float* w) {
-    constexpr float h = (W & 1) ? 0.5f : 0.0f;
-    const float t0 = f - h;
-    const float z = 2.0f * (ceilf(t0) - t0) - 1.0f;
-#pragma unroll
-    for (int l = 0; l < W; ++l) {
-        float acc = P.c[l][kKbDeg];
-#pragma unroll
-        for (int j = kKbDeg - 1; j >= 0; --j) acc = fmaf(acc, z, P.c[l][j]);
-        w[l] = acc;
-    }
-}
-
-// Dither of the kernel channel's fixed-point rounding: a value in [-1/2, 1/2) fixed by
-// the point id (a 32-bit integer hash), added to every tap of the point before it is
-// rounded to an integer.  Rounding to nearest drops every tap below half a unit, and
-// the far taps of the window are that small: without the dither the kernel's sums come
-// out biased low (~1e-6 relative, a smooth error that moves a 10-iteration CG volume by
-// 1e-4 on the N=64 workload).  With it the rounding is unbiased, E[round(v + d)] = v
-// for d uniform, and its error is white (a 1e-6 white error in Ker moves that volume by
-// ~4e-7).
-__device__ __forceinline__ float point_dither(uint32_t id) {
-    uint32_t h = id * 2654435761u;
-    h ^= h >> 15;
-    h *= 2246822519u;
-    h ^= h >> 13;
-    return (float)(h >> 8) * (1.0f / 16777216.0f) - 0.5f;
-}
-
-// Rank (mod W) of this lane's point among the lanes of its warp with the same bank
-// class (base mod 32; base < 0: no point).  Called by all 32 lanes.  Most warp steps of
-// a round-robin piece hold 32 distinct classes: one OR-reduction of the class bits
-// finds those, and only the others pay for the match.
-template <int W>
-__device__ __forceinline__ int class_rank(int base, int lane) {
-    const bool pt = base >= 0;
-    const unsigned bits = __reduce_or_sync(0xffffffffu, pt ? 1u << (base & 31) : 0u);
-    const unsigned pts = __ballot_sync(0xffffffffu, pt);
-    if (__popc(bits) == __popc(pts)) return 0;
-    const unsigned same = __match_any_sync(0xffffffffu, pt ? (base & 31) : -1 - lane);
-    const int r = __popc(same & ((1u << lane) - 1u));
-    return r < W ? r : r % W;
-}
-
-// Bricks: 8 x 8 x BZ cells (BZ = kBrickZk for the kernel channel, 8 for A*b).
-template <bool KC> struct Brick { static constexpr int BZ = KC ? kBrickZk : kBrick; };
-
-// Index of the first tap of a point inside its brick's (8 + W) x (8 + W) x (BZ + W)
-// region (x fastest), or -1 if the point is not inside the brick (never expected:
-// binning uses the same code).
-template <int W, int BZ>
-__device__ __forceinline__ int region_base(const PointPos& p, int lo0, int lo1, int lo2) {
-    constexpr int RG = kBrick + W;
-    const int r0 = p.I[0] - lo0 + tap_shift<W>(p.f[0]);
-    const int r1 = p.I[1] - lo1 + tap_shift<W>(p.f[1]);
-    const int r2 = p.I[2] - lo2 + tap_shift<W>(p.f[2]);
-    if ((unsigned)r0 > (unsigned)kBrick || (unsigned)r1 > (unsigned)kBrick || (unsigned)r2 > (unsigned)BZ)
-        return -1;
-    return (r2 * RG + r1) * RG + r0;
 }
 
 // ---------------------------------------------------------------------------
@@ -183,9 +73,14 @@ struct BinArgs {
     uint8_t* cls;          // scatter pass output: bank class of each point
     const float2* samples; // A*b channel: weights [m][t], copied to samples_b[slot] by the scatter
     float2* samples_b;     //   (consecutive lanes read consecutive t: coalesced)
+    uint4* pts;            // tensor-core form: placed points
+    float2* pts_w;
+    const float* h2;
+    const int32_t* gid;
+    int n_ctf;
     long long npts;        // M * nH
     int nH, G, halfG, nb;  // nb = bricks per axis
-    float scale;
+    int ls;                // log2(G / N)
 };
 
 template <int W, bool SCATTER, bool KC>
@@ -199,7 +94,7 @@ __global__ void __launch_bounds__(256) k_bin(BinArgs a, int M) {
         const bool valid = t < a.nH;
         int key = -1, c = 0;
         if (valid) {
-            const PointPos p = point_pos(a.geom[m], __ldg(&a.htab[t]), a.scale, a.halfG, a.G);
+            const PointPos p = point_pos(a.geom[m], __ldg(&a.htab[t]), a.ls, a.halfG, a.G);
             const int bx = p.I[0] / kBrick, by = p.I[1] / kBrick, bz = p.I[2] / BZ;
             key = (bz * a.nb + by) * a.nb + bx;
             if (SCATTER) c = region_base<W, BZ>(p, bx * kBrick, by * kBrick, bz * BZ) & 31;
@@ -233,7 +128,10 @@ __global__ void __launch_bounds__(256) k_bin(BinArgs a, int M) {
 // 2D piece of the slice and fall in few bricks; lanes with equal bricks are grouped
 // with __match_any_sync, one cursor atomic per group (about half as many as runs along
 // one column give).  col[k1] = (first index t of column k1, its lowest k2, its highest k2).
-template <int W, bool KC>
+// CH > 0 (1 kernel channel, 2 A*b, 3 both): the tensor-core form, whose points are placed
+// as coordinates and weights instead of ids: an image's geometry is the same for the
+// whole warp here, where the sort that follows would have to look it up per point.
+template <int W, bool KC, int CH>
 __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN, const int4* __restrict__ col,
                                                        int tiles_x, int n_tiles) {
     constexpr int BZ = Brick<KC>::BZ;
@@ -251,11 +149,24 @@ __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN,
     const int32_t kk = (int32_t)((uint32_t)(k1 & 0xffff) | ((uint32_t)k2 << 16));
     for (int m = blockIdx.y; m < M; m += gridDim.y) {
         int key = -1, c = 0;
+        uint4 pt = make_uint4(0u, 0u, 0u, 0u);
+        float2 wv = make_float2(0.0f, 0.0f);
         if (valid) {
-            const PointPos p = point_pos(a.geom[m], kk, a.scale, a.halfG, a.G);
+            const PointPos p = point_pos(a.geom[m], kk, a.ls, a.halfG, a.G);
             const int bx = p.I[0] / kBrick, by = p.I[1] / kBrick, bz = p.I[2] / BZ;
             key = (bz * a.nb + by) * a.nb + bx;
-            c = region_base<W, BZ>(p, bx * kBrick, by * kBrick, bz * BZ) & 31;
+            if (CH > 0) {
+                pt.x = coord_word<W>(p.I[0] - bx * kBrick, p.q[0]);
+                pt.y = coord_word<W>(p.I[1] - by * kBrick, p.q[1]);
+                pt.z = coord_word<W>(p.I[2] - bz * BZ, p.q[2]);
+                if (CH != 2) {
+                    const int g = min(max(__ldg(&a.gid[m]), 0), a.n_ctf - 1);
+                    pt.w = __float_as_uint(__ldg(&a.h2[(size_t)g * a.nH + t]));
+                }
+                if (CH >= 2) wv = __ldg(&a.samples[(size_t)m * a.nH + t]);
+            } else {
+                c = region_base<W, BZ>(p, bx * kBrick, by * kBrick, bz * BZ) & 31;
+            }
         }
         const unsigned grp = __match_any_sync(0xffffffffu, key);
         const int leader = __ffs(grp) - 1;
@@ -264,9 +175,16 @@ __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN,
         base = __shfl_sync(0xffffffffu, base, leader);
         if (valid) {
             const uint32_t slot = base + (uint32_t)__popc(grp & ((1u << lane) - 1u));
-            a.payload[slot] = ((uint32_t)m << kTBits) | (uint32_t)t;
-            a.cls[slot] = (uint8_t)c;
-            if (a.samples) a.samples_b[slot] = __ldg(&a.samples[(size_t)m * a.nH + t]);
+            if (CH > 0) {
+                if (CH == 2) pt.w = __float_as_uint(wv.x);
+                a.pts[slot] = pt;
+                if (CH == 2) reinterpret_cast<float*>(a.pts_w)[slot] = wv.y;
+                if (CH == 3) a.pts_w[slot] = wv;
+            } else {
+                a.payload[slot] = ((uint32_t)m << kTBits) | (uint32_t)t;
+                a.cls[slot] = (uint8_t)c;
+                if (a.samples) a.samples_b[slot] = __ldg(&a.samples[(size_t)m * a.nH + t]);
+            }
         }
     }
 }
@@ -351,6 +269,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* __
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) {
         counters[0] = (int)min(woff, (long long)max_work);
         counters[1] = 0;
+        counters[3] = 0;
+        counters[4] = 0;
     }
 }
 
@@ -375,15 +295,15 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_parts(ScanPart* __restric
     }
 }
 
-static void launch_scan(Plan& P, int nbricks) {
+static void launch_scan(Plan& P, int nbricks, int chunk) {
     Workspace& w = P.ws;
     const int nblk = (nbricks + kScanSpan - 1) / kScanSpan;
     ScanPart* part = reinterpret_cast<ScanPart*>(w.scan_part);
     k_scan_bricks<false><<<nblk, kScanThreads, 0, P.stream>>>(w.count, w.cursor, nbricks, part, w.work,
-                                                               w.counters, (int)P.max_work, P.chunk);
+                                                               w.counters, (int)P.max_work, chunk);
     k_scan_parts<<<1, kScanThreads, 0, P.stream>>>(part, nblk);
     k_scan_bricks<true><<<nblk, kScanThreads, 0, P.stream>>>(w.count, w.cursor, nbricks, part, w.work,
-                                                              w.counters, (int)P.max_work, P.chunk);
+                                                              w.counters, (int)P.max_work, chunk);
     P.launches += 3;
 }
 
@@ -502,60 +422,122 @@ __global__ void __launch_bounds__(256) k_class_sort(uint32_t* __restrict__ paylo
     }
 }
 
-template <int W>
-static void bin_w(Plan& P, const BinArgs& a0, int nbricks, bool kc) {
+// The class sort of a plan's binned points (not the tensor-core form, which sorts its own).
+static void launch_class_sort(Plan& P, bool kc) {
     Workspace& w = P.ws;
-    BinArgs a = a0;
-    const int M = (int)(a.npts / a.nH);
-    const dim3 grid((a.nH + 255) / 256, (unsigned)(M < 65535 ? M : 65535));
-    if (kc) k_bin<W, false, true><<<grid, 256, 0, P.stream>>>(a, M);
-    else k_bin<W, false, false><<<grid, 256, 0, P.stream>>>(a, M);
-    launch_scan(P, nbricks);
-    a.count = w.cursor;
-    const int hN = P.N / 2, tiles_x = (hN + 1 + 3) / 4, n_tiles = tiles_x * ((P.N + 1 + 7) / 8);
-    const dim3 grid2((n_tiles + 7) / 8, (unsigned)(M < 65535 ? M : 65535));
-    if (kc) k_bin_scatter2d<W, true><<<grid2, 256, 0, P.stream>>>(a, M, hN, w.colinfo, tiles_x, n_tiles);
-    else k_bin_scatter2d<W, false><<<grid2, 256, 0, P.stream>>>(a, M, hN, w.colinfo, tiles_x, n_tiles);
     cudaFuncSetAttribute(k_class_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem);
     const bool keep = kc && w.payload_scat;       // fused plans keep the scatter order
     k_class_sort<<<P.num_sms * 4, 256, kSortSmem, P.stream>>>(w.payload, w.cls, w.work, w.counters,
                                                                kc ? nullptr : w.perm, keep ? w.payload_scat : nullptr,
                                                                keep ? w.inv_perm : nullptr);
+    P.launches += 1;
 }
 
-cudaError_t launch_bin(Plan& P, int M, bool kc) {
+template <int W>
+static void bin_count_w(Plan& P, const BinArgs& a, int M, bool kc) {
+    const dim3 grid((a.nH + 255) / 256, (unsigned)(M < 65535 ? M : 65535));
+    if (kc) k_bin<W, false, true><<<grid, 256, 0, P.stream>>>(a, M);
+    else k_bin<W, false, false><<<grid, 256, 0, P.stream>>>(a, M);
+    P.launches += 1;
+}
+
+template <int W>
+static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
+    const int hN = P.N / 2, tiles_x = (hN + 1 + 3) / 4, n_tiles = tiles_x * ((P.N + 1 + 7) / 8);
+    const dim3 g((n_tiles + 7) / 8, (unsigned)(M < 65535 ? M : 65535));
+    const int4* col = P.ws.colinfo;
+    const bool sm = a.samples != nullptr;
+    if (P.bin_mma) {
+        if (kc && sm) k_bin_scatter2d<W, true, 3><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
+        else if (kc) k_bin_scatter2d<W, true, 1><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
+        else k_bin_scatter2d<W, false, 2><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
+    } else {
+        if (kc) k_bin_scatter2d<W, true, 0><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
+        else k_bin_scatter2d<W, false, 0><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
+    }
+    P.launches += 1;
+}
+
+// Average points per brick of the ball from which the tensor-core form is the faster one
+// (binning and spreading together).  Its cost per brick is high -- 27 classes padded to 16
+// points, each flushed to the region -- and its cost per point low, the lower the more
+// channels share the window arithmetic.  Measured at N = 64, W = 6, in ms, bank-class form
+// against tensor-core form: kernel channel 0.65 / 0.76 at 282 points a brick, 0.88 / 0.91
+// at 470, 1.30 / 1.20 at 846; A*b 0.158 / 0.154 at 226, 0.47 / 0.23 at 754; both in one
+// pass 0.83 / 1.00 at 94, 1.05 / 1.08 at 188, 1.32 / 1.16 at 282.
+bool mma_rule(const firm_params& p, size_t points, int nb, int ch) {
+    const double least = ch == 1 ? 500.0 : ch == 2 ? 220.0 : 200.0;
+    return p.W == 6 && (double)points >= least * 0.5236 * nb * nb * (double)nb;
+}
+
+size_t mma_slots(size_t points, int nb) {
+    const size_t items = std::min((size_t)nb * nb * nb, points) + points / kMmaChunk;
+    return points + items * kMmaPad;
+}
+
+bool spread_uses_mma(const Plan& P, int M, int ch) {
+    return mma_rule(P.p, (size_t)M * P.nH, ch == 2 ? P.nbr : P.nbk, ch);
+}
+
+static BinArgs bin_args(Plan& P, int M, bool kc) {
     Workspace& w = P.ws;
-    const int G = kc ? P.Gk : P.Gr;
-    const int nb = kc ? P.nbk : P.nbr;
-    const int nbricks = nb * nb * (kc ? P.nbkz : P.nbr);
-    cudaError_t e = cudaMemsetAsync(w.count, 0, sizeof(uint32_t) * nbricks, P.stream);
-    if (e != cudaSuccess) return e;
     BinArgs a;
     a.geom = w.geom;
     a.htab = w.htab;
     a.count = w.count;
-    a.payload = kc && w.payload_scat ? w.payload_scat : w.payload;
+    a.payload = kc && w.payload_scat && !P.bin_mma ? w.payload_scat : w.payload;
     a.cls = w.cls;
     a.samples = kc ? nullptr : w.samples;
     a.samples_b = w.samples_b;
+    a.pts = w.pts;
+    a.pts_w = w.pts_w;
+    a.h2 = w.h2;
+    a.gid = P.cur_gid;
+    a.n_ctf = P.n_ctf;
     a.npts = (long long)M * P.nH;
     a.nH = P.nH;
-    a.G = G;
-    a.halfG = G / 2;
-    a.nb = nb;
-    a.scale = (float)(G / P.N);
-    const long long blocks = (a.npts + 255) / 256;
-    if (blocks == 0) {
-        launch_scan(P, nbricks);
-        return cudaGetLastError();
+    a.G = kc ? P.Gk : P.Gr;
+    a.halfG = a.G / 2;
+    a.nb = kc ? P.nbk : P.nbr;
+    a.ls = kc ? 2 : 1;
+    return a;
+}
+
+cudaError_t launch_bin_count(Plan& P, int M, int ch, bool spread) {
+    const bool kc = ch != 2;
+    const int nb = kc ? P.nbk : P.nbr;
+    const int nbricks = nb * nb * (kc ? P.nbkz : P.nbr);
+    P.bin_mma = spread && spread_uses_mma(P, M, ch);
+    cudaError_t e = cudaMemsetAsync(P.ws.count, 0, sizeof(uint32_t) * nbricks, P.stream);
+    if (e != cudaSuccess) return e;
+    if (M > 0) {
+        const BinArgs a = bin_args(P, M, kc);
+        switch (P.p.W) {
+            case 6: bin_count_w<6>(P, a, M, kc); break;
+            case 7: bin_count_w<7>(P, a, M, kc); break;
+            case 8: bin_count_w<8>(P, a, M, kc); break;
+            default: return cudaErrorInvalidValue;
+        }
     }
+    launch_scan(P, nbricks, P.bin_mma ? kMmaChunk : P.chunk);
+    return cudaGetLastError();
+}
+
+static SpreadArgs spread_args(Plan& P, bool kc);
+cudaError_t launch_bin_place(Plan& P, int M, int ch) {
+    const bool kc = ch != 2;
+    if (M <= 0) return cudaSuccess;
+    BinArgs a = bin_args(P, M, kc);
+    a.count = P.ws.cursor;
+    if (ch == 3 && P.bin_mma) a.samples = P.ws.samples;      // the A*b weights go with the points
     switch (P.p.W) {
-        case 6: bin_w<6>(P, a, nbricks, kc); break;
-        case 7: bin_w<7>(P, a, nbricks, kc); break;
-        case 8: bin_w<8>(P, a, nbricks, kc); break;
+        case 6: bin_place_w<6>(P, a, M, kc); break;
+        case 7: bin_place_w<7>(P, a, M, kc); break;
+        case 8: bin_place_w<8>(P, a, M, kc); break;
         default: return cudaErrorInvalidValue;
     }
-    P.launches += 3;
+    if (P.bin_mma) return launch_mma_sort(P, spread_args(P, kc), ch);
+    launch_class_sort(P, kc);
     return cudaGetLastError();
 }
 
@@ -570,25 +552,6 @@ cudaError_t launch_bin(Plan& P, int M, bool kc) {
 // so a cell can never exceed 2^30.  Level 2 is added into the FP64 grid when the work
 // item ends.
 // ---------------------------------------------------------------------------
-struct SpreadArgs {
-    const uint32_t* payload;
-    const int4* work;
-    int* counters;
-    const ImgGeom* geom;
-    const int32_t* htab;
-    const int32_t* gid;
-    const float* h2;          // kernel channel weights [group][t]
-    const float2* samples_b;  // right-hand-side weights in scatter order
-    const float2* samples;    // fused form: the weights h b at [m][t]
-    const uint16_t* perm;     // per payload position: the point's index in scatter order
-    double* grid;             // G^3 real, or G^3 complex interleaved (re, im)
-    int G, halfG, nb, nH, n_ctf;
-    float scale;
-    float wmax_fixed;         // > 0: bound on |w| known in advance (no pre-pass)
-    const float* wmax_item;   // fused form: per work item, the largest |h b| of its points
-    KbPoly poly;
-};
-
 constexpr int kSpreadThreads = 256;
 constexpr int kSpreadWarps = kSpreadThreads / 32;
 
@@ -670,7 +633,7 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
             int base = -1;
             if (live) {
                 id = __ldg(&a.payload[s0 + kSpreadThreads * i]);
-                p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.scale, a.halfG,
+                p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.ls, a.halfG,
                               a.G);
                 base = region_base<W, BZ>(p, lo0, lo1, lo2);
                 if (base < 0) atomicOr(&a.counters[2], 1);   // point outside its brick: reported, never written
@@ -685,9 +648,9 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
             const int t = (int)(id & ((1u << kTBits) - 1u));
             const float2 wv = point_weight(a, CPLX, m, t, (uint32_t)wk.y, s0 + kSpreadThreads * i);
             float wx[W], wy[W], wz[W];
-            window_taps<W>(poly, p.f[0], wx);
-            window_taps<W>(poly, p.f[1], wy);
-            window_taps<W>(poly, p.f[2], wz);
+            window_taps<W>(poly, p.f(0), wx);
+            window_taps<W>(poly, p.f(1), wy);
+            window_taps<W>(poly, p.f(2), wz);
             const float dth = CPLX ? 0.0f : point_dither(id);
 #pragma unroll
             for (int r = 1; r < W; ++r)
@@ -825,13 +788,15 @@ __global__ void __launch_bounds__(kSpreadThreads, CPLX ? 5 : 6) k_spread_batch(c
     }
 }
 
-// item_off = exclusive prefix of the plans' work-item counts; queue = 0.  One warp.
-__global__ void k_batch_items(const SpreadArgs* __restrict__ desc, int n, int* __restrict__ item_off, int* queue) {
+// item_off = exclusive prefix of the work-item counts of the plans of one form (mma 0 or
+// 1; the others count 0); queue = 0.  One warp.
+__global__ void k_batch_items(const SpreadArgs* __restrict__ desc, int n, int mma, int* __restrict__ item_off,
+                              int* queue) {
     const int lane = threadIdx.x;
     int carry = 0;
     for (int p0 = 0; p0 < n; p0 += 32) {
         const int p = p0 + lane;
-        const int c = p < n ? desc[p].counters[0] : 0;
+        const int c = p < n && desc[p].mma == mma ? desc[p].counters[0] : 0;
         int v = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -907,7 +872,7 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
             int base = -1;
             if (live) {
                 id = __ldg(&a.payload[s0 + T * i]);
-                p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.scale, a.halfG,
+                p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.ls, a.halfG,
                               a.G);
                 base = region_base<W, BZ>(p, lo0, lo1, lo2);
                 if (base < 0) atomicOr(&a.counters[2], 1);   // point outside its brick: reported, never written
@@ -924,9 +889,9 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
             const float2 w2 = make_float2(wv.x * Sb, wv.y * Sb);
             const float dth = point_dither(id);
             float wx[W], wy[W], wz[W];
-            window_taps<W>(poly, p.f[0], wx);
-            window_taps<W>(poly, p.f[1], wy);
-            window_taps<W>(poly, p.f[2], wz);
+            window_taps<W>(poly, p.f(0), wx);
+            window_taps<W>(poly, p.f(1), wy);
+            window_taps<W>(poly, p.f(2), wz);
 #pragma unroll
             for (int rr = 1; rr < W; ++rr)
                 if (rr <= sh) {
@@ -1101,7 +1066,7 @@ static cudaError_t spread_batch_w(int n, const SpreadArgs* desc, int* item_off, 
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_batch<W, CPLX>, kSpreadThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_batch_items<<<1, 32, 0, s>>>(desc, n, item_off, queue);
+    k_batch_items<<<1, 32, 0, s>>>(desc, n, 0, item_off, queue);
     k_spread_batch<W, CPLX><<<num_sms * per_sm, kSpreadThreads, smem, s>>>(desc, n, item_off, queue, poly);
     return cudaGetLastError();
 }
@@ -1111,6 +1076,12 @@ static SpreadArgs spread_args(Plan& P, bool kc) {
     const int G = kc ? P.Gk : P.Gr;
     SpreadArgs a;
     a.payload = w.payload;
+    a.pts = w.pts;
+    a.pts_w = w.pts_w;
+    a.rec = w.rec;
+    a.rec_cls = w.rec_cls;
+    a.rec_item = w.rec_item;
+    a.rec_slots = (uint32_t)std::min<size_t>(mma_slots((size_t)P.p.M * P.nH, kc ? P.nbk : P.nbr), 0xffffffffu);
     a.work = w.work;
     a.counters = w.counters;
     a.geom = w.geom;
@@ -1126,7 +1097,8 @@ static SpreadArgs spread_args(Plan& P, bool kc) {
     a.nb = kc ? P.nbk : P.nbr;
     a.nH = P.nH;
     a.n_ctf = P.n_ctf;
-    a.scale = (float)(G / P.N);
+    a.ls = kc ? 2 : 1;
+    a.mma = P.bin_mma ? 1 : 0;
     a.wmax_fixed = kc ? P.h2_max : 0.0f;
     a.wmax_item = nullptr;
     a.poly = P.poly;
@@ -1142,6 +1114,7 @@ cudaError_t launch_spread_clear(Plan& P, bool kc) {
 cudaError_t launch_spread_only(Plan& P, int M, bool kc) {
     if (M <= 0) return cudaSuccess;
     const SpreadArgs a = spread_args(P, kc);
+    if (P.bin_mma) return launch_spread_mma(P, a, kc ? 1 : 2);
     switch (P.p.W) {
         case 6: return kc ? spread_w<6, false>(P, a) : spread_w<6, true>(P, a);
         case 7: return kc ? spread_w<7, false>(P, a) : spread_w<7, true>(P, a);
@@ -1160,6 +1133,7 @@ cudaError_t launch_fused_gather(Plan& P, int M) {
     if (M <= 0) return cudaSuccess;
     Workspace& w = P.ws;
     if (!w.payload_scat) return cudaErrorInvalidValue;      // fused plans only
+    if (P.bin_mma) return cudaSuccess;                       // the spreading kernel gathers its weights itself
     k_fused_gather<<<P.num_sms * 8, 256, 0, P.stream>>>(w.payload_scat, w.inv_perm, w.work, w.counters, w.samples,
                                                        P.nH, w.samples_b, w.wmax_item);
     P.launches += 1;
@@ -1173,6 +1147,7 @@ cudaError_t launch_spread_fused(Plan& P, int M) {
     SpreadArgs a = spread_args(P, true);
     a.samples_b = P.ws.samples_b;
     a.wmax_item = P.ws.wmax_item;
+    if (P.bin_mma) return launch_spread_mma(P, a, 3);
     switch (P.p.W) {
         case 6: return spread_fused_w<6>(P, a);
         case 7: return spread_fused_w<7>(P, a);
@@ -1183,13 +1158,20 @@ cudaError_t launch_spread_fused(Plan& P, int M) {
 
 size_t spread_batch_desc_bytes() { return sizeof(SpreadArgs); }
 
-void spread_batch_fill_desc(Plan& P, bool kc, void* host_desc) {
-    *reinterpret_cast<SpreadArgs*>(host_desc) = spread_args(P, kc);
+void spread_batch_fill_desc(Plan& P, int M, bool kc, void* host_desc) {
+    SpreadArgs a = spread_args(P, kc);
+    a.mma = spread_uses_mma(P, M, kc ? 1 : 2) ? 1 : 0;
+    *reinterpret_cast<SpreadArgs*>(host_desc) = a;
 }
 
-cudaError_t launch_spread_batch(int n, bool kc, int W, const KbPoly& poly, const void* dev_desc, int* item_off,
-                                int* queue, int num_sms, cudaStream_t s) {
+cudaError_t launch_spread_batch(int n, int n_mma, bool kc, int W, const KbPoly& poly, const void* dev_desc,
+                                int* item_off, int* queue, int num_sms, cudaStream_t s) {
     const SpreadArgs* d = reinterpret_cast<const SpreadArgs*>(dev_desc);
+    if (n_mma > 0) {
+        k_batch_items<<<1, 32, 0, s>>>(d, n, 1, item_off + n + 1, queue + 1);
+        const cudaError_t e = launch_spread_mma_batch(n, kc, d, item_off + n + 1, queue + 1, poly, num_sms, s);
+        if (e != cudaSuccess || n_mma == n) return e;
+    }
     switch (W) {
         case 6: return kc ? spread_batch_w<6, false>(n, d, item_off, queue, poly, num_sms, s)
                           : spread_batch_w<6, true>(n, d, item_off, queue, poly, num_sms, s);
@@ -1227,7 +1209,7 @@ struct InterpArgs {
     float2* out;              // forward mode: [m][t]
     double* item_part;        // residual mode: per work item (sum c|r|^2, sum c|b|^2)
     int G, halfG, nb, nH, n_ctf;
-    float scale;
+    int ls;                // log2(G / N)
     KbPoly poly;
 };
 
@@ -1274,16 +1256,16 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
             const uint32_t id = __ldg(&a.payload[pos]);
             const int m = (int)(id >> kTBits);
             const int t = (int)(id & ((1u << kTBits) - 1u));
-            const PointPos p = point_pos(a.geom[m], __ldg(&a.htab[t]), a.scale, a.halfG, a.G);
+            const PointPos p = point_pos(a.geom[m], __ldg(&a.htab[t]), a.ls, a.halfG, a.G);
             const int base = region_base<W, BZ>(p, lo0, lo1, lo2);
             if (base < 0) {
                 atomicOr(&a.counters[2], 1);   // point outside its brick: reported, never read
                 continue;
             }
             float wx[W], wy[W], wz[W];
-            window_taps<W>(a.poly, p.f[0], wx);
-            window_taps<W>(a.poly, p.f[1], wy);
-            window_taps<W>(a.poly, p.f[2], wz);
+            window_taps<W>(a.poly, p.f(0), wx);
+            window_taps<W>(a.poly, p.f(1), wy);
+            window_taps<W>(a.poly, p.f(2), wz);
             float fr = 0.0f, fi = 0.0f;
 #pragma unroll
             for (int dz = 0; dz < W; ++dz) {
@@ -1396,7 +1378,7 @@ cudaError_t launch_interp(Plan& P, int M, const float2* ghat, float2* out, doubl
     a.nb = P.nbr;
     a.nH = P.nH;
     a.n_ctf = P.n_ctf;
-    a.scale = (float)(P.Gr / P.N);
+    a.ls = 1;
     a.poly = P.poly;
     const bool resid = item_part != nullptr;
     cudaError_t e;

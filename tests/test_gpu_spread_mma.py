@@ -1,0 +1,54 @@
+"""The tensor-core spreading (dense bricks, W = 6) against the FP64 gridding oracle with the
+same Kaiser-Bessel window (eq. kernel, eq. backprojection), which leaves the arithmetic's
+own error: the sizes run from just above the rule's threshold, where most classes of a
+brick hold less than one group of points, to bricks of several work items.
+
+Tolerance 3e-6: taps and weights carry 22 bits and the window polynomials 2e-7; a cell's
+sum over at most 4096 points is rounded to 2^-18 of the largest weight about ten times,
+which is 1e-6 of a cell's sum of weights of rms a third of the largest."""
+import numpy as np
+import pytest
+
+import oracle as O
+from oracle import gridding as GR
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("N,M,cfg,fused", [(16, 118, "C2", False), (16, 1361, "C5", False), (16, 6001, "C3", False),
+                                           (32, 2900, "C5", False), (16, 541, "C3", True), (16, 2003, "C5", True),
+                                           (32, 801, "C2", True)])
+def test_tensor_core_spreading_matches_oracle(N, M, cfg, fused):
+    import __graft_entry__ as g
+    g.build()
+    import paper_1307_5824_gb300 as F
+    inp = synth.config_inputs(cfg, M=M, N=N)
+    K = O.disc(N)
+    kw = dict(W=6, window="kb", beta=GR.kb_beta(6))
+    Ker = GR.kernel_gridded(inp["R"], inp["groups"], inp["group_id"], K, N, **kw).real
+    rhs_o = GR.backproject_gridded(inp["images"], inp["shifts"], inp["R"], inp["groups"], inp["group_id"], K,
+                                   sigma=4 if fused else 2, **kw)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    rec = F.Reconstructor(N, M, groups=inp["groups"], W=6, lam=1e-3, fused=fused)
+    R, gid = dev(inp["R"].reshape(M, 9)), dev(inp["group_id"])
+    ker = torch.empty(rec.half_shape(), device="cuda")
+    rhs = torch.empty((N, N, N), device="cuda")
+    if fused:
+        rec.kernel_backproject(dev(inp["images"]), dev(inp["shifts"]), R, gid, rhs_out=rhs)
+    else:
+        rec.kernel(R, gid)
+        rec.backproject(dev(inp["images"]), dev(inp["shifts"]), R, gid, rhs_out=rhs)
+    rec.copy_out(F._lib.FIRM_OUT_KER, ker)
+    assert rec.lambda_eff() > 0.0                    # waits for the stream and the device's error flag
+    e_k = rel(ker.cpu().numpy()[1:, 1:, :N], Ker[1:, 1:, N:])
+    e_r = rel(rhs.cpu().numpy(), rhs_o)
+    print(f"N={N} M={M} {cfg} fused={fused}: Ker {e_k:.2e} A*b {e_r:.2e}")
+    assert e_k <= 3e-6 and e_r <= 3e-6
+    rec.close()
