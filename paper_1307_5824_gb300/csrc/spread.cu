@@ -147,43 +147,56 @@ __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN,
     }
     const bool valid = t >= 0;
     const int32_t kk = (int32_t)((uint32_t)(k1 & 0xffff) | ((uint32_t)k2 << 16));
-    for (int m = blockIdx.y; m < M; m += gridDim.y) {
-        int key = -1, c = 0;
-        uint4 pt = make_uint4(0u, 0u, 0u, 0u);
-        float2 wv = make_float2(0.0f, 0.0f);
-        if (valid) {
-            const PointPos p = point_pos(a.geom[m], kk, a.ls, a.halfG, a.G);
-            const int bx = p.I[0] / kBrick, by = p.I[1] / kBrick, bz = p.I[2] / BZ;
-            key = (bz * a.nb + by) * a.nb + bx;
-            if (CH > 0) {
-                pt.x = coord_word<W>(p.I[0] - bx * kBrick, p.q[0]);
-                pt.y = coord_word<W>(p.I[1] - by * kBrick, p.q[1]);
-                pt.z = coord_word<W>(p.I[2] - bz * BZ, p.q[2]);
-                if (CH != 2) {
-                    const int g = min(max(__ldg(&a.gid[m]), 0), a.n_ctf - 1);
-                    pt.w = __float_as_uint(__ldg(&a.h2[(size_t)g * a.nH + t]));
+    // U images at a time: their cursor atomics are in flight together
+    constexpr int U = CH > 0 ? 2 : 1;
+    for (int m0 = blockIdx.y * U; m0 < M; m0 += gridDim.y * U) {
+        int key[U], c[U];
+        uint4 pt[U];
+        float2 wv[U];
+        unsigned grp[U];
+        uint32_t base[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const int m = m0 + j;
+            key[j] = -1;
+            c[j] = 0;
+            pt[j] = make_uint4(0u, 0u, 0u, 0u);
+            wv[j] = make_float2(0.0f, 0.0f);
+            if (valid && m < M) {
+                const PointPos p = point_pos(a.geom[m], kk, a.ls, a.halfG, a.G);
+                const int bx = p.I[0] / kBrick, by = p.I[1] / kBrick, bz = p.I[2] / BZ;
+                key[j] = (bz * a.nb + by) * a.nb + bx;
+                if (CH > 0) {
+                    pt[j].x = coord_word<W>(p.I[0] - bx * kBrick, p.q[0]);
+                    pt[j].y = coord_word<W>(p.I[1] - by * kBrick, p.q[1]);
+                    pt[j].z = coord_word<W>(p.I[2] - bz * BZ, p.q[2]);
+                    if (CH != 2) {
+                        const int g = min(max(__ldg(&a.gid[m]), 0), a.n_ctf - 1);
+                        pt[j].w = __float_as_uint(__ldg(&a.h2[(size_t)g * a.nH + t]));
+                    }
+                    if (CH >= 2) wv[j] = __ldg(&a.samples[(size_t)m * a.nH + t]);
+                } else {
+                    c[j] = region_base<W, BZ>(p, bx * kBrick, by * kBrick, bz * BZ) & 31;
                 }
-                if (CH >= 2) wv = __ldg(&a.samples[(size_t)m * a.nH + t]);
-            } else {
-                c = region_base<W, BZ>(p, bx * kBrick, by * kBrick, bz * BZ) & 31;
             }
+            grp[j] = __match_any_sync(0xffffffffu, key[j]);
+            base[j] = 0;
+            if (key[j] >= 0 && lane == __ffs(grp[j]) - 1) base[j] = atomicAdd(&a.count[key[j]], (uint32_t)__popc(grp[j]));
         }
-        const unsigned grp = __match_any_sync(0xffffffffu, key);
-        const int leader = __ffs(grp) - 1;
-        uint32_t base = 0;
-        if (valid && lane == leader) base = atomicAdd(&a.count[key], (uint32_t)__popc(grp));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (valid) {
-            const uint32_t slot = base + (uint32_t)__popc(grp & ((1u << lane) - 1u));
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t slot =
+                __shfl_sync(0xffffffffu, base[j], __ffs(grp[j]) - 1) + (uint32_t)__popc(grp[j] & ((1u << lane) - 1u));
+            if (key[j] < 0) continue;
             if (CH > 0) {
-                if (CH == 2) pt.w = __float_as_uint(wv.x);
-                a.pts[slot] = pt;
-                if (CH == 2) reinterpret_cast<float*>(a.pts_w)[slot] = wv.y;
-                if (CH == 3) a.pts_w[slot] = wv;
+                if (CH == 2) pt[j].w = __float_as_uint(wv[j].x);
+                a.pts[slot] = pt[j];
+                if (CH == 2) reinterpret_cast<float*>(a.pts_w)[slot] = wv[j].y;
+                if (CH == 3) a.pts_w[slot] = wv[j];
             } else {
-                a.payload[slot] = ((uint32_t)m << kTBits) | (uint32_t)t;
-                a.cls[slot] = (uint8_t)c;
-                if (a.samples) a.samples_b[slot] = __ldg(&a.samples[(size_t)m * a.nH + t]);
+                a.payload[slot] = ((uint32_t)(m0 + j) << kTBits) | (uint32_t)t;
+                a.cls[slot] = (uint8_t)c[j];
+                if (a.samples) a.samples_b[slot] = __ldg(&a.samples[(size_t)(m0 + j) * a.nH + t]);
             }
         }
     }
@@ -444,7 +457,8 @@ static void bin_count_w(Plan& P, const BinArgs& a, int M, bool kc) {
 template <int W>
 static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
     const int hN = P.N / 2, tiles_x = (hN + 1 + 3) / 4, n_tiles = tiles_x * ((P.N + 1 + 7) / 8);
-    const dim3 g((n_tiles + 7) / 8, (unsigned)(M < 65535 ? M : 65535));
+    const int mb = P.bin_mma ? (M + 1) / 2 : M;
+    const dim3 g((n_tiles + 7) / 8, (unsigned)(mb < 65535 ? mb : 65535));
     const int4* col = P.ws.colinfo;
     const bool sm = a.samples != nullptr;
     if (P.bin_mma) {

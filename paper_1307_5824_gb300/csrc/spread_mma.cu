@@ -149,21 +149,27 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
     const int n_work = a.counters[0];
     const float* const im2 = reinterpret_cast<const float*>(a.pts_w);      // A*b alone: imaginary parts
     if (tid == 0) s_item = atomicAdd(&a.counters[3], 1);
-    for (;;) {
-        if (tid < 32) s_hist[tid] = 0;
-        __syncthreads();
-        const int item = s_item;
+    __syncthreads();
+    int item = s_item;
+    int4 wk = make_int4(0, 0, 0, 0);
+    uint4 pt[PT];
+    // an item's points are loaded while the block writes out the item before it
+    auto fetch = [&]() {
         if (item >= n_work) return;
-        const int4 wk = a.work[item];
-        // the item's points; their rank in their class (arbitrary order); largest |h b|
-        uint4 pt[PT];
-        int cr[PT];                                // class | rank << 8
-        float wmax = 0.0f;
+        wk = a.work[item];
 #pragma unroll
         for (int u = 0; u < PT; ++u) {
             const int i = u * kSortThreads + tid;
             if (i < wk.z) pt[u] = __ldg(&a.pts[wk.y + i]);
         }
+    };
+    fetch();
+    while (item < n_work) {
+        if (tid < 32) s_hist[tid] = 0;
+        __syncthreads();
+        // rank of the points in their class (arbitrary order); largest |h b|
+        int cr[PT];                                // class | rank << 8
+        float wmax = 0.0f;
         if (CH >= 2) {
 #pragma unroll
             for (int u = 0; u < PT; ++u) {
@@ -267,15 +273,18 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
             if (fits)
                 for (int g = tid & 15; g < end / 16; g += 16) a.rec_cls[s_base + off / 16 + g] = (uint8_t)k;
         }
-        __syncthreads();
-        if (fits) {
-            uint4* out = reinterpret_cast<uint4*>(a.rec + (size_t)s_base * 16 * (RW / 16));
-            const uint4* in4 = reinterpret_cast<const uint4*>(s_rec);
-            for (int i = tid; i < total / 16 * (RW / 4); i += kSortThreads) out[i] = in4[i];
-        }
+        const int base = s_base;
         if (tid == 0) {
             if (!fits) atomicOr(&a.counters[2], 1);
-            a.rec_item[item] = make_int4(wk.x, s_base, fits ? total / 16 : 0, lgn | (ek + 128) << 8 | (eb + 128) << 16);
+            a.rec_item[item] = make_int4(wk.x, base, fits ? total / 16 : 0, lgn | (ek + 128) << 8 | (eb + 128) << 16);
+        }
+        __syncthreads();
+        item = s_item;
+        fetch();
+        if (fits) {
+            uint4* out = reinterpret_cast<uint4*>(a.rec + (size_t)base * RW);
+            const uint4* in4 = reinterpret_cast<const uint4*>(s_rec);
+            for (int i = tid; i < total / 16 * (RW / 4); i += kSortThreads) out[i] = in4[i];
         }
     }
 }
