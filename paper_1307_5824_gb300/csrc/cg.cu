@@ -2,9 +2,10 @@
 // (A*A + lam_eff I) x = A*b from x = 0, vectors FP32, scalars FP64.
 //
 // One iteration is the Toeplitz apply (whose first pass forms p = r + beta p and
-// whose last pass reduces <p, q>) followed by k_cg_update below.  Reductions are
-// two-level and deterministic: every block writes one FP64 partial, the last block
-// to finish (ticket counter) sums the partials in block order.  All scalar logic
+// whose last pass leaves partial sums of <p, q>) followed by k_cg_update below.
+// Reductions are two-level and deterministic: every block writes one FP64 partial; those
+// of <p, q> (and <r, z>) are summed by every block of the kernel that needs them, those
+// of <r, r> by the last block to finish (ticket counter), which also decides the stop.  All scalar logic
 // (alpha, beta, the stop test, breakdown) runs on the device; a kernel that finds
 // the `done` flag set returns at once, so batches of iterations can be queued
 // without reading anything back.  Scalars are FP64; the residual vector and the
@@ -13,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "dw.cuh"
+#include "fft_planes.cuh"
 #include "firm_internal.h"
 
 namespace firm {
@@ -29,17 +31,20 @@ __device__ __forceinline__ double block_sum(float2 v2, double* s_warp) {
     return b;   // valid in thread 0
 }
 
-// Sum of the gridDim.x partials in a fixed order (thread-strided, then a tree).
-__device__ __forceinline__ double final_sum(const double* red, double* s_fin) {
+// Sum of the gridDim.x partials in a fixed order (thread-strided, then within warps, then
+// over warps); valid in thread 0.
+__device__ __forceinline__ double final_sum(const double* red, double* s_warp) {
     double v = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += ((volatile const double*)red)[i];
-    s_fin[threadIdx.x] = v;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(&red[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) s_fin[threadIdx.x] += s_fin[threadIdx.x + s];
-        __syncthreads();
-    }
-    return s_fin[0];
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double b = 0.0;
+    if (threadIdx.x == 0)
+        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) b += s_warp[i];
+    return b;
 }
 
 // Returns true in every thread of the last block to finish.
@@ -60,7 +65,6 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(const float* __restrict_
                                                         CgState* cg, double* red, double* hist, int max_iter,
                                                         double rel_tol, int use_pc) {
     __shared__ double s_warp[kCgThreads / 32];
-    __shared__ double s_fin[kCgThreads];
     __shared__ bool s_last;
     float2 acc = make_float2(0.0f, 0.0f);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -73,20 +77,20 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(const float* __restrict_
     const double bs = block_sum(acc, s_warp);
     if (threadIdx.x == 0) red[blockIdx.x] = bs;
     if (!last_block(&cg->ticket_b, &s_last)) return;
-    const double rr = final_sum(red, s_fin);
+    const double rr = final_sum(red, s_warp);
     if (threadIdx.x == 0) {
         cg->rr = rr;
         cg->pq = 0.0;
         cg->beta = 0.0;
         cg->beta_f[0] = cg->beta_f[1] = 0.0f;
         cg->alpha = 0.0;
-        cg->alpha_f[0] = cg->alpha_f[1] = 0.0f;
         cg->bnorm = sqrt(rr);
         cg->tol = rel_tol > 0.0 ? rel_tol * sqrt(rr) : 0.0;
         cg->it = 0;
         cg->max_iter = max_iter;
         cg->status = FIRM_OK;
-        cg->rz = 0.0;
+        cg->rz = cg->rz_next = 0.0;
+        cg->pc_stop = 0;
         cg->use_pc = use_pc;
         cg->first = 1;
         cg->done = (rr == 0.0 || max_iter <= 0 || (cg->tol > 0.0 && sqrt(rr) <= cg->tol)) ? 1 : 0;
@@ -96,20 +100,39 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(const float* __restrict_
     }
 }
 
-// x += alpha p, r -= alpha q (alpha from the Toeplitz apply's last block), then
-// <r, r> and the next beta.
+// alpha from the Toeplitz apply's n_pq partial sums of <p, q> (every block forms it), then
+// x += alpha p, r -= alpha q, <r, r> and the next beta.
 __global__ void __launch_bounds__(kCgThreads) k_cg_update(float* __restrict__ x, float2* __restrict__ r,
                                                           const float* __restrict__ p, const float* __restrict__ q,
-                                                          size_t n4, CgState* cg, double* red, double* hist) {
+                                                          size_t n4, CgState* cg, double* red, double* hist,
+                                                          const double* red_pq, int n_pq) {
     __shared__ double s_warp[kCgThreads / 32];
-    __shared__ double s_fin[kCgThreads];
     __shared__ bool s_last;
+    pdl_wait();
+    pdl_launch();
+    __shared__ double s_pq, s_alpha;
     if (cg->done) return;
-    const double pq = cg->pq, rr = cg->rr;
-    const bool ok = pq > 0.0 && isfinite(cg->alpha);
+    if (cg->use_pc && cg->pc_stop) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            if (!(cg->rz_next == 0.0)) cg->status = FIRM_EBREAKDOWN;
+            cg->done = 1;
+        }
+        return;
+    }
+    const double rr = cg->rr, rz = cg->rz_next;
+    if (threadIdx.x < 32) {
+        const double v = partial_sum(red_pq, n_pq);
+        if (threadIdx.x == 0) {
+            s_pq = v;
+            s_alpha = (cg->use_pc ? rz : rr) / v;
+        }
+    }
+    __syncthreads();
+    const double pq = s_pq, alpha = s_alpha;
+    const bool ok = pq > 0.0 && isfinite(alpha);
     float2 acc = make_float2(0.0f, 0.0f);
     if (ok) {
-        const float2 a = make_float2(cg->alpha_f[0], cg->alpha_f[1]);
+        const float2 a = dw_from_double(alpha);
         float4* x4 = reinterpret_cast<float4*>(x);
         float4* r4 = reinterpret_cast<float4*>(r);
         const float4* p4 = reinterpret_cast<const float4*>(p);
@@ -136,9 +159,13 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_update(float* __restrict__ x,
     const double bs = block_sum(acc, s_warp);
     if (threadIdx.x == 0) red[blockIdx.x] = bs;
     if (!last_block(&cg->ticket_b, &s_last)) return;
-    const double rr_new = final_sum(red, s_fin);
+    const double rr_new = final_sum(red, s_warp);
     if (threadIdx.x == 0) {
         cg->ticket_b = 0;
+        cg->pq = pq;
+        cg->alpha = alpha;
+        cg->rz = rz;
+        cg->first = 0;
         if (!ok || !(rr_new == rr_new)) {
             cg->status = FIRM_EBREAKDOWN;
             cg->done = 1;
@@ -160,11 +187,12 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_update(float* __restrict__ x,
     }
 }
 
-// Four blocks per SM: enough loads in flight, and few enough blocks that the
-// last-block ticket (one atomic per block on one address) stays cheap.
+// At most four blocks per SM: enough loads in flight, and few enough blocks that the
+// last-block ticket (one atomic per block on one address) stays cheap; no more than the
+// volume's float4s give every thread one.
 static int cg_blocks(const Plan& P) {
-    const int b = P.num_sms * 4;
-    return b < kRedSlots ? b : kRedSlots;
+    const int b = P.num_sms * 4, n = (P.N * P.N * P.N / 4 + kCgThreads - 1) / kCgThreads;
+    return min(min(b, n), kRedSlots);
 }
 
 cudaError_t launch_cg_init(Plan& P, const float* rhs, int max_iter, double rel_tol, bool use_pc) {
@@ -181,9 +209,9 @@ cudaError_t launch_cg_init(Plan& P, const float* rhs, int max_iter, double rel_t
 cudaError_t launch_cg_update(Plan& P) {
     Workspace& w = P.ws;
     const size_t n4 = (size_t)P.N * P.N * P.N / 4;
-    k_cg_update<<<cg_blocks(P), kCgThreads, 0, P.stream>>>(w.x, w.r, w.p, w.q, n4, w.cg, w.red_b, w.hist);
     P.launches += 1;
-    return cudaGetLastError();
+    return launch_pdl(k_cg_update, cg_blocks(P), kCgThreads, 0, P.stream, w.x, w.r, w.p, w.q, n4, w.cg, w.red_b,
+                      w.hist, w.red_a, P.N);
 }
 
 }  // namespace firm

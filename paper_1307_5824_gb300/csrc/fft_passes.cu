@@ -29,6 +29,7 @@
 #include "bulk.cuh"
 #include "dw.cuh"
 #include "fft.cuh"
+#include "fft_planes.cuh"
 #include "firm_internal.h"
 
 namespace firm {
@@ -587,27 +588,11 @@ cudaError_t launch_image_dft(Plan& P, int M, const void* images, const double* s
 // ---------------------------------------------------------------------------
 // Toeplitz apply (CG-fused when cg != nullptr)
 // ---------------------------------------------------------------------------
+// Row and column passes of the static entry point (firm_toeplitz_apply_static)
 struct TRowsFwdOp : NoFinish {
-    const float* x; float* p; const float2* r; const CgState* cg; float2* out; const float2* tw; int n_rows, N;
-    const float* z = nullptr;   // preconditioned residual: p = z + beta p when set
-    float bh = 0.0f, bl = 0.0f; // beta as a double-word, read once per block
-    __device__ __forceinline__ void prepare() {
-        if (cg) { bh = cg->beta_f[0]; bl = cg->beta_f[1]; }
-    }
+    const float* x; float2* out; const float2* tw; int n_rows, N;
     __device__ __forceinline__ float2 load(int row, int n) const {
-        if (n >= N) return make_float2(0.0f, 0.0f);
-        const size_t i = (size_t)row * N + n;
-        if (cg) {   // p = r + beta p (r, beta double-words) or p = z + beta p; stored by post()
-            const float pv = __ldg(&p[i]);
-            float ah, al;
-            if (z) { ah = __ldg(&z[i]); al = 0.0f; }
-            else { const float2 rv = __ldg(&r[i]); ah = rv.x; al = rv.y; }
-            return make_float2(fmaf(bh, pv, ah) + fmaf(bl, pv, al), 0.0f);
-        }
-        return make_float2(__ldg(&x[i]), 0.0f);
-    }
-    __device__ __forceinline__ void post(int row, int n, float2 v) const {
-        if (cg && n < N) p[(size_t)row * N + n] = v.x;
+        return make_float2(n < N ? __ldg(&x[(size_t)row * N + n]) : 0.0f, 0.0f);
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
         if (k <= N) out[(size_t)row * (N + 1) + k] = v;
@@ -631,28 +616,17 @@ struct TColsYInvOp {
         if (k < N) out[((size_t)o * N + k) * (N + 1) + i] = v;
     }
 };
-struct TRowsInvOp {
-    const float2* in; const float* x; float* y; double* red; CgState* cg; const float2* tw;
-    int n_rows, N; float scale, lam;
-    const float* lam_p;   // device lam_eff (overrides lam when set)
-    float2* acc;   // per-thread partial <x, y> (CG), double-word
-    __device__ __forceinline__ void prepare() {
-        if (lam_p) lam = __ldg(lam_p);
-    }
+struct TRowsInvOp : NoFinish {
+    const float2* in; const float* x; float* y; const float2* tw; int n_rows, N; float scale, lam;
     __device__ __forceinline__ float2 load(int row, int n) const {
         const float2* rr = in + (size_t)row * (N + 1);
         return n <= N ? __ldg(&rr[n]) : c_conj(__ldg(&rr[2 * N - n]));
     }
-    __device__ __forceinline__ float pre(int row, int k) const {
-        return k < N ? __ldg(&x[(size_t)row * N + k]) : 0.0f;
-    }
-    __device__ __forceinline__ void store(int row, int k, float2 v, float xv) const {
+    __device__ __forceinline__ void store(int row, int k, float2 v) const {
         if (k >= N) return;
-        const float yv = fmaf(v.x, scale, lam * xv);
-        y[(size_t)row * N + k] = yv;
-        if (cg) *acc = dw_acc_prod(*acc, xv, yv);
+        const size_t i = (size_t)row * N + k;
+        y[i] = fmaf(v.x, scale, lam * __ldg(&x[i]));
     }
-    __device__ __forceinline__ void finish() const {}
 };
 
 // The z pass: forward, times K-hat, inverse; tile of TX<L>() adjacent (j2, j1) columns.
@@ -661,6 +635,8 @@ __global__ void __launch_bounds__(kThreads) k_toep_z(float2* __restrict__ t2, co
                                                      const float2* __restrict__ tw, int n_inner, int N,
                                                      const CgState* cg) {
     extern __shared__ float2 S[];
+    pdl_wait();
+    pdl_launch();
     if (cg && cg->done) return;
     const int c0 = blockIdx.x * TX<L>();
     const int nl = min(TX<L>(), n_inner - c0);
@@ -674,189 +650,124 @@ __global__ void __launch_bounds__(kThreads) k_toep_z(float2* __restrict__ t2, co
     block_fft_mul_ifft<L>(nl, ld, mul, st, S, tw);
 }
 
-// Last pass of the apply with the CG reduction of <p, Ap> (last-block pattern).
-template <int L>
-__global__ void __launch_bounds__(kThreads) k_toep_rows_inv(TRowsInvOp op) {
-    extern __shared__ float2 S[];
-    __shared__ double s_red[kThreads / 32];
-    __shared__ bool s_last;
-    if (op.cg && op.cg->done) return;
-    constexpr int ROWS = rows_per_block<L>();
-    const int r0 = blockIdx.x * ROWS;
-    const int nl = min(ROWS, op.n_rows - r0);
-    float2 acc = make_float2(0.0f, 0.0f);
-    op.prepare();
-    op.acc = &acc;
-    auto ld = [&](int line, int n) { return op.load(r0 + line, n); };
-    auto pre = [&](int line, int k) { return op.pre(r0 + line, k); };
-    auto st = [&](int line, int k, float2 v, float xv) { op.store(r0 + line, k, v, xv); };
-    fft_step1<L, +1, false>(nl, ld, S, op.tw);
-    __syncthreads();
-    fft_step2_pre<L, +1, false>(nl, pre, st, S);
-    if (!op.cg) return;
-    // block reduction
-    const float2 wsum = dw_warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = dw_to_double(wsum);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double b = 0.0;
-        for (int i = 0; i < kThreads / 32; ++i) b += s_red[i];
-        op.red[blockIdx.x] = b;
-        __threadfence();
-        const unsigned t = atomicAdd(&op.cg->ticket_a, 1u);
-        s_last = (t == gridDim.x - 1);
+// The Toeplitz apply's x and y transforms (fft_planes.cuh); the z pass runs between them.
+// x rows (p = r + beta p, or p = z + beta p, when CG-fused), then y (N nonzero of 2N).
+template <int N> struct ToepFwdOp {
+    const float* x; float* p; const float2* r; const float* z; const CgState* cg;
+    float bh, bl;               // beta as a double-word
+    size_t base;                // first voxel of the plane
+    __device__ __forceinline__ float one(size_t i) const {
+        if (!cg) return __ldg(&x[i]);
+        const float pv = p[i];
+        float ah, al;
+        if (z) { ah = __ldg(&z[i]); al = 0.0f; }
+        else { const float2 rv = __ldg(&r[i]); ah = rv.x; al = rv.y; }
+        return fmaf(bh, pv, ah) + fmaf(bl, pv, al);
     }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // deterministic final sum over block partials, in block order
-    double v = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += ((volatile double*)op.red)[i];
-    // fixed-order tree over threads
-    __shared__ double s_fin[kThreads];
-    s_fin[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = kThreads / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) s_fin[threadIdx.x] += s_fin[threadIdx.x + s];
-        __syncthreads();
+    __device__ __forceinline__ float2 load(int pair, int n) const {
+        if (n >= N) return make_float2(0.0f, 0.0f);
+        const size_t i = base + (size_t)(2 * pair) * N + n;
+        return make_float2(one(i), one(i + N));
     }
-    if (threadIdx.x == 0) {
-        const double pq = s_fin[0];
-        const double alpha = (op.cg->use_pc ? op.cg->rz : op.cg->rr) / pq;
-        op.cg->pq = pq;
-        op.cg->alpha = alpha;
-        const float2 af = dw_from_double(isfinite(alpha) ? alpha : 0.0);
-        op.cg->alpha_f[0] = af.x;
-        op.cg->alpha_f[1] = af.y;
-        op.cg->ticket_a = 0;
+    __device__ __forceinline__ void post(int pair, int n, float2 v) const {
+        if (!cg || n >= N) return;
+        const size_t i = base + (size_t)(2 * pair) * N + n;
+        p[i] = v.x;
+        p[i + N] = v.y;
     }
-}
-
-// The Toeplitz apply's x and y transforms, one z-plane per CTA (the z pass between
-// them stays a column pass): the plane's N x (N+1) half spectrum (rows of 2N padded
-// samples, k1 in [0, N]) stays in shared memory between the row and the column
-// transforms, so the intermediate never goes through L2 or HBM and the apply is three
-// launches instead of five.  Rows and columns go in the fewest batches that fit the
-// exchange buffer beside the plane in 224 KB.
-template <int L> struct TPlane {
-    static constexpr int N = L / 2, H = N + 1;
-    static constexpr int kBudget = 224 * 1024 / (int)sizeof(float2);
-    static constexpr int kPlane = N * H;
-    static constexpr int kRowElems = Split<L>::L1 * (Split<L>::L2 + 1);
-    static constexpr int rb0 = (kBudget - kPlane) / kRowElems < N ? (kBudget - kPlane) / kRowElems : N;
-    static constexpr int RB = (N + (N + rb0 - 1) / rb0 - 1) / ((N + rb0 - 1) / rb0);     // rows per batch
-    static constexpr int cb0 = (kBudget - kPlane) / L < H ? (kBudget - kPlane) / L : H;
-    static constexpr int CB = (H + (H + cb0 - 1) / cb0 - 1) / ((H + cb0 - 1) / cb0);     // columns per batch
-    static constexpr int kX = smem_elems<L, false>(RB) > smem_elems<L, true>(CB) ? smem_elems<L, false>(RB)
-                                                                                   : smem_elems<L, true>(CB);
-    static constexpr int kSmem = kPlane + kX;                                          // float2 elements
-    static constexpr int kL = Split<L>::L1 > Split<L>::L2 ? Split<L>::L1 : Split<L>::L2;
-    static constexpr int kItems = (RB > CB ? RB : CB) * kL;
-    static constexpr int kThreadsP = kItems < 1024 ? (kItems + 31) / 32 * 32 : 1024;
 };
 
-// x rows (p = r + beta p, or p = z + beta p, when CG-fused) forward into the plane,
-// then y forward (N nonzero of 2N) into t2[z][k2][k1].
 template <int L>
-__global__ void __launch_bounds__(TPlane<L>::kThreadsP) k_toep_plane_fwd(TRowsFwdOp op, float2* __restrict__ t2,
-                                                                        const CgState* cg) {
-    using T = TPlane<L>;
-    constexpr int N = T::N, H = T::H;
+__global__ void __launch_bounds__(PlaneCfg<L, L / 2>::kThreads) k_toep_plane_fwd(const float* x, float* p, const float2* r,
+                                                                                const float* z, float2* t2,
+                                                                                const float2* tw, const double* red,
+                                                                                CgState* cg) {
+    constexpr int N = L / 2;
     extern __shared__ float2 S[];
+    pdl_wait();
+    pdl_launch();
     if (cg && cg->done) return;
-    float2* plane = S;                          // [y][k1]
-    float2* X = S + T::kPlane;
-    const int row0 = blockIdx.x * N;            // rows of this plane in [z][y] order
-    op.prepare();
-    for (int r0 = 0; r0 < N; r0 += T::RB) {
-        const int nl = min(T::RB, N - r0);
-        auto ld = [&](int line, int n) { return op.load(row0 + r0 + line, n); };
-        auto post = [&](int line, int n, float2 v) { op.post(row0 + r0 + line, n, v); };
-        auto st = [&](int line, int k, float2 v) {
-            if (k <= N) plane[(r0 + line) * H + k] = v;
-        };
-        fft_step1_post<L, -1, false>(nl, ld, post, X, op.tw);
+    const int plane = blockIdx.x;
+    ToepFwdOp<N> op{x, p, r, z, cg, 0.0f, 0.0f, (size_t)plane * N * N};
+    if (cg && z) {                               // preconditioned CG: beta from the preconditioner's partial sums
+        __shared__ float2 s_beta;
+        __shared__ bool s_stop;
+        if (threadIdx.x < 32) {
+            // flexible (Polak-Ribiere) beta = (<r,z_new> - <r,z_old>) / <r_old,z_old>, which
+            // tolerates the FP32 rounding of the preconditioner apply; P must be positive
+            // definite
+            const double rz = partial_sum(red, N, 2), rz_old = partial_sum(red + 1, N, 2);
+            if (threadIdx.x == 0) {
+                const double beta = cg->first ? 0.0 : fmax(0.0, (rz - rz_old) / cg->rz);
+                const bool stop = !(rz > 0.0) || !isfinite(rz);
+                s_beta = dw_from_double(beta);
+                s_stop = stop;
+                if (blockIdx.x == 0) {           // taken over by the vector update
+                    cg->rz_next = rz;
+                    cg->beta = beta;
+                    cg->pc_stop = stop ? 1 : 0;
+                }
+            }
+        }
         __syncthreads();
-        fft_step2<L, -1, false>(nl, st, X);
-        __syncthreads();
+        if (s_stop) return;
+        op.bh = s_beta.x;
+        op.bl = s_beta.y;
+    } else if (cg) {
+        op.bh = cg->beta_f[0];
+        op.bl = cg->beta_f[1];
     }
-    float2* out = t2 + (size_t)blockIdx.x * 2 * N * H;
-    for (int c0 = 0; c0 < H; c0 += T::CB) {
-        const int nl = min(T::CB, H - c0);
-        auto ld = [&](int line, int n) { return n < N ? plane[n * H + c0 + line] : make_float2(0.0f, 0.0f); };
-        auto st = [&](int line, int k, float2 v) { out[(size_t)k * H + c0 + line] = v; };
-        block_fft<L, -1, true>(nl, ld, st, X, op.tw);
-    }
+    plane_forward<L, N>(op, t2 + (size_t)plane * L * (N + 1), tw, S);
 }
 
-// y inverse of t2[z] keeping y < N into the plane, then the Hermitian x rows back to
-// real with the crop, 1/(2N)^3 and + lam x (op.store); CG-fused: <x, y> reduced, the
-// last CTA forms alpha (sums in CTA order).
+// y inverse of t2[z] keeping y < N, then the Hermitian x rows back to real with the crop,
+// 1/(2N)^3 and + lam x; CG-fused: every block leaves its part of <x, y> in red.
+template <int N> struct ToepInvOp {
+    const float* x; float* y;
+    float scale, lam;
+    bool dot;
+    float2 acc;                 // partial <x, y>, double-word
+    size_t base;
+    __device__ __forceinline__ float2 pre(int pair, int n) const {
+        if (n >= N) return make_float2(0.0f, 0.0f);
+        const size_t i = base + (size_t)(2 * pair) * N + n;
+        return make_float2(__ldg(&x[i]), __ldg(&x[i + N]));
+    }
+    __device__ __forceinline__ void store(int pair, int n, float2 v, float2 xv) {
+        if (n >= N) return;
+        const size_t i = base + (size_t)(2 * pair) * N + n;
+        const float ya = fmaf(v.x, scale, lam * xv.x), yb = fmaf(v.y, scale, lam * xv.y);
+        y[i] = ya;
+        y[i + N] = yb;
+        if (dot) {
+            acc = dw_acc_prod(acc, xv.x, ya);
+            acc = dw_acc_prod(acc, xv.y, yb);
+        }
+    }
+};
+
 template <int L>
-__global__ void __launch_bounds__(TPlane<L>::kThreadsP) k_toep_plane_inv(TRowsInvOp op, const float2* __restrict__ t2) {
-    using T = TPlane<L>;
-    constexpr int N = T::N, H = T::H;
+__global__ void __launch_bounds__(PlaneCfg<L, L / 2>::kThreads) k_toep_plane_inv(const float* x, float* y, const float2* t2,
+                                                                                const float2* tw, const float* lam_p,
+                                                                                float scale, double* red, CgState* cg) {
+    constexpr int N = L / 2;
     extern __shared__ float2 S[];
     __shared__ double s_red[32];
-    __shared__ bool s_last;
-    if (op.cg && op.cg->done) return;
-    float2* plane = S;                          // [y][k1]
-    float2* X = S + T::kPlane;
-    const float2* in = t2 + (size_t)blockIdx.x * 2 * N * H;
-    for (int c0 = 0; c0 < H; c0 += T::CB) {
-        const int nl = min(T::CB, H - c0);
-        auto ld = [&](int line, int n) { return __ldg(&in[(size_t)n * H + c0 + line]); };
-        auto st = [&](int line, int k, float2 v) {
-            if (k < N) plane[k * H + c0 + line] = v;
-        };
-        block_fft<L, +1, true>(nl, ld, st, X, op.tw);
-    }
-    float2 acc = make_float2(0.0f, 0.0f);
-    op.prepare();
-    op.acc = &acc;
-    const int row0 = blockIdx.x * N;
-    for (int r0 = 0; r0 < N; r0 += T::RB) {
-        const int nl = min(T::RB, N - r0);
-        auto ld = [&](int line, int n) {
-            const float2* row = plane + (r0 + line) * H;
-            return n <= N ? row[n] : c_conj(row[2 * N - n]);
-        };
-        auto pre = [&](int line, int k) { return op.pre(row0 + r0 + line, k); };
-        auto st = [&](int line, int k, float2 v, float xv) { op.store(row0 + r0 + line, k, v, xv); };
-        fft_step1<L, +1, false>(nl, ld, X, op.tw);
-        __syncthreads();
-        fft_step2_pre<L, +1, false>(nl, pre, st, X);
-        __syncthreads();
-    }
-    if (!op.cg) return;
+    pdl_wait();
+    pdl_launch();
+    if (cg && cg->done) return;
+    const int plane = blockIdx.x;
+    ToepInvOp<N> op{x, y, scale, __ldg(lam_p), cg != nullptr, make_float2(0.0f, 0.0f), (size_t)plane * N * N};
+    plane_inverse<L, N>(op, t2 + (size_t)plane * L * (N + 1), tw, S);
+    if (!cg) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    const float2 wsum = dw_warp_sum(acc);
+    const float2 wsum = dw_warp_sum(op.acc);
     if (lane == 0) s_red[wid] = dw_to_double(wsum);
     __syncthreads();
     if (threadIdx.x == 0) {
         double b = 0.0;
         for (int i = 0; i < nw; ++i) b += s_red[i];
-        op.red[blockIdx.x] = b;
-        __threadfence();
-        const unsigned t = atomicAdd(&op.cg->ticket_a, 1u);
-        s_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!s_last || wid != 0) return;
-    __threadfence();
-    double v = 0.0;
-    for (int i = lane; i < (int)gridDim.x; i += 32) v += ((volatile double*)op.red)[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) {
-        const double pq = v;
-        const double alpha = (op.cg->use_pc ? op.cg->rz : op.cg->rr) / pq;
-        op.cg->pq = pq;
-        op.cg->alpha = alpha;
-        const float2 af = dw_from_double(isfinite(alpha) ? alpha : 0.0);
-        op.cg->alpha_f[0] = af.x;
-        op.cg->alpha_f[1] = af.y;
-        op.cg->ticket_a = 0;
+        red[blockIdx.x] = b;
     }
 }
 
@@ -892,30 +803,27 @@ __global__ void __launch_bounds__(kThreads) k_cols_cg(const Op op, const CgState
 template <int L>
 static cudaError_t toeplitz_l(Plan& P, const float* x, float* y, const float2* cg_r, CgState* cg,
                               const float* cg_z) {
-    using T = TPlane<L>;
+    constexpr int N = L / 2;
+    using T = PlaneCfg<L, N>;
     Workspace& w = P.ws;
-    const int N = P.N;
-    const size_t smem_plane = sizeof(float2) * T::kSmem;
     const size_t smem_cols = sizeof(float2) * smem_elems<L, true>(TX<L>());
     cudaError_t e;
     // pass 1: per z-plane, rows of x (or p = r + beta p) forward, then y forward
-    TRowsFwdOp a{{}, x, cg ? const_cast<float*>(x) : nullptr, cg_r, cg, nullptr, w.tw_2n, N * N, N, cg_z};
-    if ((e = cudaFuncSetAttribute(k_toep_plane_fwd<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plane)))
-        return e;
-    k_toep_plane_fwd<L><<<N, T::kThreadsP, smem_plane, P.stream>>>(a, w.t2, cg);
+    e = launch_pdl(k_toep_plane_fwd<L>, N, T::kThreads, T::kSmem, P.stream, x,
+                   cg ? const_cast<float*>(x) : nullptr, cg_r, cg_z, w.t2, w.tw_2n, w.red_a, cg);
+    if (e != cudaSuccess) return e;
     // pass 2: z forward x K-hat x z inverse
     const int n_inner = 2 * N * (N + 1);
-    if ((e = cudaFuncSetAttribute(k_toep_z<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols))) return e;
-    k_toep_z<L><<<(n_inner + TX<L>() - 1) / TX<L>(), kThreads, smem_cols, P.stream>>>(w.t2, w.khat, w.tw_2n, n_inner, N, cg);
+    e = launch_pdl(k_toep_z<L>, (n_inner + TX<L>() - 1) / TX<L>(), kThreads, smem_cols, P.stream, w.t2, w.khat, w.tw_2n,
+                   n_inner, N, cg);
+    if (e != cudaSuccess) return e;
     // pass 3: per z-plane, y inverse (keep y < N), rows inverse (Hermitian), crop,
     // scale, + lam x, <x, y>
     const float scale = 1.0f / ((float)L * (float)L * (float)L);
-    TRowsInvOp f{nullptr, x, y, w.red_a, cg, w.tw_2n, N * N, N, scale, 0.0f, w.lam, nullptr};
-    if ((e = cudaFuncSetAttribute(k_toep_plane_inv<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plane)))
-        return e;
-    k_toep_plane_inv<L><<<N, T::kThreadsP, smem_plane, P.stream>>>(f, w.t2);
+    e = launch_pdl(k_toep_plane_inv<L>, N, T::kThreads, T::kSmem, P.stream, x, y, w.t2, w.tw_2n, w.lam,
+                   scale, w.red_a, cg);
     P.launches += 3;
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_toeplitz(Plan& P, const float* x, float* y, const float2* cg_r, CgState* cg,
@@ -960,6 +868,8 @@ template <int L>
 __global__ void __launch_bounds__(kThreads) k_pc_z(float2* __restrict__ u, const float* __restrict__ d,
                                                    const float2* __restrict__ tw, int n_inner, const CgState* cg) {
     extern __shared__ float2 S[];
+    pdl_wait();
+    pdl_launch();
     if (cg->done) return;
     const int c0 = blockIdx.x * TX<L>();
     const int nl = min(TX<L>(), n_inner - c0);
@@ -969,87 +879,65 @@ __global__ void __launch_bounds__(kThreads) k_pc_z(float2* __restrict__ u, const
     block_fft_mul_ifft<L>(nl, ld, mul, st, S, tw);
 }
 
-// The preconditioner's x and y transforms, one z-plane per CTA: the plane's N x (N/2+1)
-// half spectrum stays in shared memory between the row and the column transforms, so
-// the N^3 transform is three passes (plane forward, z with the diagonal, plane
-// inverse) instead of five, and each plane is read and written once per direction.
-// All rows of the plane are one batch and all columns one batch, with up to 1024
-// threads, so a CTA has the whole plane's loads in flight at once (214 KB of shared
-// memory at N = 128).
-template <int L> __host__ __device__ constexpr int plane_threads() {
-    return L * Split<L>::L2 < 1024 ? L * Split<L>::L2 : 1024;
-}
-template <int L> __host__ __device__ constexpr int pc_plane_smem_elems() {
-    constexpr int a = smem_elems<L, false>(L), b = smem_elems<L, true>(L / 2 + 1);
-    return L * (L / 2 + 1) + (a > b ? a : b);
-}
-
 // u[z][k2][k1] = forward 2D DFT over (x, y) of plane z of r (double-word, summed to FP32)
+template <int N> struct PcFwdOp {
+    const float2* r;
+    __device__ __forceinline__ float2 load(int pair, int n) const {
+        const float2 a = __ldg(&r[(size_t)(2 * pair) * N + n]), b = __ldg(&r[(size_t)(2 * pair + 1) * N + n]);
+        return make_float2(a.x + a.y, b.x + b.y);
+    }
+    __device__ __forceinline__ void post(int, int, float2) const {}
+};
+
 template <int L>
-__global__ void __launch_bounds__(plane_threads<L>()) k_pc_plane_fwd(const float2* __restrict__ r,
-                                                                    float2* __restrict__ u,
-                                                                    const float2* __restrict__ tw, const CgState* cg) {
-    extern __shared__ float2 S[];
-    if (cg->done) return;
+__global__ void __launch_bounds__(PlaneCfg<L, L>::kThreads) k_pc_plane_fwd(const float2* r, float2* u, const float2* tw,
+                                                                          const CgState* cg) {
     constexpr int N = L, H = L / 2 + 1;
-    float2* plane = S;                          // [y][k1]
-    float2* X = S + N * H;                      // exchange buffer of the transforms
-    const float2* rz = r + (size_t)blockIdx.x * N * N;
-    auto ld_r = [&](int line, int n) {
-        const float2 v = __ldg(&rz[(size_t)line * N + n]);
-        return make_float2(v.x + v.y, 0.0f);
-    };
-    auto st_r = [&](int line, int k, float2 v) {
-        if (k <= N / 2) plane[line * H + k] = v;
-    };
-    block_fft<L, -1, false>(N, ld_r, st_r, X, tw);
-    float2* uz = u + (size_t)blockIdx.x * N * H;
-    auto ld_c = [&](int line, int n) { return plane[n * H + line]; };
-    auto st_c = [&](int line, int k, float2 v) { uz[(size_t)k * H + line] = v; };
-    block_fft<L, -1, true>(H, ld_c, st_c, X, tw);
+    extern __shared__ float2 S[];
+    pdl_wait();
+    pdl_launch();
+    if (cg->done) return;
+    const int plane = blockIdx.x;
+    PcFwdOp<N> op{r + (size_t)plane * N * N};
+    plane_forward<L, N>(op, u + (size_t)plane * N * H, tw, S);
 }
 
-// Plane z of the inverse 2D DFT of u (Hermitian along x) is the new z = P r; the CTA
-// also reduces <r, z_new> and <r, z_old> for the flexible (Polak-Ribiere)
-// beta = (<r,z_new> - <r,z_old>) / <r_old,z_old>, which tolerates the FP32 rounding of
-// the preconditioner apply; the last CTA forms beta (sums in CTA order).
+// Plane z of the inverse 2D DFT of u (Hermitian along x) is the new z = P r; every block
+// leaves its parts of <r, z_new> and <r, z_old> in red (beta is formed by the next
+// Toeplitz apply).
+template <int N> struct PcInvOp {
+    struct Pre { float2 ra, rb; float za, zb; };
+    const float2* r; float* z;
+    float2 acc, acc_old;
+    __device__ __forceinline__ Pre pre(int pair, int n) const {
+        const size_t i = (size_t)(2 * pair) * N + n;
+        return Pre{__ldg(&r[i]), __ldg(&r[i + N]), z[i], z[i + N]};
+    }
+    __device__ __forceinline__ void store(int pair, int n, float2 v, const Pre& p) {
+        const size_t i = (size_t)(2 * pair) * N + n;
+        acc_old = dw_acc_mul(acc_old, p.ra, p.za);
+        acc_old = dw_acc_mul(acc_old, p.rb, p.zb);
+        z[i] = v.x;
+        z[i + N] = v.y;
+        acc = dw_acc_mul(acc, p.ra, v.x);
+        acc = dw_acc_mul(acc, p.rb, v.y);
+    }
+};
+
 template <int L>
-__global__ void __launch_bounds__(plane_threads<L>()) k_pc_plane_inv(const float2* __restrict__ u,
-                                                                    const float2* __restrict__ r,
-                                                                    float* __restrict__ z, double* red, CgState* cg,
-                                                                    const float2* __restrict__ tw) {
+__global__ void __launch_bounds__(PlaneCfg<L, L>::kThreads) k_pc_plane_inv(const float2* u, const float2* r, float* z,
+                                                                          double* red, const CgState* cg, const float2* tw) {
+    constexpr int N = L, H = L / 2 + 1;
     extern __shared__ float2 S[];
     __shared__ double s_red[2][32];
-    __shared__ bool s_last;
+    pdl_wait();
+    pdl_launch();
     if (cg->done) return;
-    constexpr int N = L, H = L / 2 + 1;
-    float2* plane = S;                          // [y][k1]
-    float2* X = S + N * H;
-    const float2* uz = u + (size_t)blockIdx.x * N * H;
-    auto ld_c = [&](int line, int n) { return uz[(size_t)n * H + line]; };
-    auto st_c = [&](int line, int k, float2 v) { plane[k * H + line] = v; };
-    block_fft<L, +1, true>(H, ld_c, st_c, X, tw);
-    float2 acc = make_float2(0.0f, 0.0f), acc_old = make_float2(0.0f, 0.0f);
-    const size_t zbase = (size_t)blockIdx.x * N * N;
-    auto ld = [&](int line, int n) {
-        const float2* row = plane + line * H;
-        return n <= N / 2 ? row[n] : c_conj(row[N - n]);
-    };
-    auto pre = [&](int line, int k) {           // r (double-word) and the previous z
-        const size_t i = zbase + (size_t)line * N + k;
-        const float2 ri = __ldg(&r[i]);
-        return make_float3(ri.x, ri.y, z[i]);
-    };
-    auto st = [&](int line, int k, float2 v, float3 rzv) {
-        const float2 ri = make_float2(rzv.x, rzv.y);
-        acc_old = dw_acc_mul(acc_old, ri, rzv.z);
-        z[zbase + (size_t)line * N + k] = v.x;
-        acc = dw_acc_mul(acc, ri, v.x);
-    };
-    fft_step1<L, +1, false>(N, ld, X, tw);
-    __syncthreads();
-    fft_step2_pre<L, +1, false>(N, pre, st, X);
-    const float2 w0 = dw_warp_sum(acc), w1 = dw_warp_sum(acc_old);
+    const int plane = blockIdx.x;
+    const size_t zbase = (size_t)plane * N * N;
+    PcInvOp<N> op{r + zbase, z + zbase, make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+    plane_inverse<L, N>(op, u + (size_t)plane * N * H, tw, S);
+    const float2 w0 = dw_warp_sum(op.acc), w1 = dw_warp_sum(op.acc_old);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     if (lane == 0) {
         s_red[0][wid] = dw_to_double(w0);
@@ -1061,36 +949,6 @@ __global__ void __launch_bounds__(plane_threads<L>()) k_pc_plane_inv(const float
         for (int i = 0; i < nw; ++i) { b0 += s_red[0][i]; b1 += s_red[1][i]; }
         red[2 * blockIdx.x] = b0;
         red[2 * blockIdx.x + 1] = b1;
-        __threadfence();
-        const unsigned t = atomicAdd(&cg->ticket_c, 1u);
-        s_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!s_last || wid != 0) return;
-    __threadfence();
-    double v0 = 0.0, v1 = 0.0;
-    for (int i = lane; i < (int)gridDim.x; i += 32) {
-        v0 += ((volatile double*)red)[2 * i];
-        v1 += ((volatile double*)red)[2 * i + 1];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-    }
-    if (lane == 0) {
-        const double rz_new = v0, rz_old_new_r = v1;
-        cg->beta = cg->first ? 0.0 : fmax(0.0, (rz_new - rz_old_new_r) / cg->rz);
-        const float2 bf = dw_from_double(cg->beta);
-        cg->beta_f[0] = bf.x;
-        cg->beta_f[1] = bf.y;
-        cg->rz = rz_new;
-        cg->first = 0;
-        cg->ticket_c = 0;
-        if (!(rz_new > 0.0) || !isfinite(rz_new)) {     // P must be positive definite
-            if (!(rz_new == 0.0)) cg->status = FIRM_EBREAKDOWN;
-            cg->done = 1;
-        }
     }
 }
 
@@ -1098,21 +956,18 @@ template <int L>
 static cudaError_t precond_l(Plan& P, const float2* r, float* z, CgState* cg) {
     Workspace& w = P.ws;
     constexpr int N = L, H = L / 2 + 1;
-    const size_t smem_plane = sizeof(float2) * pc_plane_smem_elems<L>();
+    using T = PlaneCfg<L, N>;
     const size_t smem_cols = sizeof(float2) * smem_elems<L, true>(TX<L>());
     float2* u = w.t1;                       // N x N x (N/2+1) complex
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_pc_plane_fwd<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plane)))
-        return e;
-    k_pc_plane_fwd<L><<<N, plane_threads<L>(), smem_plane, P.stream>>>(r, u, w.tw_n, cg);
+    cudaError_t e = launch_pdl(k_pc_plane_fwd<L>, N, T::kThreads, T::kSmem, P.stream, r, u, w.tw_n, cg);
+    if (e != cudaSuccess) return e;
     const int n_inner = N * H;
-    if ((e = cudaFuncSetAttribute(k_pc_z<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols))) return e;
-    k_pc_z<L><<<(n_inner + TX<L>() - 1) / TX<L>(), kThreads, smem_cols, P.stream>>>(u, w.pc_diag, w.tw_n, n_inner, cg);
-    if ((e = cudaFuncSetAttribute(k_pc_plane_inv<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_plane)))
-        return e;
-    k_pc_plane_inv<L><<<N, plane_threads<L>(), smem_plane, P.stream>>>(u, r, z, w.red_a, cg, w.tw_n);
+    e = launch_pdl(k_pc_z<L>, (n_inner + TX<L>() - 1) / TX<L>(), kThreads, smem_cols, P.stream, u, w.pc_diag, w.tw_n,
+                   n_inner, cg);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(k_pc_plane_inv<L>, N, T::kThreads, T::kSmem, P.stream, u, r, z, w.red_a, cg, w.tw_n);
     P.launches += 3;
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_precond(Plan& P, const float2* r, float* z, CgState* cg) {
@@ -1266,7 +1121,7 @@ static cudaError_t toeplitz_static_l(float2* scratch, const float* khat, const f
     constexpr int ROWS = rows_per_block<L>();
     const size_t smem_rows = sizeof(float2) * smem_elems<L, false>(ROWS);
     const size_t smem_cols = sizeof(float2) * smem_elems<L, true>(TX<L>());
-    TRowsFwdOp a{{}, x, nullptr, nullptr, nullptr, t1, tw, N * N, N};
+    TRowsFwdOp a{{}, x, t1, tw, N * N, N};
     if ((e = cudaFuncSetAttribute(k_rows_cg<L, TRowsFwdOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows)))
         return e;
     k_rows_cg<L, TRowsFwdOp><<<(N * N + ROWS - 1) / ROWS, kThreads, smem_rows, s>>>(a, nullptr);
@@ -1283,10 +1138,8 @@ static cudaError_t toeplitz_static_l(float2* scratch, const float* khat, const f
         return e;
     k_cols_cg<L, +1, TColsYInvOp><<<N * tiles_b, kThreads, smem_cols, s>>>(d, nullptr);
     const float scale = 1.0f / ((float)L * (float)L * (float)L);
-    TRowsInvOp f{t1, x, y, nullptr, nullptr, tw, N * N, N, scale, lam, nullptr, nullptr};
-    if ((e = cudaFuncSetAttribute(k_toep_rows_inv<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows)))
-        return e;
-    k_toep_rows_inv<L><<<(N * N + ROWS - 1) / ROWS, kThreads, smem_rows, s>>>(f);
+    TRowsInvOp f{{}, t1, x, y, tw, N * N, N, scale, lam};
+    if ((e = run_rows<L, +1>(f, s)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

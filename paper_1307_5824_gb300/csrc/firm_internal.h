@@ -58,11 +58,11 @@ struct CgState {
     double rz;        // <r, z> with z = P r (preconditioned solve)
     int use_pc;       // 1: preconditioned CG
     int first;        // 1 until the first preconditioner application
-    unsigned int ticket_c;
+    int pc_stop;      // 1: the preconditioner's <r, z> is not a positive number
     int pad_;
-    double alpha;     // step length of the current iteration (set with pq)
-    float alpha_f[2]; // alpha and beta as double-words (hi, lo) for the vector updates
-    float beta_f[2];
+    double rz_next;   // <r, z> of this iteration, taken into rz by the vector update
+    double alpha;     // step length of the last iteration
+    float beta_f[2];  // beta as a double-word (hi, lo)
 };
 
 struct Workspace {
