@@ -473,15 +473,22 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 }
 
 // Average points per brick of the ball from which the tensor-core form is the faster one
-// (binning and spreading together).  Its cost per brick is high -- 27 classes padded to 16
-// points, each flushed to the region -- and its cost per point low, the lower the more
-// channels share the window arithmetic.  Measured at N = 64, W = 6, in ms, bank-class form
-// against tensor-core form: kernel channel 0.65 / 0.76 at 282 points a brick, 0.88 / 0.91
-// at 470, 1.30 / 1.20 at 846; A*b 0.158 / 0.154 at 226, 0.47 / 0.23 at 754; both in one
-// pass 0.83 / 1.00 at 94, 1.05 / 1.08 at 188, 1.32 / 1.16 at 282.
+// (binning and spreading together).  Its cost per brick is high -- 25 or 27 classes padded
+// to 16 points, each flushed to the region -- and its cost per point low, the lower the
+// more channels share the window arithmetic.  Measured at N = 64, in ms, bank-class form
+// against tensor-core form.  W = 6: kernel channel 0.65 / 0.76 at 282 points a brick,
+// 0.88 / 0.91 at 470, 1.30 / 1.20 at 846; A*b 0.158 / 0.154 at 226, 0.47 / 0.23 at 754;
+// both in one pass 0.83 / 1.00 at 94, 1.05 / 1.08 at 188, 1.32 / 1.16 at 282.  W = 7:
+// kernel channel 0.85 / 1.06 at 282, 4.64 / 4.46 at 622 (N = 96), 1.84 / 1.62 at 846;
+// A*b 0.21 / 0.24 at 226, 0.73 / 0.37 at 754.  Both channels in one pass at W = 7 would
+// need 96 accumulators a thread, and W = 8 windows leave one first tap a class: neither is
+// built.
 bool mma_rule(const firm_params& p, size_t points, int nb, int ch) {
-    const double least = ch == 1 ? 500.0 : ch == 2 ? 220.0 : 200.0;
-    return p.W == 6 && (double)points >= least * 0.5236 * nb * nb * (double)nb;
+    double least;
+    if (p.W == 6) least = ch == 1 ? 500.0 : ch == 2 ? 220.0 : 200.0;
+    else if (p.W == 7 && ch < 3) least = ch == 1 ? 560.0 : 280.0;
+    else return false;
+    return (double)points >= least * 0.5236 * nb * nb * (double)nb;
 }
 
 size_t mma_slots(size_t points, int nb) {
@@ -1183,7 +1190,7 @@ cudaError_t launch_spread_batch(int n, int n_mma, bool kc, int W, const KbPoly& 
     const SpreadArgs* d = reinterpret_cast<const SpreadArgs*>(dev_desc);
     if (n_mma > 0) {
         k_batch_items<<<1, 32, 0, s>>>(d, n, 1, item_off + n + 1, queue + 1);
-        const cudaError_t e = launch_spread_mma_batch(n, kc, d, item_off + n + 1, queue + 1, poly, num_sms, s);
+        const cudaError_t e = launch_spread_mma_batch(n, kc, W, d, item_off + n + 1, queue + 1, poly, num_sms, s);
         if (e != cudaSuccess || n_mma == n) return e;
     }
     switch (W) {

@@ -156,7 +156,7 @@ __device__ __forceinline__ uint32_t coord_word(int cell, uint32_t q) {
 // Tensor-core form (spread_mma.cu); ch: 1 kernel channel, 2 A*b, 3 both.
 cudaError_t launch_mma_sort(Plan& P, const SpreadArgs& a, int ch);
 cudaError_t launch_spread_mma(Plan& P, const SpreadArgs& a, int ch);
-cudaError_t launch_spread_mma_batch(int n, bool kc, const SpreadArgs* desc, const int* item_off, int* queue,
+cudaError_t launch_spread_mma_batch(int n, bool kc, int W, const SpreadArgs* desc, const int* item_off, int* queue,
                                     const KbPoly& poly, int num_sms, cudaStream_t s);
 
 }  // namespace firm

@@ -38,12 +38,6 @@ constexpr int kMmaThreads = 256;
 constexpr int kMmaWarps = kMmaThreads / 32;
 constexpr int kSortThreads = 512;
 constexpr int kRunGroups = 8;                     // groups summed in FP32 before a class goes to the region
-// Staging of one warp: x and z windows of 2 groups of 16 points, y windows of 4 groups.
-// Strides are 8 mod 32 words, so that the four groups a warp stores together meet
-// different banks.
-constexpr int kXZWords = 264;                     // X hi 64 | X lo 64 | Z hi 64 | Z lo 64 | pad
-constexpr int kYWords = 136;                      // hi 64 | lo 64 | pad
-constexpr int kWarpWords = 2 * kXZWords + 4 * kYWords;
 // fp16 operands carry each axis window scaled by 2^kTapBits; the weights' scale is chosen
 // so that the products come out in the region's integer units.
 constexpr int kTapBits = 5;
@@ -51,15 +45,28 @@ constexpr float kTapScale = (float)(1 << kTapBits);
 
 // CH: 1 kernel channel, 2 A*b, 3 both (Ker, Re, Im).
 template <int W, int CH> struct MmaCfg {
-    static constexpr int kBases = 9 - W;                              // first taps per class and axis (8-cell window)
-    static constexpr int kPer = (kBrick + 1 + kBases - 1) / kBases;   // classes per axis
-    static constexpr int kClasses = kPer * kPer * kPer;
-    static constexpr int RG = kBrick + W, RG3 = RG * RG * RG;
+    // First taps per class: y and z windows fit 8 cells; x windows 8 cells at W = 6 (3 first
+    // taps, 27 classes) and 16 at W = 7 (all 9 first taps: 2 per class and axis would make
+    // 125 classes, too few points in each on the 4N grid; this way there are 25).
+    static constexpr int XS = W == 6 ? 8 : 16;                        // x cells of a class
+    static constexpr int kBases = 9 - W, kBasesX = XS + 1 - W > 9 ? 9 : XS + 1 - W;
+    static constexpr int kPer = (kBrick + 1 + kBases - 1) / kBases;   // classes along y and z
+    static constexpr int kPerX = (kBrick + 1 + kBasesX - 1) / kBasesX;
+    static constexpr int kClasses = kPer * kPer * kPerX;
+    // Region, with planes padded so that 4 planes x 8 cells of a flush meet 32 banks
+    static constexpr int RG = kBrick + W, PS = (RG * RG - 4 + 15) / 16 * 16 + 4, RG3 = PS * RG;
+    static constexpr int T = XS == 8 ? 4 : 8;                         // 16-row tiles of (y, x)
     static constexpr int kSlots = (kMmaChunk + kClasses * 15 + 15) / 16 * 16;   // most slots of an item
     // A group's record: x, y, z coordinate words [16], then weights [pair 8][CH][hi, lo],
     // each word the fp16 parts of the pair's two points.
     static constexpr int kRecWords = 16 * (3 + CH);
     static constexpr size_t kSortSmem = sizeof(int) * (size_t)(kSlots / 16) * kRecWords;
+    // Staging of one warp: windows of 4 groups along x (2 at 8 cells) and y, of 2 along z,
+    // each axis hi | lo of 8 pairs per cell.  Strides are 8 mod 32 words, so that the four
+    // groups a warp stores together meet different banks.
+    static constexpr int kXG = XS == 8 ? 2 : 4;
+    static constexpr int kXWords = 16 * XS + 8, kYWords = 136, kZWords = 136;
+    static constexpr int kWarpWords = kXG * kXWords + 4 * kYWords + 2 * kZWords;
     // staging | record buffers [warp][2][4 groups] | region
     static constexpr size_t kSmem =
         sizeof(int) * ((size_t)kMmaWarps * (kWarpWords + 8 * kRecWords) + (size_t)CH * RG3);
@@ -97,12 +104,12 @@ __device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Window taps of two points along one axis, scaled by kTapScale, in the 8 slots of their
+// Window taps of two points along one axis, scaled by kTapScale, in the S slots of their
 // class's cells: slot off + l holds tap l (off < BASES may differ between the points),
 // the others 0.  c: the points' coordinate words.  hi[s], lo[s]: the two points' values
 // as fp16 pairs.  Taps l and W - 1 - l are one polynomial at z and -z: even and odd parts
 // are shared.
-template <int W, int BASES>
+template <int W, int BASES, int S>
 __device__ __forceinline__ void slot_taps(const float2* __restrict__ poly, uint2 c, uint32_t* hi, uint32_t* lo) {
     const int off0 = (int)(c.x >> (32 - kOffBits)), off1 = (int)(c.y >> (32 - kOffBits));
     // z = 2u - 1 from the 28-bit offset u: (u - 1/2) as a signed 32-bit fraction
@@ -112,25 +119,32 @@ __device__ __forceinline__ void slot_taps(const float2* __restrict__ poly, uint2
     const float2 z2 = __fmul2_rn(z, z);
 #pragma unroll
     for (int l = 0; l < (W + 1) / 2; ++l) {
-        const float2* c = poly + l * (kKbDeg + 1);
-        const float2 ev = __ffma2_rn(__ffma2_rn(__ffma2_rn(c[6], z2, c[4]), z2, c[2]), z2, c[0]);
-        const float2 od = __ffma2_rn(__ffma2_rn(__ffma2_rn(c[7], z2, c[5]), z2, c[3]), z2, c[1]);
+        const float2* p = poly + l * (kKbDeg + 1);
+        const float2 ev = __ffma2_rn(__ffma2_rn(__ffma2_rn(p[6], z2, p[4]), z2, p[2]), z2, p[0]);
+        const float2 od = __ffma2_rn(__ffma2_rn(__ffma2_rn(p[7], z2, p[5]), z2, p[3]), z2, p[1]);
         split2(__ffma2_rn(od, z, ev), hi[l], lo[l]);
         if (W - 1 - l != l) split2(__ffma2_rn(od, nz, ev), hi[W - 1 - l], lo[W - 1 - l]);
     }
 #pragma unroll
-    for (int s = W; s < 8; ++s) { hi[s] = 0u; lo[s] = 0u; }
+    for (int s = W; s < S; ++s) { hi[s] = 0u; lo[s] = 0u; }
+    // shift by `n` slots in each point's half where its condition holds; `top`: last tap's slot
+    auto shift = [&](bool c0, bool c1, int n, int top) {
+        const uint32_t sel = (c0 ? 0x0054u : 0x0010u) | (c1 ? 0x7600u : 0x3200u);
 #pragma unroll
-    for (int st = 1; st < BASES; ++st) {            // shift by one slot where off >= st
-        const uint32_t sel = (off0 >= st ? 0x0054u : 0x0010u) | (off1 >= st ? 0x7600u : 0x3200u);
-#pragma unroll
-        for (int s = 7; s > 0; --s) {
-            if (s > W - 1 + st) continue;
-            hi[s] = __byte_perm(hi[s], hi[s - 1], sel);
-            lo[s] = __byte_perm(lo[s], lo[s - 1], sel);
+        for (int s = S - 1; s >= 0; --s) {
+            if (s > top) continue;
+            hi[s] = __byte_perm(hi[s], s >= n ? hi[s - n] : 0u, sel);
+            lo[s] = __byte_perm(lo[s], s >= n ? lo[s - n] : 0u, sel);
         }
-        hi[0] = __byte_perm(hi[0], 0u, sel);
-        lo[0] = __byte_perm(lo[0], 0u, sel);
+    };
+    if (BASES <= 3) {
+#pragma unroll
+        for (int st = 1; st < BASES; ++st) shift(off0 >= st, off1 >= st, 1, W - 1 + st);
+    } else {                                       // 0..8, by its bits (8 alone has bit 3)
+        shift(off0 & 1, off1 & 1, 1, W);
+        shift(off0 & 2, off1 & 2, 2, W + 2);
+        shift(off0 & 4, off1 & 4, 4, W + 6);
+        shift(off0 & 8, off1 & 8, 8, W + 7);
     }
 }
 
@@ -140,7 +154,7 @@ __device__ __forceinline__ void slot_taps(const float2* __restrict__ poly, uint2
 template <int W, int CH>
 __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a) {
     using C = MmaCfg<W, CH>;
-    constexpr int BASES = C::kBases, PER = C::kPer, RW = C::kRecWords, PT = kMmaChunk / kSortThreads;
+    constexpr int BASES = C::kBases, BX = C::kBasesX, RW = C::kRecWords, PT = kMmaChunk / kSortThreads;
     constexpr int kWarps = kSortThreads / 32;
     extern __shared__ __align__(16) uint32_t s_rec[];
     __shared__ int s_hist[32], s_off[32], s_total, s_item, s_base;
@@ -186,11 +200,11 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
             if (u * kSortThreads + tid >= wk.z) continue;
             const uint32_t r[3] = {pt[u].x >> 28, pt[u].y >> 28, pt[u].z >> 28};
             in = in && r[0] <= (uint32_t)kBrick && r[1] <= (uint32_t)kBrick && r[2] <= (uint32_t)kBrick;
-            const uint32_t k[3] = {min(r[0], (uint32_t)kBrick) / BASES, min(r[1], (uint32_t)kBrick) / BASES,
+            const uint32_t k[3] = {min(r[0], (uint32_t)kBrick) / BX, min(r[1], (uint32_t)kBrick) / BASES,
                                    min(r[2], (uint32_t)kBrick) / BASES};
-            cr[u] = (int)((k[2] * PER + k[1]) * PER + k[0]);
+            cr[u] = (int)((k[2] * C::kPer + k[1]) * C::kPerX + k[0]);
             // the first tap's slot within the class's cells takes the place of r
-            pt[u].x -= (k[0] * BASES) << 28;
+            pt[u].x -= (k[0] * BX) << 28;
             pt[u].y -= (k[1] * BASES) << 28;
             pt[u].z -= (k[2] * BASES) << 28;
             cr[u] |= atomicAdd(&s_hist[cr[u]], 1) << 8;
@@ -294,21 +308,39 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
 // ---------------------------------------------------------------------------
 // A class's sums into the brick's region (one rounding to the region's unit per cell).
 template <int W, int CH>
-__device__ __forceinline__ void flush_class(const float (&D)[4][CH][4], int cls, int* lev1, int row, int c) {
+__device__ __forceinline__ void flush_class(const float (&D)[MmaCfg<W, CH>::T][CH][4], int cls, int* lev1, int row, int c) {
     using C = MmaCfg<W, CH>;
-    constexpr int RG = C::RG, RG3 = C::RG3, BASES = C::kBases, PER = C::kPer;
-    const int z0 = cls / (PER * PER) * BASES, y0 = (cls / PER) % PER * BASES, x0 = cls % PER * BASES;
-    int* dst = lev1 + ((z0 + 2 * c) * RG + y0) * RG + x0 + row;
+    constexpr int RG = C::RG, PS = C::PS, RG3 = C::RG3, PER = C::kPer, PERX = C::kPerX;
+    const int z0 = cls / (PER * PERX) * C::kBases, y0 = cls / PERX % PER * C::kBases, x0 = cls % PERX * C::kBasesX;
+    int* dst = lev1 + (z0 + 2 * c) * PS + y0 * RG + x0 + row;
+    if (C::XS == 8) {                              // rows: 8 x of y = 2t, 8 x of y = 2t + 1
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
+        for (int t = 0; t < C::T; ++t)
 #pragma unroll
-        for (int ch = 0; ch < CH; ++ch) {
-            int* d = dst + ch * RG3 + 2 * t * RG;
-            atomicAdd(d, __float2int_rn(D[t][ch][0]));
-            atomicAdd(d + RG * RG, __float2int_rn(D[t][ch][1]));
-            atomicAdd(d + RG, __float2int_rn(D[t][ch][2]));
-            atomicAdd(d + RG * RG + RG, __float2int_rn(D[t][ch][3]));
+            for (int ch = 0; ch < CH; ++ch) {
+                int* d = dst + ch * RG3 + 2 * t * RG;
+                atomicAdd(d, __float2int_rn(D[t][ch][0]));
+                atomicAdd(d + PS, __float2int_rn(D[t][ch][1]));
+                atomicAdd(d + RG, __float2int_rn(D[t][ch][2]));
+                atomicAdd(d + PS + RG, __float2int_rn(D[t][ch][3]));
+            }
+    } else {                                       // rows: 16 x of y = t
+        // a class with fewer than kBases first taps, and x cell 15, reach past the region
+        // with sums that are zero
+        const bool z1 = z0 + 2 * c + 1 < RG, x1 = row < RG - 8;
+#pragma unroll
+        for (int t = 0; t < C::T; ++t) {
+            if (y0 + t >= RG) break;
+#pragma unroll
+            for (int ch = 0; ch < CH; ++ch) {
+                int* d = dst + ch * RG3 + t * RG;
+                atomicAdd(d, __float2int_rn(D[t][ch][0]));
+                if (z1) atomicAdd(d + PS, __float2int_rn(D[t][ch][1]));
+                if (x1) atomicAdd(d + 8, __float2int_rn(D[t][ch][2]));
+                if (x1 && z1) atomicAdd(d + PS + 8, __float2int_rn(D[t][ch][3]));
+            }
         }
+    }
 }
 
 // float -> double by its bits (the conversion instruction runs at the FP64 rate); v is a
@@ -331,7 +363,8 @@ template <int W, int CH>
 __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float2* s_poly, const int4 wk, int* lev1,
                                                 uint32_t* wbuf) {
     using C = MmaCfg<W, CH>;
-    constexpr int RG = C::RG, RG3 = C::RG3, BASES = C::kBases, RW = C::kRecWords;
+    constexpr int RG = C::RG, RG3 = C::RG3, BASES = C::kBases, RW = C::kRecWords, XS = C::XS, T = C::T;
+    constexpr int XO = XS * 8;                     // hi -> lo distance of the x windows
     __shared__ uint8_t s_cls[C::kSlots / 16];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_groups = wk.z;
@@ -339,9 +372,10 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
     // every warp takes a run of consecutive groups, in its own buffers
     const int per = (n_groups + kMmaWarps - 1) / kMmaWarps;
     const int ga = min(n_groups, warp * per), gb = min(n_groups, ga + per);
-    uint32_t* const xz = wbuf;
-    uint32_t* const ys = xz + 2 * kXZWords;
-    uint32_t* const in = wbuf + kWarpWords;
+    uint32_t* const xs = wbuf;
+    uint32_t* const ys = xs + C::kXG * C::kXWords;
+    uint32_t* const zs = ys + 4 * C::kYWords;
+    uint32_t* const in = wbuf + C::kWarpWords;
     const uint32_t* const rec = a.rec + (size_t)wk.y * RW;
     copy_async(in, rec + (size_t)ga * RW, min(4, gb - ga) * (RW / 4), lane);
     __syncthreads();
@@ -352,9 +386,9 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
         const int cls = s_cls[g];
         int ge = g + 1;                            // end of this class's run
         while (ge < gb && ge < g + kRunGroups && s_cls[ge] == cls) ++ge;
-        float D[4][CH][4];
+        float D[T][CH][4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
+        for (int t = 0; t < T; ++t)
 #pragma unroll
             for (int ch = 0; ch < CH; ++ch)
 #pragma unroll
@@ -365,7 +399,6 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
             const uint32_t* const cur = in + ((r >> 2) & 1) * 4 * RW;
             if (gi == 0) {                         // stage the windows of the next groups
                 __syncwarp();
-                uint32_t hi[8], lo[8];
                 if ((r & 2) == 0) {
                     copy_async(in + (((r >> 2) & 1) ^ 1) * 4 * RW, rec + (size_t)(g + 4) * RW,
                                max(0, min(4, gb - g - 4)) * (RW / 4), lane);
@@ -373,25 +406,39 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
                     __syncwarp();
                     // y windows of 4 groups, a pair of points per lane: [pair][slot], halves of
                     // four slots swapped for pairs 4-7 (16-byte accesses)
+                    const int pr = lane & 7, sw = pr >> 2;
                     if (lane < 8 * (gb - g)) {
-                        const int pr = lane & 7, sw = pr >> 2;
-                        slot_taps<W, BASES>(
+                        uint32_t hi[8], lo[8];
+                        slot_taps<W, BASES, 8>(
                             s_poly, *reinterpret_cast<const uint2*>(cur + (lane >> 3) * RW + 16 + 2 * pr), hi, lo);
-                        uint4* y = reinterpret_cast<uint4*>(ys + (lane >> 3) * kYWords + pr * 8);
+                        uint4* y = reinterpret_cast<uint4*>(ys + (lane >> 3) * C::kYWords + pr * 8);
                         y[sw] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                         y[sw ^ 1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
                         y[16 + sw] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                         y[16 + (sw ^ 1)] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
+                        if (XS == 16) {            // x windows of 4 groups, layout as below
+                            uint32_t xh[16], xl[16];
+                            slot_taps<W, C::kBasesX, 16>(
+                                s_poly, *reinterpret_cast<const uint2*>(cur + (lane >> 3) * RW + 2 * pr), xh, xl);
+                            uint32_t* Gs = xs + (lane >> 3) * C::kXWords;
+#pragma unroll
+                            for (int s = 0; s < 16; ++s) {
+                                Gs[s * 8 + (pr ^ (s & 4))] = xh[s];
+                                Gs[XO + s * 8 + (pr ^ (s & 4))] = xl[s];
+                            }
+                        }
                     }
                 }
-                // x (lanes 0-15) and z (16-31) windows of 2 groups: [slot][pair], the pair's bit
-                // 2 flipped for slots 4-7 (a fragment read then meets 32 different banks)
+                // x (lanes 0-15, unless staged above) and z (16-31) windows of 2 groups:
+                // [slot][pair], the pair's bit 2 flipped for slots 4-7 of every 8 (a fragment
+                // read then meets 32 different banks)
                 const int l16 = lane & 15, ax = lane >> 4, pr = l16 & 7;
-                if (l16 < 8 * (gb - g)) {
-                    slot_taps<W, BASES>(s_poly, *reinterpret_cast<const uint2*>(
-                                                    cur + ((r & 2) + (l16 >> 3)) * RW + 32 * ax + 2 * pr),
-                                        hi, lo);
-                    uint32_t* Gs = xz + (l16 >> 3) * kXZWords + ax * 128;
+                if (l16 < 8 * (gb - g) && (XS == 8 || ax == 1)) {
+                    uint32_t hi[8], lo[8];
+                    slot_taps<W, BASES, 8>(s_poly, *reinterpret_cast<const uint2*>(
+                                                       cur + ((r & 2) + (l16 >> 3)) * RW + 32 * ax + 2 * pr),
+                                           hi, lo);
+                    uint32_t* Gs = ax ? zs + (l16 >> 3) * C::kZWords : xs + (l16 >> 3) * C::kXWords;
 #pragma unroll
                     for (int s = 0; s < 8; ++s) {
                         Gs[s * 8 + (pr ^ (s & 4))] = hi[s];
@@ -400,12 +447,12 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
                 }
                 __syncwarp();
             }
-            // ---- contract ----
-            const uint32_t* G = xz + gi * kXZWords + row * 8 + (c ^ sx);      // pair c
-            const uint32_t* G4 = xz + gi * kXZWords + row * 8 + ((c + 4) ^ sx);
+            // ---- contract: pairs c and c + 4 of the group are this lane's ----
+            const int f0 = row * 8 + (c ^ sx), f1 = row * 8 + ((c + 4) ^ sx);
             // weighted z operand: B[k][n = z], k = points (2c, 2c + 1) and (2c + 8, 2c + 9)
             uint32_t bh[CH][2], bl[CH][2];
-            const uint32_t zh0 = G[128], zh1 = G4[128], zl0 = G[192], zl1 = G4[192];
+            const uint32_t* Z = zs + gi * C::kZWords;
+            const uint32_t zh0 = Z[f0], zh1 = Z[f1], zl0 = Z[64 + f0], zl1 = Z[64 + f1];
             const uint2* w0 = reinterpret_cast<const uint2*>(cur + (r & 3) * RW + 48) + c * CH;
 #pragma unroll
             for (int ch = 0; ch < CH; ++ch) {
@@ -413,8 +460,16 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
                 mul_split(wa.x, wa.y, zh0, zl0, bh[ch][0], bl[ch][0]);
                 mul_split(wb.x, wb.y, zh1, zl1, bh[ch][1], bl[ch][1]);
             }
-            const uint32_t xh0 = G[0], xh1 = G4[0], xl0 = G[64], xl1 = G4[64];
-            const uint4* y0 = reinterpret_cast<const uint4*>(ys + (r & 3) * kYWords + c * 8);
+            const uint32_t* X = xs + (r & (C::kXG - 1)) * C::kXWords;
+            uint32_t xh[2][2], xl[2][2];           // [x = row, row + 8][pair]
+#pragma unroll
+            for (int q = 0; q < XS / 8; ++q) {
+                xh[q][0] = X[64 * q + f0];
+                xh[q][1] = X[64 * q + f1];
+                xl[q][0] = X[XO + 64 * q + f0];
+                xl[q][1] = X[XO + 64 * q + f1];
+            }
+            const uint4* y0 = reinterpret_cast<const uint4*>(ys + (r & 3) * C::kYWords + c * 8);
             const uint4* y1 = y0 + 8;
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
@@ -422,13 +477,15 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
                 const uint32_t yh0[4] = {yh0v.x, yh0v.y, yh0v.z, yh0v.w}, yl0[4] = {yl0v.x, yl0v.y, yl0v.z, yl0v.w};
                 const uint32_t yh1[4] = {yh1v.x, yh1v.y, yh1v.z, yh1v.w}, yl1[4] = {yl1v.x, yl1v.y, yl1v.z, yl1v.w};
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int t = half * 2 + q;
+                for (int q = 0; q < T / 2; ++q) {
+                    // operand rows: (x, y = 2t), (x, 2t + 1) at 8 x cells; (x, t), (x + 8, t) at 16
+                    const int t = half * (T / 2) + q;
+                    const int ya = XS == 8 ? 2 * q : q, yb = XS == 8 ? 2 * q + 1 : q, xb = XS == 8 ? 0 : 1;
                     uint32_t ah[4], al[4];
-                    mul_split(xh0, xl0, yh0[2 * q], yl0[2 * q], ah[0], al[0]);
-                    mul_split(xh0, xl0, yh0[2 * q + 1], yl0[2 * q + 1], ah[1], al[1]);
-                    mul_split(xh1, xl1, yh1[2 * q], yl1[2 * q], ah[2], al[2]);
-                    mul_split(xh1, xl1, yh1[2 * q + 1], yl1[2 * q + 1], ah[3], al[3]);
+                    mul_split(xh[0][0], xl[0][0], yh0[ya], yl0[ya], ah[0], al[0]);
+                    mul_split(xh[xb][0], xl[xb][0], yh0[yb], yl0[yb], ah[1], al[1]);
+                    mul_split(xh[0][1], xl[0][1], yh1[ya], yl1[ya], ah[2], al[2]);
+                    mul_split(xh[xb][1], xl[xb][1], yh1[yb], yl1[yb], ah[3], al[3]);
 #pragma unroll
                     for (int ch = 0; ch < CH; ++ch) mma16816(D[t][ch], al, bh[ch][0], bh[ch][1]);
 #pragma unroll
@@ -462,7 +519,7 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
             if (++gz == a.G) gz = 0;
 #pragma unroll
             for (int ch = 0; ch < CH; ++ch) {
-                int* p = &lev1[ch * RG3 + rz * RG * RG + tid];
+                int* p = &lev1[ch * RG3 + rz * C::PS + tid];
                 const int v = *p;
                 if (v == 0) continue;
                 *p = 0;
@@ -488,8 +545,8 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs 
     extern __shared__ __align__(16) int sm_mma[];
     __shared__ float2 s_poly[(W + 1) / 2 * (kKbDeg + 1)];
     __shared__ int s_item;
-    int* const lev1 = sm_mma + kMmaWarps * (kWarpWords + 8 * C::kRecWords);
-    uint32_t* const wbuf = reinterpret_cast<uint32_t*>(sm_mma) + (threadIdx.x >> 5) * (kWarpWords + 8 * C::kRecWords);
+    int* const lev1 = sm_mma + kMmaWarps * (C::kWarpWords + 8 * C::kRecWords);
+    uint32_t* const wbuf = reinterpret_cast<uint32_t*>(sm_mma) + (threadIdx.x >> 5) * (C::kWarpWords + 8 * C::kRecWords);
     load_poly<W>(a.poly, s_poly);
     for (int i = threadIdx.x; i < CH * C::RG3; i += kMmaThreads) lev1[i] = 0;
     const int n_work = a.counters[0];
@@ -513,8 +570,8 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma_batch(const Sprea
     extern __shared__ __align__(16) int sm_mma[];
     __shared__ float2 s_poly[(W + 1) / 2 * (kKbDeg + 1)];
     __shared__ int s_item, s_prob;
-    int* const lev1 = sm_mma + kMmaWarps * (kWarpWords + 8 * C::kRecWords);
-    uint32_t* const wbuf = reinterpret_cast<uint32_t*>(sm_mma) + (threadIdx.x >> 5) * (kWarpWords + 8 * C::kRecWords);
+    int* const lev1 = sm_mma + kMmaWarps * (C::kWarpWords + 8 * C::kRecWords);
+    uint32_t* const wbuf = reinterpret_cast<uint32_t*>(sm_mma) + (threadIdx.x >> 5) * (C::kWarpWords + 8 * C::kRecWords);
     load_poly<W>(poly, s_poly);
     for (int i = threadIdx.x; i < CH * C::RG3; i += kMmaThreads) lev1[i] = 0;
     const int total = item_off[n];
@@ -554,8 +611,11 @@ static cudaError_t spread_mma_batch_w(int n, const SpreadArgs* desc, const int* 
     return cudaGetLastError();
 }
 
-cudaError_t launch_spread_mma_batch(int n, bool kc, const SpreadArgs* desc, const int* item_off, int* queue,
+cudaError_t launch_spread_mma_batch(int n, bool kc, int W, const SpreadArgs* desc, const int* item_off, int* queue,
                                     const KbPoly& poly, int num_sms, cudaStream_t s) {
+    if (W == 7)
+        return kc ? spread_mma_batch_w<7, 1>(n, desc, item_off, queue, poly, num_sms, s)
+                  : spread_mma_batch_w<7, 2>(n, desc, item_off, queue, poly, num_sms, s);
     return kc ? spread_mma_batch_w<6, 1>(n, desc, item_off, queue, poly, num_sms, s)
               : spread_mma_batch_w<6, 2>(n, desc, item_off, queue, poly, num_sms, s);
 }
@@ -585,7 +645,8 @@ static cudaError_t mma_sort_w(Plan& P, const SpreadArgs& a) {
 }
 
 cudaError_t launch_mma_sort(Plan& P, const SpreadArgs& a, int ch) {
-    if (P.p.W != 6) return cudaErrorInvalidValue;
+    if (P.p.W == 7)
+        return ch == 1 ? mma_sort_w<7, 1>(P, a) : ch == 2 ? mma_sort_w<7, 2>(P, a) : cudaErrorInvalidValue;
     switch (ch) {
         case 1: return mma_sort_w<6, 1>(P, a);
         case 2: return mma_sort_w<6, 2>(P, a);
@@ -595,7 +656,8 @@ cudaError_t launch_mma_sort(Plan& P, const SpreadArgs& a, int ch) {
 }
 
 cudaError_t launch_spread_mma(Plan& P, const SpreadArgs& a, int ch) {
-    if (P.p.W != 6) return cudaErrorInvalidValue;
+    if (P.p.W == 7)
+        return ch == 1 ? spread_mma_w<7, 1>(P, a) : ch == 2 ? spread_mma_w<7, 2>(P, a) : cudaErrorInvalidValue;
     switch (ch) {
         case 1: return spread_mma_w<6, 1>(P, a);
         case 2: return spread_mma_w<6, 2>(P, a);

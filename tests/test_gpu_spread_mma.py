@@ -1,4 +1,4 @@
-"""The tensor-core spreading (dense bricks, W = 6) against the FP64 gridding oracle with the
+"""The tensor-core spreading (dense bricks, W = 6 and 7) against the FP64 gridding oracle with the
 same Kaiser-Bessel window (eq. kernel, eq. backprojection), which leaves the arithmetic's
 own error: the sizes run from just above the rule's threshold, where most classes of a
 brick hold less than one group of points, to bricks of several work items.
@@ -22,21 +22,22 @@ def rel(a, b):
     return float(np.linalg.norm(a - b) / np.linalg.norm(b))
 
 
-@pytest.mark.parametrize("N,M,cfg,fused", [(16, 118, "C2", False), (16, 1361, "C5", False), (16, 6001, "C3", False),
-                                           (32, 2900, "C5", False), (16, 541, "C3", True), (16, 2003, "C5", True),
-                                           (32, 801, "C2", True)])
-def test_tensor_core_spreading_matches_oracle(N, M, cfg, fused):
+@pytest.mark.parametrize("N,M,cfg,fused,W", [
+    (16, 118, "C2", False, 6), (16, 1361, "C5", False, 6), (16, 6001, "C3", False, 6), (32, 2900, "C5", False, 6),
+    (16, 541, "C3", True, 6), (16, 2003, "C5", True, 6), (32, 801, "C2", True, 6),
+    (16, 1521, "C5", False, 7), (16, 6001, "C3", False, 7), (32, 1001, "C2", False, 7)])
+def test_tensor_core_spreading_matches_oracle(N, M, cfg, fused, W):
     import __graft_entry__ as g
     g.build()
     import paper_1307_5824_gb300 as F
     inp = synth.config_inputs(cfg, M=M, N=N)
     K = O.disc(N)
-    kw = dict(W=6, window="kb", beta=GR.kb_beta(6))
+    kw = dict(W=W, window="kb", beta=GR.kb_beta(W))
     Ker = GR.kernel_gridded(inp["R"], inp["groups"], inp["group_id"], K, N, **kw).real
     rhs_o = GR.backproject_gridded(inp["images"], inp["shifts"], inp["R"], inp["groups"], inp["group_id"], K,
                                    sigma=4 if fused else 2, **kw)
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
-    rec = F.Reconstructor(N, M, groups=inp["groups"], W=6, lam=1e-3, fused=fused)
+    rec = F.Reconstructor(N, M, groups=inp["groups"], W=W, lam=1e-3, fused=fused)
     R, gid = dev(inp["R"].reshape(M, 9)), dev(inp["group_id"])
     ker = torch.empty(rec.half_shape(), device="cuda")
     rhs = torch.empty((N, N, N), device="cuda")
@@ -49,6 +50,6 @@ def test_tensor_core_spreading_matches_oracle(N, M, cfg, fused):
     assert rec.lambda_eff() > 0.0                    # waits for the stream and the device's error flag
     e_k = rel(ker.cpu().numpy()[1:, 1:, :N], Ker[1:, 1:, N:])
     e_r = rel(rhs.cpu().numpy(), rhs_o)
-    print(f"N={N} M={M} {cfg} fused={fused}: Ker {e_k:.2e} A*b {e_r:.2e}")
+    print(f"N={N} M={M} {cfg} W={W} fused={fused}: Ker {e_k:.2e} A*b {e_r:.2e}")
     assert e_k <= 3e-6 and e_r <= 3e-6
     rec.close()
