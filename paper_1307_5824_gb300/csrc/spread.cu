@@ -23,6 +23,7 @@
 
 #include <algorithm>
 
+#include "dw.cuh"
 #include "firm_internal.h"
 #include "spread.cuh"
 
@@ -1239,9 +1240,10 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
     constexpr int BZ = kBrick;
     constexpr int RG = kBrick + W;
     constexpr int RG3 = RG * RG * (BZ + W);
-    extern __shared__ float s_f[];
-    float* s_re = s_f;
-    float* s_im = s_f + RG3;
+    // (re, im) together: one 8-byte load and one packed FMA per tap.  The round-robin order
+    // of the bank classes (base mod 32) keeps the 16 lanes of each half of such a load on
+    // distinct pairs of banks.
+    extern __shared__ float2 s_g[];
     __shared__ int s_item;
     __shared__ double s_red[2][kSpreadWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1266,12 +1268,11 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
             gy -= (gy >= a.G) ? a.G : 0;
             gz += (gz < 0) ? a.G : 0;
             gz -= (gz >= a.G) ? a.G : 0;
-            const float2 v = __ldg(&a.ghat[((size_t)gz * a.G + gy) * a.G + gx]);
-            s_re[i] = v.x;
-            s_im[i] = v.y;
+            s_g[i] = __ldg(&a.ghat[((size_t)gz * a.G + gy) * a.G + gx]);
         }
         __syncthreads();
-        double acc_r = 0.0, acc_b = 0.0;
+        // sums of a thread's points in double-words: 48 bits, at the FP32 rate
+        float2 acc_r = make_float2(0.0f, 0.0f), acc_b = make_float2(0.0f, 0.0f);
         for (int i = threadIdx.x; i < wk.z; i += blockDim.x) {
             const uint32_t pos = (uint32_t)wk.y + i;
             const uint32_t id = __ldg(&a.payload[pos]);
@@ -1287,44 +1288,44 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
             window_taps<W>(a.poly, p.f(0), wx);
             window_taps<W>(a.poly, p.f(1), wy);
             window_taps<W>(a.poly, p.f(2), wz);
-            float fr = 0.0f, fi = 0.0f;
+            float2 f = make_float2(0.0f, 0.0f);
 #pragma unroll
             for (int dz = 0; dz < W; ++dz) {
 #pragma unroll
                 for (int dy = 0; dy < W; ++dy) {
-                    const int row = base + (dz * RG + dy) * RG;
-                    float rr = 0.0f, ri = 0.0f;
+                    const float2* row = s_g + base + (dz * RG + dy) * RG;
+                    float2 rr = make_float2(0.0f, 0.0f);
 #pragma unroll
-                    for (int dx = 0; dx < W; ++dx) {
-                        rr = fmaf(wx[dx], s_re[row + dx], rr);
-                        ri = fmaf(wx[dx], s_im[row + dx], ri);
-                    }
+                    for (int dx = 0; dx < W; ++dx) rr = __ffma2_rn(make_float2(wx[dx], wx[dx]), row[dx], rr);
                     const float wyz = wz[dz] * wy[dy];
-                    fr = fmaf(wyz, rr, fr);
-                    fi = fmaf(wyz, ri, fi);
+                    f = __ffma2_rn(make_float2(wyz, wyz), rr, f);
                 }
             }
             const int g = a.gid ? min(max(__ldg(&a.gid[m]), 0), a.n_ctf - 1) : 0;
             const float h = __ldg(&a.h1[(size_t)g * a.nH + t]);
             if (!RESID) {
-                a.out[(size_t)m * a.nH + t] = make_float2(h * fr, h * fi);
+                a.out[(size_t)m * a.nH + t] = make_float2(h * f.x, h * f.y);
             } else {
                 const float2 bv = __ldg(&a.samples_b[wk.y + __ldg(&a.perm[pos])]);
-                const double dr = (double)bv.x - (double)h * fr, di = (double)bv.y - (double)h * fi;
-                const double c = t == 0 ? 1.0 : 2.0;
-                acc_r += c * (dr * dr + di * di);
-                acc_b += c * ((double)bv.x * bv.x + (double)bv.y * bv.y);
+                const float2 one = make_float2(h, 0.0f);
+                const float2 dr = dw_sub_mul(make_float2(bv.x, 0.0f), one, f.x);
+                const float2 di = dw_sub_mul(make_float2(bv.y, 0.0f), one, f.y);
+                // c = 2 off the origin: the conjugate half; the origin counts once
+                float2 pr = dw_acc_sq(make_float2(0.0f, 0.0f), dr), pb = make_float2(0.0f, 0.0f);
+                pr = dw_acc_sq(pr, di);
+                pb = dw_acc_prod(pb, bv.x, bv.x);
+                pb = dw_acc_prod(pb, bv.y, bv.y);
+                const float c = t == 0 ? 1.0f : 2.0f;
+                acc_r = dw_add(acc_r, c * pr.x, c * pr.y);
+                acc_b = dw_add(acc_b, c * pb.x, c * pb.y);
             }
         }
         if (RESID) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                acc_r += __shfl_xor_sync(0xffffffffu, acc_r, o);
-                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, o);
-            }
+            acc_r = dw_warp_sum(acc_r);
+            acc_b = dw_warp_sum(acc_b);
             if (lane == 0) {
-                s_red[0][warp] = acc_r;
-                s_red[1][warp] = acc_b;
+                s_red[0][warp] = dw_to_double(acc_r);
+                s_red[1][warp] = dw_to_double(acc_b);
             }
             __syncthreads();
             if (threadIdx.x == 0) {
