@@ -33,35 +33,41 @@ __device__ __forceinline__ int freq_bin(float q1, float q2, float q3, float half
 }
 
 // second moment of the viewing directions d = third row of R_m (sum of d d^T)
-__global__ void __launch_bounds__(1024) k_view_moment(const double* __restrict__ R, int M, double* __restrict__ out9) {
-    __shared__ double s[32][9];
-    double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
+constexpr int kMomentBlocks = 64, kMomentThreads = 256;
+__global__ void __launch_bounds__(kMomentThreads) k_view_moment(const double* __restrict__ R, int M,
+                                                               double* __restrict__ part) {
+    __shared__ double s[kMomentThreads / 32][6];
+    double acc[6] = {0, 0, 0, 0, 0, 0};            // xx, xy, xz, yy, yz, zz
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
         const double* d = R + 9 * (size_t)m + 6;
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) acc[3 * i + j] += d[i] * d[j];
+        const double x = d[0], y = d[1], z = d[2];
+        acc[0] += x * x; acc[1] += x * y; acc[2] += x * z;
+        acc[3] += y * y; acc[4] += y * z; acc[5] += z * z;
     }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int k = 0; k < 9; ++k) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
         double v = acc[k];
+#pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if (lane == 0) s[wid][k] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 9) {
+    if (threadIdx.x < 6) {
         double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += s[w][threadIdx.x];
-        out9[threadIdx.x] = v;
+        for (int w = 0; w < kMomentThreads / 32; ++w) v += s[w][threadIdx.x];
+        part[6 * blockIdx.x + threadIdx.x] = v;
     }
 }
 
 // h^2-weighted histogram of the half-disc samples (the mirrored half falls in the same
-// bin).  A thread owns one image and walks a range of samples t (blockIdx.y picks the
+// bin).  Four threads own one image and walk a range of samples t (blockIdx.y picks the
 // range): |xi| = |k| fixes the shell and the cone only needs |k1 <u, a> + k2 <v, a>| /
 // |k| (u, v the slice axes, a the viewing axis), so the block first tabulates, per t of
 // its range, the shell and k / |k|, and every point is then two FMAs, a cone index and
 // one shared-memory atomic into the block's histogram.
-constexpr int kFeatThreads = 256;
+constexpr int kFeatImgs = 256;         // images per block
+constexpr int kFeatThreads = 1024;     // four threads per image: the loop is bound by the atomics' latency
 constexpr int kFeatT = 1024;          // samples t per block (the table: 12 B each)
 __global__ void __launch_bounds__(kFeatThreads) k_pc_features(const ImgGeom* __restrict__ geom,
                                                               const int32_t* __restrict__ htab,
@@ -84,7 +90,7 @@ __global__ void __launch_bounds__(kFeatThreads) k_pc_features(const ImgGeom* __r
         s_s[t - t0] = min(kShells - 1, (int)floorf((float)kShells * rk / halfN));
     }
     __syncthreads();
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m = blockIdx.x * kFeatImgs + threadIdx.x % kFeatImgs, q = threadIdx.x / kFeatImgs;
     if (m < M) {
         const ImgGeom g = geom[m];
         constexpr float unit = 1.0f / (float)(1ll << kGeomBits);
@@ -92,7 +98,7 @@ __global__ void __launch_bounds__(kFeatThreads) k_pc_features(const ImgGeom* __r
         const float ua = f(g.uh[0], g.ul[0]) * a1 + f(g.uh[1], g.ul[1]) * a2 + f(g.uh[2], g.ul[2]) * a3;
         const float va = f(g.vh[0], g.vl[0]) * a1 + f(g.vh[1], g.vl[1]) * a2 + f(g.vh[2], g.vl[2]) * a3;
         const float* h2g = h2 + (size_t)min(max(gid[m], 0), n_ctf - 1) * nH;
-        for (int t = t0; t < t1; ++t) {
+        for (int t = t0 + q; t < t1; t += kFeatThreads / kFeatImgs) {
             const float2 kr = s_k[t - t0];
             const float c = fabsf(fmaf(kr.x, ua, kr.y * va));
             const int cb = min(kCones - 1, (int)((float)kCones * c));
@@ -150,33 +156,44 @@ __global__ void __launch_bounds__(256) k_pc_from_table(const float* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// Principal axis: Jacobi eigenvalue iterations on the symmetric 3x3 moment, on the
-// device (one thread), so that firm_kernel needs no host round trip.
+// Principal axis of the symmetric 3x3 moment, on the device (one thread), so that
+// firm_kernel needs no host round trip: Jacobi eigenvalue iterations in FP32, then the
+// eigenvector corrected in FP64 by first-order perturbation steps, each of which takes its
+// error e to about 1e-7 e + e^2 / gap.  (Jacobi in FP64 throughout took 45 us: this part's
+// FP64 sine, cosine and division are long chains of slow operations.)
 // ---------------------------------------------------------------------------
-__device__ static void principal_axis(const double* S, float* a) {
-    double A[3][3], V[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
+__device__ static void principal_axis(const double* S, float* a) {     // S: xx, xy, xz, yy, yz, zz
+    const double B[3][3] = {{S[0], S[1], S[2]}, {S[1], S[3], S[4]}, {S[2], S[4], S[5]}};
+    const float tr = (float)(S[0] + S[3] + S[5]);
+    const double unit = tr > 0.0f ? (double)(1.0f / tr) : 1.0;
+    float A[3][3], V[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
+    double D[3][3];
     for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) A[i][j] = 0.5 * (S[3 * i + j] + S[3 * j + i]);
-    for (int sweep = 0; sweep < 50; ++sweep) {
-        double off = fabs(A[0][1]) + fabs(A[0][2]) + fabs(A[1][2]);
-        if (off < 1e-15 * (fabs(A[0][0]) + fabs(A[1][1]) + fabs(A[2][2]) + 1e-300)) break;
+        for (int j = 0; j < 3; ++j) {
+            D[i][j] = B[i][j] * unit;
+            A[i][j] = (float)D[i][j];
+        }
+    for (int sweep = 0; sweep < 12; ++sweep) {
+        const float off = fabsf(A[0][1]) + fabsf(A[0][2]) + fabsf(A[1][2]);
+        if (off < 1e-9f) break;
         for (int p = 0; p < 2; ++p)
             for (int q = p + 1; q < 3; ++q) {
-                if (A[p][q] == 0.0) continue;
-                const double th = 0.5 * atan2(2 * A[p][q], A[q][q] - A[p][p]);
-                const double c = cos(th), s = sin(th);
+                if (A[p][q] == 0.0f) continue;
+                const float th = 0.5f * atan2f(2 * A[p][q], A[q][q] - A[p][p]);
+                float s, c;
+                sincosf(th, &s, &c);
                 for (int k = 0; k < 3; ++k) {       // A <- J^T A J
-                    const double akp = A[k][p], akq = A[k][q];
+                    const float akp = A[k][p], akq = A[k][q];
                     A[k][p] = c * akp - s * akq;
                     A[k][q] = s * akp + c * akq;
                 }
                 for (int k = 0; k < 3; ++k) {
-                    const double apk = A[p][k], aqk = A[q][k];
+                    const float apk = A[p][k], aqk = A[q][k];
                     A[p][k] = c * apk - s * aqk;
                     A[q][k] = s * apk + c * aqk;
                 }
                 for (int k = 0; k < 3; ++k) {
-                    const double vkp = V[k][p], vkq = V[k][q];
+                    const float vkp = V[k][p], vkq = V[k][q];
                     V[k][p] = c * vkp - s * vkq;
                     V[k][q] = s * vkp + c * vkq;
                 }
@@ -185,18 +202,48 @@ __device__ static void principal_axis(const double* S, float* a) {
     int best = 0;
     for (int i = 1; i < 3; ++i)
         if (A[i][i] > A[best][best]) best = i;
-    const double n = sqrt(V[0][best] * V[0][best] + V[1][best] * V[1][best] + V[2][best] * V[2][best]);
-    for (int i = 0; i < 3; ++i) a[i] = (float)(V[i][best] / (n > 0 ? n : 1.0));
+    double v[3] = {V[0][best], V[1][best], V[2][best]};
+    for (int it = 0; it < 3; ++it) {
+        double w[3], lam = 0.0, n2 = 0.0;
+        for (int i = 0; i < 3; ++i) {
+            w[i] = D[i][0] * v[0] + D[i][1] * v[1] + D[i][2] * v[2];
+            lam += w[i] * v[i];
+            n2 += v[i] * v[i];
+        }
+        lam *= 2.0 - n2;                            // Rayleigh quotient, |v| = 1 to 1e-6
+        for (int i = 0; i < 3; ++i) w[i] -= lam * v[i];
+        for (int j = 0; j < 3; ++j) {
+            const float gap = A[best][best] - A[j][j];
+            if (j == best || !(gap > 1e-6f)) continue;         // (nearly) equal eigenvalues: any axis of them
+            const double c = (w[0] * V[0][j] + w[1] * V[1][j] + w[2] * V[2][j]) * (double)(1.0f / gap);
+            for (int i = 0; i < 3; ++i) v[i] += c * V[i][j];
+        }
+        n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        const double r = 1.5 - 0.5 * n2;            // 1 / |v| to (n2 - 1)^2
+        for (int i = 0; i < 3; ++i) v[i] *= r;
+    }
+    for (int i = 0; i < 3; ++i) a[i] = (float)v[i];
 }
 
-__global__ void k_view_axis(const double* __restrict__ S, float* __restrict__ axis) {
-    principal_axis(S, axis);
+__global__ void k_view_axis(const double* __restrict__ part, int n, float* __restrict__ axis) {
+    __shared__ double s[6];
+    const int lane = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        double v = 0.0;
+        for (int i = lane; i < n; i += 32) v += part[6 * i + k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) s[k] = v;
+    }
+    if (lane == 0) principal_axis(s, axis);
 }
 
 cudaError_t launch_view_axis(Plan& P, const double* R, int M) {
-    double* tmp = P.ws.red_b;      // 9 doubles of scratch
-    k_view_moment<<<1, 1024, 0, P.stream>>>(R, M, tmp);
-    k_view_axis<<<1, 1, 0, P.stream>>>(tmp, P.ws.axis);
+    double* part = P.ws.red_b;      // scratch
+    const int n = min(kMomentBlocks, (M + kMomentThreads - 1) / kMomentThreads);
+    k_view_moment<<<n, kMomentThreads, 0, P.stream>>>(R, M, part);
+    k_view_axis<<<1, 32, 0, P.stream>>>(part, n, P.ws.axis);
     P.launches += 2;
     return cudaGetLastError();
 }
@@ -204,7 +251,7 @@ cudaError_t launch_view_axis(Plan& P, const double* R, int M) {
 cudaError_t launch_pc_features(Plan& P, int M, float* hist) {
     cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(float) * kBins, P.stream);
     if (e != cudaSuccess || M <= 0) return e;
-    const dim3 grid((M + kFeatThreads - 1) / kFeatThreads, (P.nH + kFeatT - 1) / kFeatT);
+    const dim3 grid((M + kFeatImgs - 1) / kFeatImgs, (P.nH + kFeatT - 1) / kFeatT);
     k_pc_features<<<grid, kFeatThreads, 0, P.stream>>>(P.ws.geom, P.ws.htab, P.cur_gid, P.ws.h2, M, P.nH, P.n_ctf,
                                                        0.5f * P.N, P.ws.axis, hist);
     P.launches += 1;
@@ -416,9 +463,45 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const float* __restrict__ A, co
             }
 }
 
+// Few rows (inference of up to 16 reconstructions): y = x W^T + bias with BF16 weights,
+// W N x K row-major, activations rounded to BF16.  A warp per 8 outputs, operands loaded
+// straight into the fragments: the same instruction over the same K steps as k_gemm_tc, so
+// the same sums to the bit (BF16 activations would turn another order's rounding into
+// differences of 2^-9), on N / 8 warps instead of N / 64 blocks that pass 64 rows of
+// mostly padding through shared memory (130 us a layer at K = 1024, 6 us here).
+constexpr int kFewRows = 16;
+__global__ void __launch_bounds__(32) k_gemm_few(const float* __restrict__ A, const __nv_bfloat16* __restrict__ B,
+                                                 float* __restrict__ C, int M, int N, int K,
+                                                 const float* __restrict__ bias, int relu) {
+    const int lane = threadIdx.x, g = lane >> 2, t = lane & 3, n0 = blockIdx.x * 8;
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(B + (size_t)(n0 + g) * K);
+    auto x2 = [&](int m, int k) { return m < M ? bf16x2(__ldg(&A[(size_t)m * K + k]), __ldg(&A[(size_t)m * K + k + 1])) : 0u; };
+    float acc[4] = {};
+#pragma unroll 8
+    for (int k0 = 0; k0 < K; k0 += kTcK) {
+        const uint32_t a[4] = {x2(g, k0 + 2 * t), x2(g + 8, k0 + 2 * t), x2(g, k0 + 2 * t + 8), x2(g + 8, k0 + 2 * t + 8)};
+        const uint32_t b[2] = {__ldg(&w[k0 / 2 + t]), __ldg(&w[k0 / 2 + t + 4])};
+        mma_bf16(acc, a, b);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int m = g + (q >= 2 ? 8 : 0), n = n0 + 2 * t + (q & 1);
+        if (m >= M) continue;
+        float v = acc[q];
+        if (bias) v += bias[n];
+        C[(size_t)m * N + n] = relu ? fmaxf(v, 0.0f) : v;
+    }
+}
+
 template <bool TA, bool TB, class WT>
 static void gemm(cudaStream_t s, const float* A, const WT* B, float* C, int M, int N, int K, const float* bias, bool relu,
                  bool acc = false) {
+    if constexpr (sizeof(WT) == 2 && !TA && TB) {
+        if (M <= kFewRows && !acc && N % 8 == 0 && K % kTcK == 0 && (reinterpret_cast<uintptr_t>(B) & 3) == 0) {
+            k_gemm_few<<<N / 8, 32, 0, s>>>(A, B, C, M, N, K, bias, relu ? 1 : 0);
+            return;
+        }
+    }
     const dim3 grid((N + kTcTile - 1) / kTcTile, (M + kTcTile - 1) / kTcTile);
     k_gemm_tc<TA, TB, WT><<<grid, 128, 0, s>>>(A, B, C, M, N, K, bias, relu ? 1 : 0, acc ? 1 : 0);
 }
