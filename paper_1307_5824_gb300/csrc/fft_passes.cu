@@ -131,7 +131,7 @@ struct NoFinish {
 struct KerRowsOp : NoFinish {
     const double* grid; float2* out; const float2* tw; int n_rows, G, N;
     __device__ __forceinline__ float2 load(int row, int n) const {
-        return make_float2((float)__ldg(&grid[(size_t)row * G + n]), 0.0f);
+        return make_float2(narrow(__ldg(&grid[(size_t)row * G + n])), 0.0f);
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
         if (k <= N) out[(size_t)row * (N + 1) + k] = v;
@@ -286,7 +286,7 @@ struct RhsRowsOp : NoFinish {
     const double* grid; float2* out; const float2* tw; int n_rows, G, N;
     __device__ __forceinline__ float2 load(int row, int n) const {
         const double2 g = __ldg(reinterpret_cast<const double2*>(grid) + (size_t)row * G + n);
-        return make_float2((float)g.x, (float)g.y);
+        return make_float2(narrow(g.x), narrow(g.y));
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
         const int h = N / 2;

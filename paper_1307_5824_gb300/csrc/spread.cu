@@ -595,6 +595,46 @@ __device__ __forceinline__ float2 point_weight(const SpreadArgs& a, bool cplx, i
 // PPR 2).
 template <bool CPLX> struct SpreadRound { static constexpr int PPR = CPLX ? 2 : 4; static constexpr int kScaleBits = CPLX ? 21 : 20; };
 
+// A brick's region (level 1 in units of inv_k / inv_b, plus level 2 when a fold wrote it)
+// into the FP64 grid (periodic wrap), both levels cleared.  NC planes: real (1), complex
+// (2), or the fused form's real Ker and complex A*b (3, the last NB of them A*b, whose grid
+// follows Ker's).  A thread takes an (x, y) column, so that it forms one address.
+template <int W, int NC, int NB>
+__device__ __forceinline__ void flush_region(const SpreadArgs& a, int bx, int by, int bz, int* lev1, float* lev2,
+                                             bool two, float inv_k, float inv_b) {
+    constexpr int RG = kBrick + W, RG2 = RG * RG, RG3 = RG2 * RG;
+    static_assert(RG2 <= 256, "a thread per column");
+    double* const gb = a.grid + (NC > NB ? (size_t)a.G * a.G * a.G : 0);
+    const int t = threadIdx.x;
+    if (t >= RG2) return;
+    const int ry = t / RG, rx = t - ry * RG;
+    int gx = bx * kBrick - W / 2 + rx, gy = by * kBrick - W / 2 + ry, gz = bz * kBrick - W / 2;
+    gx += gx < 0 ? a.G : gx >= a.G ? -a.G : 0;
+    gy += gy < 0 ? a.G : gy >= a.G ? -a.G : 0;
+    gz += gz < 0 ? a.G : 0;
+    const uint32_t col = (uint32_t)gy * a.G + gx, plane = (uint32_t)a.G * a.G;
+#pragma unroll 2
+    for (int rz = 0; rz < RG; ++rz) {
+        const uint32_t cell = (uint32_t)gz * plane + col;
+        if (++gz == a.G) gz = 0;
+#pragma unroll
+        for (int ch = 0; ch < NC; ++ch) {
+            const int i = ch * RG3 + rz * RG2 + t;
+            const bool ker = NC != 2 && ch == 0;
+            const float inv = ker ? inv_k : inv_b;
+            float v = (float)lev1[i] * inv;
+            if (two) {
+                v = fmaf((float)lev1[i], inv, lev2[i]);
+                lev2[i] = 0.0f;
+            }
+            lev1[i] = 0;
+            if (v == 0.0f) continue;
+            if (ker) atomicAdd(&a.grid[cell], widen(v));
+            else atomicAdd(&gb[2 * (size_t)cell + (ch - (NC - NB))], widen(v));
+        }
+    }
+}
+
 // One work item (a piece of one brick's points) into the brick's shared-memory region,
 // then the region into the FP64 grid.  lev1/lev2 are zero on entry and on return.
 template <int W, bool CPLX>
@@ -717,6 +757,7 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
             }
         }
         __syncthreads();
+        if (r + 1 == rounds) break;                // the last round goes straight to the grid
         for (int i = threadIdx.x; i < NC * RG3; i += blockDim.x) {
             const int v = lev1[i];
             if (v != 0) {
@@ -726,30 +767,7 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
         }
         __syncthreads();
     }
-    // add level 2 into the FP64 grid (periodic wrap) and clear it
-    const int o0 = lo0 - W / 2, o1 = lo1 - W / 2, o2 = lo2 - W / 2;
-    for (int i = threadIdx.x; i < RG3; i += blockDim.x) {
-        const float vr = lev2[i];
-        const float vi = CPLX ? lev2[RG3 + i] : 0.0f;
-        lev2[i] = 0.0f;
-        if (CPLX) lev2[RG3 + i] = 0.0f;
-        if (vr == 0.0f && vi == 0.0f) continue;
-        const int rx = i % RG, ry = (i / RG) % RG, rz = i / (RG * RG);
-        int gx = o0 + rx, gy = o1 + ry, gz = o2 + rz;
-        gx += (gx < 0) ? a.G : 0;
-        gx -= (gx >= a.G) ? a.G : 0;
-        gy += (gy < 0) ? a.G : 0;
-        gy -= (gy >= a.G) ? a.G : 0;
-        gz += (gz < 0) ? a.G : 0;
-        gz -= (gz >= a.G) ? a.G : 0;
-        const size_t cell = ((size_t)gz * a.G + gy) * a.G + gx;
-        if (CPLX) {
-            atomicAdd(&a.grid[2 * cell], (double)vr);
-            atomicAdd(&a.grid[2 * cell + 1], (double)vi);
-        } else {
-            atomicAdd(&a.grid[cell], (double)vr);
-        }
-    }
+    flush_region<W, NC, NC>(a, bx, by, bz, lev1, lev2, rounds > 1, invS, invS);
     __syncthreads();
 }
 
@@ -954,6 +972,7 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
             }
         }
         __syncthreads();
+        if (r + 1 == rounds) break;                // the last round goes straight to the grid
         for (int i = threadIdx.x; i < 3 * RG3; i += blockDim.x) {
             const int v = lev1[i];
             if (v != 0) {
@@ -963,29 +982,7 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
         }
         __syncthreads();
     }
-    // level 2 into the FP64 grids (periodic wrap) and cleared
-    const int o0 = lo0 - W / 2, o1 = lo1 - W / 2, o2 = lo2 - W / 2;
-    double* gk = a.grid;
-    double* gb = a.grid + (size_t)a.G * a.G * a.G;
-    for (int i = threadIdx.x; i < RG3; i += blockDim.x) {
-        const float vk = lev2[i], vr = lev2[RG3 + i], vi = lev2[2 * RG3 + i];
-        lev2[i] = 0.0f;
-        lev2[RG3 + i] = 0.0f;
-        lev2[2 * RG3 + i] = 0.0f;
-        if (vk == 0.0f && vr == 0.0f && vi == 0.0f) continue;
-        const int rx = i % RG, ry = (i / RG) % RG, rz = i / (RG * RG);
-        int gx = o0 + rx, gy = o1 + ry, gz = o2 + rz;
-        gx += (gx < 0) ? a.G : 0;
-        gx -= (gx >= a.G) ? a.G : 0;
-        gy += (gy < 0) ? a.G : 0;
-        gy -= (gy >= a.G) ? a.G : 0;
-        gz += (gz < 0) ? a.G : 0;
-        gz -= (gz >= a.G) ? a.G : 0;
-        const size_t cell = ((size_t)gz * a.G + gy) * a.G + gx;
-        if (vk != 0.0f) atomicAdd(&gk[cell], (double)vk);
-        if (vr != 0.0f) atomicAdd(&gb[2 * cell], (double)vr);
-        if (vi != 0.0f) atomicAdd(&gb[2 * cell + 1], (double)vi);
-    }
+    flush_region<W, 3, 2>(a, bx, by, bz, lev1, lev2, rounds > 1, invSk, invSb);
     __syncthreads();
 }
 

@@ -29,6 +29,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "dw.cuh"
 #include "firm_internal.h"
 #include "spread.cuh"
 
@@ -341,13 +342,6 @@ __device__ __forceinline__ void flush_class(const float (&D)[MmaCfg<W, CH>::T][C
             }
         }
     }
-}
-
-// float -> double by its bits (the conversion instruction runs at the FP64 rate); v is a
-// normal number here.
-__device__ __forceinline__ double widen(float v) {
-    const uint32_t b = __float_as_uint(v);
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
 // `n` 16-byte chunks of records from global to shared memory, asynchronously.
