@@ -628,7 +628,7 @@ int firm_kernel(firm_plan_t plan, int M, const double* R, const int32_t* group, 
     tm.start(0);
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
-    FIRM_CK(launch_bin(P, M, true, true));
+    FIRM_CK(launch_bin(P, M, true, BinFor::spread));
     tm.stop();
     tm.start(1);
     FIRM_CK(launch_spread(P, M, true));
@@ -687,7 +687,7 @@ int firm_backproject(firm_plan_t plan, int M, const void* images, const double* 
     if (from_stage) FIRM_CK(cudaEventRecord(P.ev_stage_read, P.stream));   // staging free again
     tm.stop();
     tm.start(5);
-    FIRM_CK(launch_bin(P, M, false, true));
+    FIRM_CK(launch_bin(P, M, false, BinFor::spread));
     tm.stop();
     tm.start(6);
     FIRM_CK(launch_spread(P, M, false));
@@ -726,7 +726,7 @@ int firm_kernel_backproject(firm_plan_t plan, int M, const void* images, const d
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
     tm.start(0);
-    FIRM_CK(launch_bin_count(P, M, 3, true));
+    FIRM_CK(launch_bin_count(P, M, 3, BinFor::spread));
     const bool place_first = !host_copy && !P.bin_mma;
     if (place_first) FIRM_CK(launch_bin_place(P, M, 3));
     tm.stop();
@@ -844,7 +844,7 @@ int firm_forward(firm_plan_t plan, int M, const float* V, const double* R, const
     FIRM_CK(stage_forward_inputs(P, M, V, R, group, Vd));
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += 1;
-    FIRM_CK(launch_bin(P, M, false, false));
+    FIRM_CK(launch_bin(P, M, false, BinFor::interp));
     float2* ghat = reinterpret_cast<float2*>(w.grid);
     FIRM_CK(launch_fwd_transform(P, Vd, ghat));
     const bool odev = is_device(out);
@@ -881,7 +881,7 @@ int firm_data_residual(firm_plan_t plan, int M, const float* V, const void* imag
     FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += 1;
     FIRM_CK(launch_image_dft(P, M, img, sh, P.cur_gid, true));    // b itself into samples
-    FIRM_CK(launch_bin(P, M, false, false));                                // b copied in scatter order
+    FIRM_CK(launch_bin(P, M, false, BinFor::interp));                                // b copied in scatter order
     float2* ghat = reinterpret_cast<float2*>(w.grid);
     FIRM_CK(launch_fwd_transform(P, Vd, ghat));
     FIRM_CK(launch_interp(P, M, ghat, nullptr, w.item_part, w.red_a));
@@ -1171,7 +1171,7 @@ int firm_bin(firm_plan_t plan, int M, const double* R, int channel) {
     FIRM_CK(e);
     FIRM_CK(launch_geom(Rd, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
-    FIRM_CK(launch_bin(P, M, channel == 0, false));
+    FIRM_CK(launch_bin(P, M, channel == 0, BinFor::inspect));
     P.bin_M = M;
     P.bin_kc = channel == 0;
     P.have_kernel = P.have_rhs = false;      // the ids share memory with the other stages' buffers

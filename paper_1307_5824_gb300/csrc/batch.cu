@@ -130,7 +130,7 @@ cudaError_t plan_front(Plan& P, const firm_batch_item& it, bool spread_here) {
     BCK(cudaMemsetAsync(w.counters + 2, 0, sizeof(int), P.stream));
     BCK(launch_geom(P.cur_R, M, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
-    BCK(launch_bin(P, M, true, true));
+    BCK(launch_bin(P, M, true, BinFor::spread));
     BCK(launch_spread_clear(P, true));
     if (spread_here) BCK(launch_spread_only(P, M, true));
     P.last_M = M;
@@ -146,7 +146,7 @@ cudaError_t plan_middle(Plan& P, const firm_batch_item& it, bool spread_here) {
     BCK(launch_lam_eff(P));
     BCK(launch_damping(P));
     BCK(launch_image_dft(P, M, P.cur_images, P.cur_shifts, P.cur_gid));
-    BCK(launch_bin(P, M, false, true));
+    BCK(launch_bin(P, M, false, BinFor::spread));
     BCK(launch_spread_clear(P, false));
     if (spread_here) BCK(launch_spread_only(P, M, false));
     return cudaSuccess;

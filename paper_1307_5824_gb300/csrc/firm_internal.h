@@ -199,14 +199,14 @@ double ctf_value(const firm_ctf_group& g, double r_invA);
 cudaError_t launch_geom(const double* R, int M, ImgGeom* geom, cudaStream_t s);
 // Binning in two steps: the count of points per brick and the work items (poses only),
 // then the points in the items' order.  ch: 1 kernel channel, 2 A*b, 3 both on the 4N
-// grid.  spread: the points will be spread, in the tensor-core form where spread_uses_mma
-// says so; otherwise (interpolation, inspection) they are ordered round-robin over bank
-// classes.  The tensor-core form places the A*b weights with the points: the image DFT
+// grid.  Points to be spread are ordered for the tensor-core form where spread_uses_mma
+// says so; otherwise (and for interpolation and inspection) round-robin over bank classes.  The tensor-core form places the A*b weights with the points: the image DFT
 // comes before launch_bin_place then.
-cudaError_t launch_bin_count(Plan& P, int M, int ch, bool spread);
+enum class BinFor { spread, interp, inspect };
+cudaError_t launch_bin_count(Plan& P, int M, int ch, BinFor use);
 cudaError_t launch_bin_place(Plan& P, int M, int ch);
-inline cudaError_t launch_bin(Plan& P, int M, bool kernel_channel, bool spread) {
-    const cudaError_t e = launch_bin_count(P, M, kernel_channel ? 1 : 2, spread);
+inline cudaError_t launch_bin(Plan& P, int M, bool kernel_channel, BinFor use) {
+    const cudaError_t e = launch_bin_count(P, M, kernel_channel ? 1 : 2, use);
     return e != cudaSuccess ? e : launch_bin_place(P, M, kernel_channel ? 1 : 2);
 }
 // Whether M images of a plan are spread in the tensor-core form (points: all of them, on a

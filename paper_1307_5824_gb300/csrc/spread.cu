@@ -525,7 +525,17 @@ static BinArgs bin_args(Plan& P, int M, bool kc) {
     return a;
 }
 
-cudaError_t launch_bin_count(Plan& P, int M, int ch, bool spread) {
+// Most points of an interpolation work item: a block gathers them from one brick's region,
+// whose load is the item's only fixed cost, so items are made small enough to balance the
+// blocks (about eight a block; at N = 64, 5,000 images 8e6 points were 1,000 items of 8,192
+// for 760 blocks: 0.86 ms, 0.55 with 2,048).
+static int interp_chunk(const Plan& P, int M) {
+    const long long each = (long long)M * P.nH / ((long long)P.num_sms * 40);
+    return (int)std::min<long long>(P.chunk, std::max<long long>(2048, each / 1024 * 1024));
+}
+
+cudaError_t launch_bin_count(Plan& P, int M, int ch, BinFor use) {
+    const bool spread = use == BinFor::spread;
     const bool kc = ch != 2;
     const int nb = kc ? P.nbk : P.nbr;
     const int nbricks = nb * nb * (kc ? P.nbkz : P.nbr);
@@ -541,7 +551,7 @@ cudaError_t launch_bin_count(Plan& P, int M, int ch, bool spread) {
             default: return cudaErrorInvalidValue;
         }
     }
-    launch_scan(P, nbricks, P.bin_mma ? kMmaChunk : P.chunk);
+    launch_scan(P, nbricks, P.bin_mma ? kMmaChunk : use == BinFor::interp ? interp_chunk(P, M) : P.chunk);
     return cudaGetLastError();
 }
 

@@ -75,6 +75,19 @@ template <int W, int CH> struct MmaCfg {
     static_assert(kClasses * 15 <= kMmaPad - 15, "record slots");
 };
 
+// Window polynomials of taps 0 .. (W - 1) / 2, scaled by kTapScale, every coefficient twice
+// (two points' worth): kernel parameters, so that they are operands from constant memory.
+struct MmaPoly {
+    float2 c[(kMaxW + 1) / 2][kKbDeg + 1];
+};
+
+static MmaPoly mma_poly(const KbPoly& P, int W) {
+    MmaPoly q{};
+    for (int l = 0; l < (W + 1) / 2; ++l)
+        for (int j = 0; j <= kKbDeg; ++j) q.c[l][j] = make_float2(P.c[l][j] * kTapScale, P.c[l][j] * kTapScale);
+    return q;
+}
+
 __device__ __forceinline__ uint32_t h2u(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
 __device__ __forceinline__ __half2 u2h(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 
@@ -111,7 +124,7 @@ __device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b
 // as fp16 pairs.  Taps l and W - 1 - l are one polynomial at z and -z: even and odd parts
 // are shared.
 template <int W, int BASES, int S>
-__device__ __forceinline__ void slot_taps(const float2* __restrict__ poly, uint2 c, uint32_t* hi, uint32_t* lo) {
+__device__ __forceinline__ void slot_taps(const MmaPoly& poly, uint2 c, uint32_t* hi, uint32_t* lo) {
     const int off0 = (int)(c.x >> (32 - kOffBits)), off1 = (int)(c.y >> (32 - kOffBits));
     // z = 2u - 1 from the 28-bit offset u: (u - 1/2) as a signed 32-bit fraction
     const float2 z = make_float2((float)(int)((c.x << kOffBits) ^ 0x80000000u) * (1.0f / 2147483648.0f),
@@ -120,7 +133,7 @@ __device__ __forceinline__ void slot_taps(const float2* __restrict__ poly, uint2
     const float2 z2 = __fmul2_rn(z, z);
 #pragma unroll
     for (int l = 0; l < (W + 1) / 2; ++l) {
-        const float2* p = poly + l * (kKbDeg + 1);
+        const float2* p = poly.c[l];
         const float2 ev = __ffma2_rn(__ffma2_rn(__ffma2_rn(p[6], z2, p[4]), z2, p[2]), z2, p[0]);
         const float2 od = __ffma2_rn(__ffma2_rn(__ffma2_rn(p[7], z2, p[5]), z2, p[3]), z2, p[1]);
         split2(__ffma2_rn(od, z, ev), hi[l], lo[l]);
@@ -354,7 +367,7 @@ __device__ __forceinline__ void copy_async(uint32_t* dst, const uint32_t* src, i
 
 // One work item.  lev1 is zero on entry and on return; called by the whole block.
 template <int W, int CH>
-__device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float2* s_poly, const int4 wk, int* lev1,
+__device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPoly& poly, const int4 wk, int* lev1,
                                                 uint32_t* wbuf) {
     using C = MmaCfg<W, CH>;
     constexpr int RG = C::RG, RG3 = C::RG3, BASES = C::kBases, RW = C::kRecWords, XS = C::XS, T = C::T;
@@ -404,7 +417,7 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
                     if (lane < 8 * (gb - g)) {
                         uint32_t hi[8], lo[8];
                         slot_taps<W, BASES, 8>(
-                            s_poly, *reinterpret_cast<const uint2*>(cur + (lane >> 3) * RW + 16 + 2 * pr), hi, lo);
+                            poly, *reinterpret_cast<const uint2*>(cur + (lane >> 3) * RW + 16 + 2 * pr), hi, lo);
                         uint4* y = reinterpret_cast<uint4*>(ys + (lane >> 3) * C::kYWords + pr * 8);
                         y[sw] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                         y[sw ^ 1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
@@ -413,7 +426,7 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
                         if (XS == 16) {            // x windows of 4 groups, layout as below
                             uint32_t xh[16], xl[16];
                             slot_taps<W, C::kBasesX, 16>(
-                                s_poly, *reinterpret_cast<const uint2*>(cur + (lane >> 3) * RW + 2 * pr), xh, xl);
+                                poly, *reinterpret_cast<const uint2*>(cur + (lane >> 3) * RW + 2 * pr), xh, xl);
                             uint32_t* Gs = xs + (lane >> 3) * C::kXWords;
 #pragma unroll
                             for (int s = 0; s < 16; ++s) {
@@ -429,7 +442,7 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
                 const int l16 = lane & 15, ax = lane >> 4, pr = l16 & 7;
                 if (l16 < 8 * (gb - g) && (XS == 8 || ax == 1)) {
                     uint32_t hi[8], lo[8];
-                    slot_taps<W, BASES, 8>(s_poly, *reinterpret_cast<const uint2*>(
+                    slot_taps<W, BASES, 8>(poly, *reinterpret_cast<const uint2*>(
                                                        cur + ((r & 2) + (l16 >> 3)) * RW + 32 * ax + 2 * pr),
                                            hi, lo);
                     uint32_t* Gs = ax ? zs + (l16 >> 3) * C::kZWords : xs + (l16 >> 3) * C::kXWords;
@@ -524,24 +537,13 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const float
     }
 }
 
-template <int W>
-__device__ __forceinline__ void load_poly(const KbPoly& P, float2* s_poly) {
-    constexpr int n = (W + 1) / 2 * (kKbDeg + 1);
-    for (int i = threadIdx.x; i < n; i += kMmaThreads) {
-        const float v = P.c[i / (kKbDeg + 1)][i % (kKbDeg + 1)] * kTapScale;
-        s_poly[i] = make_float2(v, v);
-    }
-}
-
 template <int W, int CH>
-__global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs a) {
+__global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs a, const __grid_constant__ MmaPoly poly) {
     using C = MmaCfg<W, CH>;
     extern __shared__ __align__(16) int sm_mma[];
-    __shared__ float2 s_poly[(W + 1) / 2 * (kKbDeg + 1)];
     __shared__ int s_item;
     int* const lev1 = sm_mma + kMmaWarps * (C::kWarpWords + 8 * C::kRecWords);
     uint32_t* const wbuf = reinterpret_cast<uint32_t*>(sm_mma) + (threadIdx.x >> 5) * (C::kWarpWords + 8 * C::kRecWords);
-    load_poly<W>(a.poly, s_poly);
     for (int i = threadIdx.x; i < CH * C::RG3; i += kMmaThreads) lev1[i] = 0;
     const int n_work = a.counters[0];
     for (;;) {
@@ -550,7 +552,7 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs 
         __syncthreads();
         const int item = s_item;
         if (item >= n_work) break;
-        spread_item_mma<W, CH>(a, s_poly, a.rec_item[item], lev1, wbuf);
+        spread_item_mma<W, CH>(a, poly, a.rec_item[item], lev1, wbuf);
     }
 }
 
@@ -559,14 +561,12 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs 
 template <int W, int CH>
 __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma_batch(const SpreadArgs* __restrict__ desc, int n,
                                                                      const int* __restrict__ item_off, int* queue,
-                                                                     const KbPoly poly) {
+                                                                     const __grid_constant__ MmaPoly poly) {
     using C = MmaCfg<W, CH>;
     extern __shared__ __align__(16) int sm_mma[];
-    __shared__ float2 s_poly[(W + 1) / 2 * (kKbDeg + 1)];
     __shared__ int s_item, s_prob;
     int* const lev1 = sm_mma + kMmaWarps * (C::kWarpWords + 8 * C::kRecWords);
     uint32_t* const wbuf = reinterpret_cast<uint32_t*>(sm_mma) + (threadIdx.x >> 5) * (C::kWarpWords + 8 * C::kRecWords);
-    load_poly<W>(poly, s_poly);
     for (int i = threadIdx.x; i < CH * C::RG3; i += kMmaThreads) lev1[i] = 0;
     const int total = item_off[n];
     for (;;) {
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma_batch(const Sprea
         if (g >= total) break;
         const int pi = s_prob;
         const SpreadArgs& a = desc[pi];
-        spread_item_mma<W, CH>(a, s_poly, a.rec_item[g - __ldg(&item_off[pi])], lev1, wbuf);
+        spread_item_mma<W, CH>(a, poly, a.rec_item[g - __ldg(&item_off[pi])], lev1, wbuf);
     }
 }
 
@@ -601,7 +601,7 @@ static cudaError_t spread_mma_batch_w(int n, const SpreadArgs* desc, const int* 
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_mma_batch<W, CH>, kMmaThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_spread_mma_batch<W, CH><<<num_sms * per_sm, kMmaThreads, smem, s>>>(desc, n, item_off, queue, poly);
+    k_spread_mma_batch<W, CH><<<num_sms * per_sm, kMmaThreads, smem, s>>>(desc, n, item_off, queue, mma_poly(poly, W));
     return cudaGetLastError();
 }
 
@@ -623,7 +623,7 @@ static cudaError_t spread_mma_w(Plan& P, const SpreadArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_mma<W, CH>, kMmaThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_spread_mma<W, CH><<<P.num_sms * per_sm, kMmaThreads, smem, P.stream>>>(a);
+    k_spread_mma<W, CH><<<P.num_sms * per_sm, kMmaThreads, smem, P.stream>>>(a, mma_poly(a.poly, W));
     P.launches += 1;
     return cudaGetLastError();
 }
