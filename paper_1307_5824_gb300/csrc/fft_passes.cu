@@ -58,6 +58,8 @@ template <int L> __host__ __device__ constexpr int TX() { return kThreads / Spli
 // ---------------------------------------------------------------------------
 template <int L, int SIGN, class Op>
 __global__ void __launch_bounds__(kThreads) k_cols(const Op op) {
+    pdl_wait();
+    pdl_launch();
     extern __shared__ float2 S[];
     const int tiles = (op.n_inner + TX<L>() - 1) / TX<L>();
     const int outer = blockIdx.x / tiles;
@@ -72,6 +74,8 @@ template <int L> __host__ __device__ constexpr int rows_per_block() { return kTh
 
 template <int L, int SIGN, class Op>
 __global__ void __launch_bounds__(kThreads) k_rows(Op op) {
+    pdl_wait();
+    pdl_launch();
     extern __shared__ float2 S[];
     constexpr int ROWS = rows_per_block<L>();
     const int r0 = blockIdx.x * ROWS;
@@ -88,7 +92,7 @@ static cudaError_t run_cols(const Op& op, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(k_cols<L, SIGN, Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int tiles = (op.n_inner + TX<L>() - 1) / TX<L>();
-    k_cols<L, SIGN, Op><<<op.n_outer * tiles, kThreads, smem, s>>>(op);
+    launch_pdl(k_cols<L, SIGN, Op>, op.n_outer * tiles, kThreads, smem, s, op);
     return cudaGetLastError();
 }
 
@@ -98,7 +102,7 @@ static cudaError_t run_rows(const Op& op, cudaStream_t s) {
     const size_t smem = sizeof(float2) * smem_elems<L, false>(ROWS);
     cudaError_t e = cudaFuncSetAttribute(k_rows<L, SIGN, Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_rows<L, SIGN, Op><<<(op.n_rows + ROWS - 1) / ROWS, kThreads, smem, s>>>(op);
+    launch_pdl(k_rows<L, SIGN, Op>, (op.n_rows + ROWS - 1) / ROWS, kThreads, smem, s, op);
     return cudaGetLastError();
 }
 
@@ -229,6 +233,8 @@ cudaError_t launch_khat(Plan& P) {
 // lam_eff = lambda Ker(0) (relative reading) or lambda (absolute), on the device, so that
 // the Toeplitz apply needs no host round trip; Ker(0) sits at (j3, j2, j1) = (N, N, 0).
 __global__ void k_lam_eff(const float* __restrict__ ker, size_t i0, double lambda, int relative, float* lam) {
+    pdl_wait();
+    pdl_launch();
     const float k0 = ker[i0];
     lam[0] = relative ? (float)(lambda * (double)k0) : (float)lambda;
     lam[1] = k0;
@@ -236,7 +242,7 @@ __global__ void k_lam_eff(const float* __restrict__ ker, size_t i0, double lambd
 
 cudaError_t launch_lam_eff(Plan& P) {
     const size_t i0 = ((size_t)P.N * 2 * P.N + P.N) * (P.N + 1);
-    k_lam_eff<<<1, 1, 0, P.stream>>>(P.ws.ker, i0, P.p.lambda, P.p.lambda_mode == FIRM_LAMBDA_RELATIVE ? 1 : 0,
+    launch_pdl(k_lam_eff, 1, 1, 0, P.stream, P.ws.ker, i0, P.p.lambda, P.p.lambda_mode == FIRM_LAMBDA_RELATIVE ? 1 : 0,
                                      P.ws.lam);
     P.launches += 1;
     return cudaGetLastError();
@@ -442,6 +448,8 @@ template <int N> __host__ __device__ constexpr int img_smem_elems() {
 
 template <int N, class T>
 __global__ void __launch_bounds__(kThreads) k_image_dft(const ImgArgs a) {
+    pdl_wait();
+    pdl_launch();
     extern __shared__ float2 sm2[];
     __shared__ __align__(8) unsigned long long s_bar;
     constexpr int H1 = N / 2 + 1;
@@ -559,7 +567,7 @@ static cudaError_t image_dft_n(Plan& P, int M, const ImgArgs& a) {
     const size_t smem = sizeof(float2) * img_smem_elems<N>();
     cudaError_t e = cudaFuncSetAttribute(k_image_dft<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_image_dft<N, T><<<M, kThreads, smem, P.stream>>>(a);
+    launch_pdl(k_image_dft<N, T>, M, kThreads, smem, P.stream, a);
     P.launches += 1;
     return cudaGetLastError();
 }

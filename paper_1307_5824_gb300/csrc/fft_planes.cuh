@@ -17,33 +17,9 @@
 #include <cuda_runtime.h>
 
 #include "fft.cuh"
+#include "pdl.cuh"
 
 namespace firm {
-
-// Programmatic dependent launch: the next kernel of the stream may start its blocks now
-// (it waits in pdl_wait until this one has finished and its writes are visible).
-__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-template <class... KArgs, class... Args>
-static cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
-                              Args... args) {
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c{};
-    c.gridDim = dim3((unsigned)grid);
-    c.blockDim = dim3((unsigned)block);
-    c.dynamicSmemBytes = smem;
-    c.stream = s;
-    c.attrs = at;
-    c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, kernel, KArgs(args)...);
-}
 
 // Sum of n partial sums by one warp, in a fixed order; valid in every lane.  The kernel that
 // needs a reduction's result sums the blocks' partials itself (every block the same way):

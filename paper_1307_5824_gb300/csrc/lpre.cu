@@ -15,6 +15,7 @@
 #include <cmath>
 
 #include "firm_internal.h"
+#include "pdl.cuh"
 
 namespace firm {
 
@@ -36,6 +37,8 @@ __device__ __forceinline__ int freq_bin(float q1, float q2, float q3, float half
 constexpr int kMomentBlocks = 64, kMomentThreads = 256;
 __global__ void __launch_bounds__(kMomentThreads) k_view_moment(const double* __restrict__ R, int M,
                                                                double* __restrict__ part) {
+    pdl_wait();
+    pdl_launch();
     __shared__ double s[kMomentThreads / 32][6];
     double acc[6] = {0, 0, 0, 0, 0, 0};            // xx, xy, xz, yy, yz, zz
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
@@ -226,6 +229,8 @@ __device__ static void principal_axis(const double* S, float* a) {     // S: xx,
 }
 
 __global__ void k_view_axis(const double* __restrict__ part, int n, float* __restrict__ axis) {
+    pdl_wait();
+    pdl_launch();
     __shared__ double s[6];
     const int lane = threadIdx.x;
 #pragma unroll
@@ -242,8 +247,8 @@ __global__ void k_view_axis(const double* __restrict__ part, int n, float* __res
 cudaError_t launch_view_axis(Plan& P, const double* R, int M) {
     double* part = P.ws.red_b;      // scratch
     const int n = min(kMomentBlocks, (M + kMomentThreads - 1) / kMomentThreads);
-    k_view_moment<<<n, kMomentThreads, 0, P.stream>>>(R, M, part);
-    k_view_axis<<<1, 32, 0, P.stream>>>(part, n, P.ws.axis);
+    launch_pdl(k_view_moment, n, kMomentThreads, 0, P.stream, R, M, part);
+    launch_pdl(k_view_axis, 1, 32, 0, P.stream, part, n, P.ws.axis);
     P.launches += 2;
     return cudaGetLastError();
 }

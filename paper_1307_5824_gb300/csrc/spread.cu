@@ -25,6 +25,7 @@
 
 #include "dw.cuh"
 #include "firm_internal.h"
+#include "pdl.cuh"
 #include "spread.cuh"
 
 namespace firm {
@@ -33,6 +34,8 @@ namespace firm {
 // Geometry
 // ---------------------------------------------------------------------------
 __global__ void k_geom(const double* __restrict__ R, int M, ImgGeom* __restrict__ g) {
+    pdl_wait();
+    pdl_launch();
     int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
     const double* r = R + 9 * (size_t)m;
@@ -54,7 +57,7 @@ __global__ void k_geom(const double* __restrict__ R, int M, ImgGeom* __restrict_
 
 cudaError_t launch_geom(const double* R, int M, ImgGeom* geom, cudaStream_t s) {
     if (M <= 0) return cudaSuccess;
-    k_geom<<<(M + 255) / 256, 256, 0, s>>>(R, M, geom);
+    launch_pdl(k_geom, (M + 255) / 256, 256, 0, s, R, M, geom);
     return cudaGetLastError();
 }
 
@@ -86,6 +89,8 @@ struct BinArgs {
 
 template <int W, bool SCATTER, bool KC>
 __global__ void __launch_bounds__(256) k_bin(BinArgs a, int M) {
+    pdl_wait();
+    pdl_launch();
     constexpr int BZ = Brick<KC>::BZ;
     // x: samples t of one image (consecutive lanes walk a column of the half disc);
     // y: images.  Runs of equal bricks among consecutive lanes are aggregated.
@@ -135,6 +140,8 @@ __global__ void __launch_bounds__(256) k_bin(BinArgs a, int M) {
 template <int W, bool KC, int CH>
 __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN, const int4* __restrict__ col,
                                                        int tiles_x, int n_tiles) {
+    pdl_wait();
+    pdl_launch();
     constexpr int BZ = Brick<KC>::BZ;
     const int lane = threadIdx.x & 31;
     const int tile = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -248,6 +255,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* __
                                                               uint32_t* __restrict__ cursor, int nbricks,
                                                               ScanPart* __restrict__ part, int4* __restrict__ work,
                                                               int* __restrict__ counters, int max_work, int chunk) {
+    pdl_wait();
+    pdl_launch();
     __shared__ ScanPart s_w[32], s_tot;
     const int b = blockIdx.x * kScanSpan + 4 * threadIdx.x;
     uint4 c4 = make_uint4(0, 0, 0, 0);
@@ -290,6 +299,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* __
 
 // Exclusive scan of the per-block totals in place (one block; n <= 32 * kScanThreads).
 __global__ void __launch_bounds__(kScanThreads) k_scan_parts(ScanPart* __restrict__ part, int n) {
+    pdl_wait();
+    pdl_launch();
     __shared__ ScanPart s_w[32], s_tot;
     const int per = (n + kScanThreads - 1) / kScanThreads;
     const int i0 = min(n, (int)threadIdx.x * per), i1 = min(n, i0 + per);
@@ -313,10 +324,10 @@ static void launch_scan(Plan& P, int nbricks, int chunk) {
     Workspace& w = P.ws;
     const int nblk = (nbricks + kScanSpan - 1) / kScanSpan;
     ScanPart* part = reinterpret_cast<ScanPart*>(w.scan_part);
-    k_scan_bricks<false><<<nblk, kScanThreads, 0, P.stream>>>(w.count, w.cursor, nbricks, part, w.work,
+    launch_pdl(k_scan_bricks<false>, nblk, kScanThreads, 0, P.stream, w.count, w.cursor, nbricks, part, w.work,
                                                                w.counters, (int)P.max_work, chunk);
-    k_scan_parts<<<1, kScanThreads, 0, P.stream>>>(part, nblk);
-    k_scan_bricks<true><<<nblk, kScanThreads, 0, P.stream>>>(w.count, w.cursor, nbricks, part, w.work,
+    launch_pdl(k_scan_parts, 1, kScanThreads, 0, P.stream, part, nblk);
+    launch_pdl(k_scan_bricks<true>, nblk, kScanThreads, 0, P.stream, w.count, w.cursor, nbricks, part, w.work,
                                                               w.counters, (int)P.max_work, chunk);
     P.launches += 3;
 }
@@ -343,6 +354,8 @@ __global__ void __launch_bounds__(256) k_class_sort(uint32_t* __restrict__ paylo
                                                     const int4* __restrict__ work, const int* __restrict__ counters,
                                                     uint16_t* __restrict__ perm, const uint32_t* __restrict__ in,
                                                     uint16_t* __restrict__ inv_perm) {
+    pdl_wait();
+    pdl_launch();
     extern __shared__ uint32_t sm_u[];
     uint32_t* s_ids = sm_u;                                         // kChunk
     uint32_t* s_mask = s_ids + kChunk;                              // kSortLevels: classes with n_c > r
@@ -441,7 +454,7 @@ static void launch_class_sort(Plan& P, bool kc) {
     Workspace& w = P.ws;
     cudaFuncSetAttribute(k_class_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem);
     const bool keep = kc && w.payload_scat;       // fused plans keep the scatter order
-    k_class_sort<<<P.num_sms * 4, 256, kSortSmem, P.stream>>>(w.payload, w.cls, w.work, w.counters,
+    launch_pdl(k_class_sort, P.num_sms * 4, 256, kSortSmem, P.stream, w.payload, w.cls, w.work, w.counters,
                                                                kc ? nullptr : w.perm, keep ? w.payload_scat : nullptr,
                                                                keep ? w.inv_perm : nullptr);
     P.launches += 1;
@@ -450,8 +463,8 @@ static void launch_class_sort(Plan& P, bool kc) {
 template <int W>
 static void bin_count_w(Plan& P, const BinArgs& a, int M, bool kc) {
     const dim3 grid((a.nH + 255) / 256, (unsigned)(M < 65535 ? M : 65535));
-    if (kc) k_bin<W, false, true><<<grid, 256, 0, P.stream>>>(a, M);
-    else k_bin<W, false, false><<<grid, 256, 0, P.stream>>>(a, M);
+    if (kc) launch_pdl(k_bin<W, false, true>, grid, 256, 0, P.stream, a, M);
+    else launch_pdl(k_bin<W, false, false>, grid, 256, 0, P.stream, a, M);
     P.launches += 1;
 }
 
@@ -463,12 +476,12 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
     const int4* col = P.ws.colinfo;
     const bool sm = a.samples != nullptr;
     if (P.bin_mma) {
-        if (kc && sm) k_bin_scatter2d<W, true, 3><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
-        else if (kc) k_bin_scatter2d<W, true, 1><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
-        else k_bin_scatter2d<W, false, 2><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
+        if (kc && sm) launch_pdl(k_bin_scatter2d<W, true, 3>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
+        else if (kc) launch_pdl(k_bin_scatter2d<W, true, 1>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
+        else launch_pdl(k_bin_scatter2d<W, false, 2>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
     } else {
-        if (kc) k_bin_scatter2d<W, true, 0><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
-        else k_bin_scatter2d<W, false, 0><<<g, 256, 0, P.stream>>>(a, M, hN, col, tiles_x, n_tiles);
+        if (kc) launch_pdl(k_bin_scatter2d<W, true, 0>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
+        else launch_pdl(k_bin_scatter2d<W, false, 0>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
     }
     P.launches += 1;
 }
@@ -783,6 +796,8 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
 
 template <int W, bool CPLX>
 __global__ void __launch_bounds__(kSpreadThreads, CPLX ? 5 : 6) k_spread(const SpreadArgs a) {
+    pdl_wait();
+    pdl_launch();
     constexpr int NC = CPLX ? 2 : 1;
     constexpr int R3 = (kBrick + W) * (kBrick + W) * (Brick<!CPLX>::BZ + W);
     extern __shared__ int sm_i[];
@@ -998,6 +1013,8 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
 
 template <int W>
 __global__ void __launch_bounds__(kFusedThreads) k_spread_fused(const SpreadArgs a) {
+    pdl_wait();
+    pdl_launch();
     constexpr int R3 = (kBrick + W) * (kBrick + W) * (kBrickZk + W);
     extern __shared__ int sm_i[];
     int* lev1 = sm_i;                                          // 3 * R3 int32
@@ -1023,6 +1040,8 @@ __global__ void __launch_bounds__(256) k_fused_gather(const uint32_t* __restrict
                                                       const int4* __restrict__ work, const int* __restrict__ counters,
                                                       const float2* __restrict__ samples, int nH,
                                                       float2* __restrict__ samples_b, float* __restrict__ wmax_item) {
+    pdl_wait();
+    pdl_launch();
     __shared__ float s_red[8];
     const int n_work = counters[0];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1060,7 +1079,7 @@ static cudaError_t spread_fused_w(Plan& P, const SpreadArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_fused<W>, kFusedThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_spread_fused<W><<<P.num_sms * per_sm, kFusedThreads, smem, P.stream>>>(a);
+    launch_pdl(k_spread_fused<W>, P.num_sms * per_sm, kFusedThreads, smem, P.stream, a);
     P.launches += 1;
     return cudaGetLastError();
 }
@@ -1080,7 +1099,7 @@ static cudaError_t spread_w(Plan& P, const SpreadArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread<W, CPLX>, kSpreadThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_spread<W, CPLX><<<P.num_sms * per_sm, kSpreadThreads, smem, P.stream>>>(a);
+    launch_pdl(k_spread<W, CPLX>, P.num_sms * per_sm, kSpreadThreads, smem, P.stream, a);
     P.launches += 1;
     return cudaGetLastError();
 }
@@ -1163,7 +1182,7 @@ cudaError_t launch_fused_gather(Plan& P, int M) {
     Workspace& w = P.ws;
     if (!w.payload_scat) return cudaErrorInvalidValue;      // fused plans only
     if (P.bin_mma) return cudaSuccess;                       // the spreading kernel gathers its weights itself
-    k_fused_gather<<<P.num_sms * 8, 256, 0, P.stream>>>(w.payload_scat, w.inv_perm, w.work, w.counters, w.samples,
+    launch_pdl(k_fused_gather, P.num_sms * 8, 256, 0, P.stream, w.payload_scat, w.inv_perm, w.work, w.counters, w.samples,
                                                        P.nH, w.samples_b, w.wmax_item);
     P.launches += 1;
     return cudaGetLastError();
@@ -1244,6 +1263,8 @@ struct InterpArgs {
 
 template <int W, bool RESID>
 __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
+    pdl_wait();
+    pdl_launch();
     constexpr int BZ = kBrick;
     constexpr int RG = kBrick + W;
     constexpr int RG3 = RG * RG * (BZ + W);
@@ -1348,6 +1369,8 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
 // out[0..1] = sums over the work items, in item order (one CTA: fixed order).
 __global__ void __launch_bounds__(1024) k_item_sum(const double* __restrict__ part, const int* __restrict__ counters,
                                                    double* __restrict__ out) {
+    pdl_wait();
+    pdl_launch();
     __shared__ double s[2][1024];
     const int n = counters[0];
     double r = 0.0, b = 0.0;
@@ -1381,7 +1404,7 @@ static cudaError_t interp_w(Plan& P, const InterpArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp<W, RESID>, kSpreadThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_interp<W, RESID><<<P.num_sms * per_sm, kSpreadThreads, smem, P.stream>>>(a);
+    launch_pdl(k_interp<W, RESID>, P.num_sms * per_sm, kSpreadThreads, smem, P.stream, a);
     P.launches += 1;
     return cudaGetLastError();
 }
@@ -1418,7 +1441,7 @@ cudaError_t launch_interp(Plan& P, int M, const float2* ghat, float2* out, doubl
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess || !resid) return e;
-    k_item_sum<<<1, 1024, 0, P.stream>>>(item_part, w.counters, sums);
+    launch_pdl(k_item_sum, 1, 1024, 0, P.stream, item_part, w.counters, sums);
     P.launches += 1;
     return cudaGetLastError();
 }

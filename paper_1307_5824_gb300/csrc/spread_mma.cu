@@ -31,6 +31,7 @@
 
 #include "dw.cuh"
 #include "firm_internal.h"
+#include "pdl.cuh"
 #include "spread.cuh"
 
 namespace firm {
@@ -167,6 +168,8 @@ __device__ __forceinline__ void slot_taps(const MmaPoly& poly, uint2 c, uint32_t
 // ---------------------------------------------------------------------------
 template <int W, int CH>
 __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a) {
+    pdl_wait();
+    pdl_launch();
     using C = MmaCfg<W, CH>;
     constexpr int BASES = C::kBases, BX = C::kBasesX, RW = C::kRecWords, PT = kMmaChunk / kSortThreads;
     constexpr int kWarps = kSortThreads / 32;
@@ -539,6 +542,8 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPo
 
 template <int W, int CH>
 __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs a, const __grid_constant__ MmaPoly poly) {
+    pdl_wait();
+    pdl_launch();
     using C = MmaCfg<W, CH>;
     extern __shared__ __align__(16) int sm_mma[];
     __shared__ int s_item;
@@ -623,7 +628,7 @@ static cudaError_t spread_mma_w(Plan& P, const SpreadArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_mma<W, CH>, kMmaThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_spread_mma<W, CH><<<P.num_sms * per_sm, kMmaThreads, smem, P.stream>>>(a, mma_poly(a.poly, W));
+    launch_pdl(k_spread_mma<W, CH>, P.num_sms * per_sm, kMmaThreads, smem, P.stream, a, mma_poly(a.poly, W));
     P.launches += 1;
     return cudaGetLastError();
 }
@@ -633,7 +638,7 @@ static cudaError_t mma_sort_w(Plan& P, const SpreadArgs& a) {
     constexpr size_t smem = MmaCfg<W, CH>::kSortSmem;
     cudaError_t e = cudaFuncSetAttribute(k_mma_sort<W, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_mma_sort<W, CH><<<P.num_sms * 2, kSortThreads, smem, P.stream>>>(a);
+    launch_pdl(k_mma_sort<W, CH>, P.num_sms * 2, kSortThreads, smem, P.stream, a);
     P.launches += 1;
     return cudaGetLastError();
 }
