@@ -626,7 +626,7 @@ int firm_kernel(firm_plan_t plan, int M, const double* R, const int32_t* group, 
     FIRM_CK(start_stage(P));                   // a staged image upload runs beside the kernel channel
     P.bin_M = -1;
     tm.start(0);
-    FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
+    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
     FIRM_CK(launch_bin(P, M, true, BinFor::spread));
     tm.stop();
@@ -681,7 +681,7 @@ int firm_backproject(firm_plan_t plan, int M, const void* images, const double* 
     }
     P.bin_M = -1;
     tm.start(4);
-    FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
+    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
     FIRM_CK(launch_image_dft(P, M, P.cur_images, P.cur_shifts, P.cur_gid));
     if (from_stage) FIRM_CK(cudaEventRecord(P.ev_stage_read, P.stream));   // staging free again
@@ -723,7 +723,7 @@ int firm_kernel_backproject(firm_plan_t plan, int M, const void* images, const d
     const bool host_copy = M > 0 && !staged && !is_device(images);
     if (staged) FIRM_CK(start_stage(P));
     P.bin_M = -1;
-    FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
+    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
     tm.start(0);
     FIRM_CK(launch_bin_count(P, M, 3, BinFor::spread));
@@ -842,7 +842,7 @@ int firm_forward(firm_plan_t plan, int M, const float* V, const double* R, const
     if (M == 0) return FIRM_OK;
     const float* Vd = nullptr;
     FIRM_CK(stage_forward_inputs(P, M, V, R, group, Vd));
-    FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
+    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
     P.launches += 1;
     FIRM_CK(launch_bin(P, M, false, BinFor::interp));
     float2* ghat = reinterpret_cast<float2*>(w.grid);
@@ -878,7 +878,7 @@ int firm_data_residual(firm_plan_t plan, int M, const float* V, const void* imag
         FIRM_CK(cudaMemcpyAsync(w.images, images, (size_t)M * P.N * P.N * esz, cudaMemcpyHostToDevice, P.stream));
         img = w.images;
     }
-    FIRM_CK(launch_geom(P.cur_R, M, w.geom, P.stream));
+    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
     P.launches += 1;
     FIRM_CK(launch_image_dft(P, M, img, sh, P.cur_gid, true));    // b itself into samples
     FIRM_CK(launch_bin(P, M, false, BinFor::interp));                                // b copied in scatter order
@@ -1169,7 +1169,7 @@ int firm_bin(firm_plan_t plan, int M, const double* R, int channel) {
     cudaError_t e = cudaSuccess;
     const double* Rd = stage(R, w.R, (size_t)M * 9, P.stream, e);
     FIRM_CK(e);
-    FIRM_CK(launch_geom(Rd, M, w.geom, P.stream));
+    FIRM_CK(launch_geom(Rd, M, P.N, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
     FIRM_CK(launch_bin(P, M, channel == 0, BinFor::inspect));
     P.bin_M = M;

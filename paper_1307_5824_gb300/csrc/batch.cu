@@ -128,7 +128,7 @@ cudaError_t plan_front(Plan& P, const firm_batch_item& it, bool spread_here) {
     if (it.shifts) P.cur_shifts = it.shifts;
     else { BCK(cudaMemsetAsync(w.shifts, 0, sizeof(double) * 2 * (M > 0 ? M : 1), P.stream)); P.cur_shifts = w.shifts; }
     BCK(cudaMemsetAsync(w.counters + 2, 0, sizeof(int), P.stream));
-    BCK(launch_geom(P.cur_R, M, w.geom, P.stream));
+    BCK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
     P.launches += M > 0 ? 1 : 0;
     BCK(launch_bin(P, M, true, BinFor::spread));
     BCK(launch_spread_clear(P, true));

@@ -196,12 +196,13 @@ double wavelength_A(double kV);
 double ctf_value(const firm_ctf_group& g, double r_invA);
 
 // ---- launchers (spread.cu) ----
-cudaError_t launch_geom(const double* R, int M, ImgGeom* geom, cudaStream_t s);
+cudaError_t launch_geom(const double* R, int M, int N, ImgGeom* geom, cudaStream_t s);
 // Binning in two steps: the count of points per brick and the work items (poses only),
 // then the points in the items' order.  ch: 1 kernel channel, 2 A*b, 3 both on the 4N
 // grid.  Points to be spread are ordered for the tensor-core form where spread_uses_mma
-// says so; otherwise (and for interpolation and inspection) round-robin over bank classes.  The tensor-core form places the A*b weights with the points: the image DFT
-// comes before launch_bin_place then.
+// says so; otherwise (and for interpolation and inspection) round-robin over bank classes.  The
+// tensor-core form places the A*b weights with the points: the image DFT comes before
+// launch_bin_place then.
 enum class BinFor { spread, interp, inspect };
 cudaError_t launch_bin_count(Plan& P, int M, int ch, BinFor use);
 cudaError_t launch_bin_place(Plan& P, int M, int ch);

@@ -33,7 +33,11 @@ namespace firm {
 // ---------------------------------------------------------------------------
 // Geometry
 // ---------------------------------------------------------------------------
-__global__ void k_geom(const double* __restrict__ R, int M, ImgGeom* __restrict__ g) {
+// Pairs (R_1d, R_2d) longer than `longest` are dropped (NaN too), so that no point leaves the
+// bricks.  Rotations have at most 1; scaled matrices are taken up to 2.9 (one wrap of the grid)
+// where 4N divides the 512 cells of a 32-bit position, else up to its +-256 cells: 2.66, 1.59
+// and 1.33 at N = 48, 80 and 96.
+__global__ void k_geom(const double* __restrict__ R, int M, double longest, ImgGeom* __restrict__ g) {
     pdl_wait();
     pdl_launch();
     int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -42,9 +46,7 @@ __global__ void k_geom(const double* __restrict__ R, int M, ImgGeom* __restrict_
     ImgGeom o;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        // a column of R longer than 1.3 (never a rotation; NaN too) would leave the grid by
-        // more than the arithmetic holds: it is dropped, so that no point leaves the bricks
-        const bool ok = r[d] * r[d] + r[3 + d] * r[3 + d] <= 1.69;
+        const bool ok = r[d] * r[d] + r[3 + d] * r[3 + d] <= longest * longest;
         const long long u = ok ? __double2ll_rn(r[d] * (double)(1ll << kGeomBits)) : 0;
         const long long v = ok ? __double2ll_rn(r[3 + d] * (double)(1ll << kGeomBits)) : 0;
         o.uh[d] = (int)(u >> 16);
@@ -55,9 +57,10 @@ __global__ void k_geom(const double* __restrict__ R, int M, ImgGeom* __restrict_
     g[m] = o;
 }
 
-cudaError_t launch_geom(const double* R, int M, ImgGeom* geom, cudaStream_t s) {
+cudaError_t launch_geom(const double* R, int M, int N, ImgGeom* geom, cudaStream_t s) {
     if (M <= 0) return cudaSuccess;
-    launch_pdl(k_geom, (M + 255) / 256, 256, 0, s, R, M, geom);
+    const double longest = 512 % (4 * N) == 0 ? 2.9 : std::min(2.9, 127.8 / N);
+    launch_pdl(k_geom, (M + 255) / 256, 256, 0, s, R, M, longest, geom);
     return cudaGetLastError();
 }
 

@@ -15,9 +15,9 @@ namespace firm {
 // cells.  ls = log2(G / N) <= 2; exact, since u = uh 2^16 + ul to the last bit.
 constexpr int kFracBits = 23;
 __device__ __forceinline__ int axis_pos(const ImgGeom& g, int d, int k1, int k2, int ls) {
-    const int p = k1 * g.uh[d] + k2 * g.vh[d];
+    const unsigned p = (unsigned)k1 * (unsigned)g.uh[d] + (unsigned)k2 * (unsigned)g.vh[d];   // wraps
     const int q = k1 * g.ul[d] + k2 * g.vl[d] + (1 << (17 - ls));
-    return (p + (q >> 16)) >> (2 - ls);
+    return (int)(p + (unsigned)(q >> 16)) >> (2 - ls);
 }
 
 // A cell I in [0, G) (periodic) and a fraction of q / 2^23 cells per axis.
@@ -33,8 +33,9 @@ __device__ __forceinline__ PointPos point_pos(const ImgGeom& g, int32_t kk, int 
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const int t = axis_pos(g, d, k1, k2, ls);
-        // |k1 u + k2 v| <= |k| <= N/2 (u, v: parts of a unit column of R), so the cell lies
-        // in [-1, G]: one wrap either way is the periodic index
+        // |k1 u + k2 v| <= |k| <= N/2 (u, v: parts of a unit column of R) puts the cell in
+        // [-1, G], and k_geom keeps longer ones within [-G, 2G): one wrap either way is the
+        // periodic index
         int I = (t >> kFracBits) + halfG;
         if (I >= G) I -= G;
         else if (I < 0) I += G;

@@ -53,3 +53,29 @@ def test_tensor_core_spreading_matches_oracle(N, M, cfg, fused, W):
     print(f"N={N} M={M} {cfg} W={W} fused={fused}: Ker {e_k:.2e} A*b {e_r:.2e}")
     assert e_k <= 3e-6 and e_r <= 3e-6
     rec.close()
+
+
+@pytest.mark.parametrize("N,scale", [(16, 2.8), (48, 2.5), (64, 1.5), (80, 1.5), (96, 1.3)])
+def test_scaled_matrices_wrap_the_grid(N, scale):
+    """Matrices longer than a rotation put samples past the grid's edge, where they wrap:
+    Ker against its direct sum at 300 lags.  KB W = 6 is within 2e-5 of the sum of |weights|
+    there; a lag's own sum is at least a tenth of their root mean square, so 1e-3 of the
+    lags' norm, against 1 for samples in wrong cells."""
+    import __graft_entry__ as g
+    g.build()
+    import paper_1307_5824_gb300 as F
+    inp = synth.config_inputs("C2", M=5, N=N)
+    K = O.disc(N)
+    Rs = inp["R"] * scale
+    rng = np.random.default_rng(N)
+    lags = rng.integers([0, -N + 1, -N + 1], N, size=(300, 3))
+    h = O.ctf_weights(N, K, inp["groups"], inp["group_id"])
+    want = O.kernel_at(Rs, h, K, N, lags).real
+    rec = F.Reconstructor(N, 5, groups=inp["groups"], lam=1e-3)
+    rec.kernel(torch.from_numpy(Rs.reshape(5, 9)).cuda(), torch.from_numpy(inp["group_id"]).cuda())
+    ker = torch.empty(rec.half_shape(), device="cuda")
+    rec.copy_out(F._lib.FIRM_OUT_KER, ker)
+    got = ker.cpu().numpy()[lags[:, 2] + N, lags[:, 1] + N, lags[:, 0]]
+    print(f"N={N} x{scale}: {rel(got, want):.2e}")
+    assert rel(got, want) <= 1e-3
+    rec.close()
