@@ -198,7 +198,9 @@ size_t layout_workspace(const firm_params& p, char* base, Workspace& w) {
     const size_t slots_k = mma_k ? mma_slots(M * nH, nb_k) : 0;
     const size_t slots_r = mma_rule(p, M * nH, nb_r, 2) ? mma_slots(M * nH, nb_r) : 0;
     const size_t rec_words = std::max(slots_k * (fused ? 6 : 4), slots_r * 5);
-    const size_t pts_bytes = (slots_k || slots_r) ? M * nH * (sizeof(uint4) + sizeof(float2)) : 0;
+    // points: 16 B, and with A*b the imaginary part, or fused both parts of its weight
+    const size_t pts_each = sizeof(uint4) + (fused ? sizeof(float2) : slots_r ? sizeof(float) : 0);
+    const size_t pts_bytes = (slots_k || slots_r) ? M * nH * pts_each : 0;
     const size_t in_bytes = std::max(pay_bytes, (pts_bytes + 255) & ~(size_t)255);
     const size_t rec_bytes = (rec_words * sizeof(uint32_t) + 255) & ~(size_t)255;
     const size_t u_bytes = std::max({M * N * N * esz, in_bytes + rec_bytes + std::max(slots_k, slots_r) / 16,

@@ -493,17 +493,22 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 // (binning and spreading together).  Its cost per brick is high -- 25 or 27 classes padded
 // to 16 points, each flushed to the region -- and its cost per point low, the lower the
 // more channels share the window arithmetic.  Measured at N = 64, in ms, bank-class form
-// against tensor-core form.  W = 6: kernel channel 0.65 / 0.76 at 282 points a brick,
-// 0.88 / 0.91 at 470, 1.30 / 1.20 at 846; A*b 0.158 / 0.154 at 226, 0.47 / 0.23 at 754;
-// both in one pass 0.83 / 1.00 at 94, 1.05 / 1.08 at 188, 1.32 / 1.16 at 282.  W = 7:
-// kernel channel 0.85 / 1.06 at 282, 4.64 / 4.46 at 622 (N = 96), 1.84 / 1.62 at 846;
-// A*b 0.21 / 0.24 at 226, 0.73 / 0.37 at 754.  Both channels in one pass at W = 7 would
-// need 96 accumulators a thread, and W = 8 windows leave one first tap a class: neither is
-// built.
+// against tensor-core form.  W = 6: kernel channel 0.70 / 0.77 at 375 points a brick,
+// 0.78 / 0.85 at 469, 1.01 / 0.99 at 657; A*b 0.158 / 0.154 at 226, 0.21 / 0.16 at 450,
+// 0.61 / 0.25 at 1,100; both in one pass 0.80 / 0.99 at 141, 0.91 / 1.02 at 188, 1.22 / 1.11
+// at 281.  W = 7: kernel channel 0.93 / 1.08 at 375, 1.24 / 1.28 at 562, 1.77 / 1.53 at 844;
+// A*b 0.12 / 0.17 at 112, 0.19 / 0.19 at 225, 0.31 / 0.24 at 450.  Both channels in one pass
+// at W = 7 would need 96 accumulators a thread, and W = 8 windows leave one first tap a
+// class: neither is built.
+// The points and their records take up to 48 bytes a point where ids take 15.  At W = 7 (1.1 to
+// 1.6 times the bank-class form's rate, 2 at W = 6) that is taken up to 4 GiB, which keeps the
+// workspace of any plan of up to 50,000 images below 10 GiB.  By the plan's number of images,
+// not the call's: a plan laid out without records never takes a call that needs them.
+constexpr double kMmaMostW7 = 4.294967296e9 / 48;
 bool mma_rule(const firm_params& p, size_t points, int nb, int ch) {
     double least;
-    if (p.W == 6) least = ch == 1 ? 500.0 : ch == 2 ? 220.0 : 200.0;
-    else if (p.W == 7 && ch < 3) least = ch == 1 ? 560.0 : 280.0;
+    if (p.W == 6) least = ch == 1 ? 600.0 : ch == 2 ? 220.0 : 235.0;
+    else if (p.W == 7 && ch < 3 && (double)p.M * p.N * p.N * 0.3927 <= kMmaMostW7) least = ch == 1 ? 600.0 : 230.0;
     else return false;
     return (double)points >= least * 0.5236 * nb * nb * (double)nb;
 }
