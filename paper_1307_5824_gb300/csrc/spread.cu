@@ -8,14 +8,16 @@
 // two rows of R_m.
 //
 // Pipeline per channel (kernel: weights h^2 on G = 4N; right-hand side: weights
-// h b on G = 2N):
-//   1. bin:    count points per 8^3 brick (warp-aggregated atomics), scan, scatter
-//              point ids into per-brick segments cut into work items of at most
-//              `chunk` points, and order each item round-robin over bank classes.
-//   2. spread: persistent CTAs take work items; each accumulates its points into an
-//              (8 + W)^3 shared-memory region in int32 fixed point (native shared
-//              atomics), folds it into FP32 every 512 or 1024 points, then adds the region
-//              into the FP64 global grid with FP64 atomics.
+// h b on G = 2N; or both at once on G = 4N):
+//   1. bin:    count points per 8^3 brick (warp-aggregated atomics), scan, and place the
+//              points in per-brick segments cut into work items.
+//   2. spread, in one of two forms by the points per brick (mma_rule):
+//      - bank classes (few): point ids, every item ordered round-robin over the bank
+//        classes; persistent CTAs accumulate an item into an (8 + W)^3 shared-memory
+//        region in int32 fixed point (one native shared atomic per tap), fold it into
+//        FP32 every 512 or 1024 points, and add the region into the FP64 global grid.
+//      - tensor cores (many; spread_mma.cu): coordinates and weights placed instead of
+//        ids, sorted by cell class, contracted by warps.
 // The forward projector's interpolation (k_interp, at the end of this file) is the
 // transpose of step 2 on the same binning: a CTA stages its brick's region of the
 // transformed grid and gathers the W^3 taps of each point, with no atomics.
@@ -92,8 +94,7 @@ struct BinArgs {
 
 template <int W, bool SCATTER, bool KC>
 __global__ void __launch_bounds__(256) k_bin(BinArgs a, int M) {
-    pdl_wait();
-    pdl_launch();
+    pdl_wait();                            // no pdl_launch: 0.19 ms of 1.3 over 1.3e6 blocks
     constexpr int BZ = Brick<KC>::BZ;
     // x: samples t of one image (consecutive lanes walk a column of the half disc);
     // y: images.  Runs of equal bricks among consecutive lanes are aggregated.
@@ -140,6 +141,11 @@ __global__ void __launch_bounds__(256) k_bin(BinArgs a, int M) {
 // CH > 0 (1 kernel channel, 2 A*b, 3 both): the tensor-core form, whose points are placed
 // as coordinates and weights instead of ids: an image's geometry is the same for the
 // whole warp here, where the sort that follows would have to look it up per point.
+// Images that a warp of the scatter takes at a time: their cursor atomics, whose returns it
+// waits for, are in flight together (ids at N = 128, 15,000 images: 0.06 ms less than one by
+// one; three or four gain nothing more).
+constexpr int kScatterImages = 2;
+
 template <int W, bool KC, int CH>
 __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN, const int4* __restrict__ col,
                                                        int tiles_x, int n_tiles) {
@@ -158,8 +164,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN,
     }
     const bool valid = t >= 0;
     const int32_t kk = (int32_t)((uint32_t)(k1 & 0xffff) | ((uint32_t)k2 << 16));
-    // U images at a time: their cursor atomics are in flight together
-    constexpr int U = CH > 0 ? 2 : 1;
+    constexpr int U = kScatterImages;
     for (int m0 = blockIdx.y * U; m0 < M; m0 += gridDim.y * U) {
         int key[U], c[U];
         uint4 pt[U];
@@ -474,7 +479,7 @@ static void bin_count_w(Plan& P, const BinArgs& a, int M, bool kc) {
 template <int W>
 static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
     const int hN = P.N / 2, tiles_x = (hN + 1 + 3) / 4, n_tiles = tiles_x * ((P.N + 1 + 7) / 8);
-    const int mb = P.bin_mma ? (M + 1) / 2 : M;
+    const int mb = (M + kScatterImages - 1) / kScatterImages;
     const dim3 g((n_tiles + 7) / 8, (unsigned)(mb < 65535 ? mb : 65535));
     const int4* col = P.ws.colinfo;
     const bool sm = a.samples != nullptr;
@@ -1021,8 +1026,6 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
 
 template <int W>
 __global__ void __launch_bounds__(kFusedThreads) k_spread_fused(const SpreadArgs a) {
-    pdl_wait();
-    pdl_launch();
     constexpr int R3 = (kBrick + W) * (kBrick + W) * (kBrickZk + W);
     extern __shared__ int sm_i[];
     int* lev1 = sm_i;                                          // 3 * R3 int32
@@ -1087,7 +1090,7 @@ static cudaError_t spread_fused_w(Plan& P, const SpreadArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_fused<W>, kFusedThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    launch_pdl(k_spread_fused<W>, P.num_sms * per_sm, kFusedThreads, smem, P.stream, a);
+    k_spread_fused<W><<<P.num_sms * per_sm, kFusedThreads, smem, P.stream>>>(a);      // as k_interp
     P.launches += 1;
     return cudaGetLastError();
 }
@@ -1271,8 +1274,6 @@ struct InterpArgs {
 
 template <int W, bool RESID>
 __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
-    pdl_wait();
-    pdl_launch();
     constexpr int BZ = kBrick;
     constexpr int RG = kBrick + W;
     constexpr int RG3 = RG * RG * (BZ + W);
@@ -1412,7 +1413,9 @@ static cudaError_t interp_w(Plan& P, const InterpArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp<W, RESID>, kSpreadThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    launch_pdl(k_interp<W, RESID>, P.num_sms * per_sm, kSpreadThreads, smem, P.stream, a);
+    // an ordinary launch: blocks placed early sit beside the class sort's under its shared-memory
+    // split, fewer per SM (data term at N = 128, 15,000 images 11.2 ms, 10.3 this way)
+    k_interp<W, RESID><<<P.num_sms * per_sm, kSpreadThreads, smem, P.stream>>>(a);
     P.launches += 1;
     return cudaGetLastError();
 }
