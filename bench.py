@@ -89,7 +89,7 @@ def parse():
     ap.add_argument("--channels", default="fused", choices=["fused", "separate"],
                     help="separate: firm_kernel then firm_backproject (the image upload of the end-to-end step "
                          "hides behind the whole kernel channel); fused: one binning and one spreading pass for Ker "
-                         "and A*b (firm_kernel_backproject; only the binning can hide the upload).  The other form "
+                         "and A*b (firm_kernel_backproject; only the counting of the points can hide the upload).  The other form "
                          "is timed beside it either way")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-cpu", action="store_true")
@@ -752,7 +752,7 @@ def main():
 
         # both channel forms, each with the upload staged ahead and in stream order,
         # alternating step by step (the same drift for all four); the staged upload
-        # overlaps the binning (fused) or the whole kernel channel (separate)
+        # overlaps the counting of the points (fused) or the whole kernel channel (separate)
         n_e2e = max(args.steps, 5)
         variants = [(f, staged) for f in (fused, not fused) for staged in (False, True)]
         res = {v: 0.0 for v in variants}
@@ -782,7 +782,7 @@ def main():
         name = lambda f: "fused" if f else "separate"
         e2e = {"value": res[(best, True)], "unit": "s/recon", "h2d_bytes_per_step": int(h2d),
                "d2h_bytes_per_step": int(x_h.numel() * 4), "form": name(best) + " channels",
-               "upload": "staged ahead (firm_stage_images), overlapped with the binning" if best else
+               "upload": "staged ahead (firm_stage_images), overlapped with the counting of the points" if best else
                          "staged ahead (firm_stage_images), overlapped with the kernel channel",
                "value_serial_upload": res[(best, False)],
                "by_form": {name(f) + ("_staged" if st else "_serial"): res[(f, st)] for f, st in variants}}
@@ -807,49 +807,70 @@ def main():
     pts = M * nK
     W = args.W
     nH = (nK + 1) // 2
-    # Spreading time of this form (the fused pass is stage 1; the separate channels are
-    # stages 1 and 6) and the roofline of the dominant kernel, the spreading pass.  Work
-    # unit: one shared-memory atomic add: W^3 per half-disc point for the kernel channel,
-    # 2 W^3 for A*b, 3 W^3 for the fused pass.  Peak: 152 SMs x 32 lanes x 2.07 GHz (one
-    # warp-wide shared atomic per clock per SM) = 10.07e12 / s.
+    # Spreading time of this form: the fused pass is stage 1, with the placement of its points
+    # (or, in the bank-class form, the gather of their weights) in stage 10; the separate
+    # channels are stages 1 and 6.
     spread_ms = stages["spread_ker"] + stages["spread_rhs"] + stages.get("gather_fused", 0.0)
 
+    def tensor_form(ch):
+        """Whether the spreading of channel form ch (1 Ker, 2 A*b, 3 both) runs on the tensor
+        cores: the library's rule on the points per brick of the ball (spread.cu, mma_rule)."""
+        least = {6: {1: 600, 2: 220, 3: 235}, 7: {1: 600, 2: 230}}.get(W, {}).get(ch)
+        bricks = 0.5236 * ((2 if ch == 2 else 4) * N / 8) ** 3
+        return least is not None and M * nH >= least * bricks
+
     def roofline_of(st, is_fused):
-        """Shared-atomic rate of the dominant spreading kernel of one channel form, with
-        its DRAM bytes per launch from an ncu capture of this workload (committed with
-        the hash of the spreading source it was taken on; null once that source changed)."""
+        """Rate of the dominant spreading kernel of one channel form.  Tensor-core form: the
+        products of its m16n8k16 instructions without padding (a group of 16 points: 64 x 8
+        cells, 3 products of the fp16 parts, at W = 6; 128 x 8 at W = 7) against the measured
+        mma.sync rate, 961 products per clock and SM.  Bank-class form: one shared-memory atomic
+        add per tap and channel against one warp-wide shared atomic per clock and SM (10.07e12
+        / s).  DRAM bytes per launch from an ncu capture of this workload (committed with the
+        hash of the spreading source it was taken on; null once that source changed)."""
         if is_fused:
-            dom, atoms, kname = "spread_ker", M * nH * W ** 3 * 3, f"k_spread_fused<{W}>"
+            dom, ch = "spread_ker", 3
         else:
             dom = "spread_rhs" if st["spread_rhs"] >= st["spread_ker"] else "spread_ker"
-            atoms = M * nH * W ** 3 * (2 if dom == "spread_rhs" else 1)
-            kname = f"k_spread<{W},{'complex' if dom == 'spread_rhs' else 'real'}>"
-        peak = 152 * 32 * 2.07e9
-        achieved = atoms / (st[dom] * 1e-3)
+            ch = 2 if dom == "spread_rhs" else 1
+        mma = tensor_form(ch)
+        if mma:
+            kname, src_file = f"k_spread_mma<{W},{ch}>", "spread_mma.cu"
+            peak = 152 * 961 * 2 * 2.07e9
+            achieved = M * nH * ch * 3 * (512 if W == 6 else 1024) * 2 / (st[dom] * 1e-3)
+            rate = {"bound": "tensor", "unit": "TFLOP/s",
+                    "peak_source": "measured: mma.sync m16n8k16 fp16, 961 products/clk/SM, x 152 SMs x 2.07 GHz"}
+        else:
+            kname = f"k_spread_fused<{W}>" if is_fused else f"k_spread<{W},{'complex' if ch == 2 else 'real'}>"
+            src_file = "spread.cu"
+            peak = 152 * 32 * 2.07e9
+            achieved = M * nH * W ** 3 * ch / (st[dom] * 1e-3)
+            rate = {"bound": "alu", "unit": "Tatomic/s",
+                    "peak_source": "derived: 152 SMs x 32 shared-atomic lanes/clk x 2.07 GHz"}
         traffic = None
         prof = os.path.join(ROOT, "profiles", "spread_traffic.json")
         if os.path.exists(prof) and (N, M, W) == (128, 50000, 6):   # the figure is for this workload
             try:
                 import hashlib
                 rec_t = json.load(open(prof)).get(kname) or {}
-                src = open(os.path.join(ROOT, "paper_1307_5824_gb300", "csrc", "spread.cu"), "rb").read()
+                src = open(os.path.join(ROOT, "paper_1307_5824_gb300", "csrc", src_file), "rb").read()
                 if rec_t.get("source_sha256") == hashlib.sha256(src).hexdigest():
                     traffic = rec_t.get("dram_bytes")
             except Exception:
                 traffic = None
-        return {"kernel": kname, "bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12,
-                "unit": "Tatomic/s", "frac": achieved / peak, "traffic": traffic,
-                "peak_source": "derived: 152 SMs x 32 shared-atomic lanes/clk x 2.07 GHz"}
+        return {"kernel": kname, "achieved": achieved / 1e12, "peak": peak / 1e12, "frac": achieved / peak,
+                "traffic": traffic, **rate}
 
     roofline = roofline_of(stages, fused)
     roofline_other = roofline_of(stages_other, not fused)
-    # the spreading pass against HBM (not its binding bound): algorithmic bytes = point ids
-    # and weights read + the FP64 fine grids written once
+    # the spreading against HBM (not its binding bound): algorithmic bytes = the points' ids or
+    # records and weights read, those that the timed stages write, and the FP64 fine grids
+    # written once.  A tensor-core record is 4 B per coordinate and 4 B per channel's weight.
     Gk, Gr = 4 * N, 2 * N
-    if fused:   # the weight gather (ids, weights by id, weights in payload order) + the pass
-        spread_bytes = M * nH * (4 + 8 + 8) + M * nH * (4 + 8) + 3 * Gk ** 3 * 8
+    if fused:   # the points placed, sorted into records and spread; or the weights gathered and spread
+        spread_bytes = M * nH * (4 * 24 if tensor_form(3) else (4 + 8 + 8) + (4 + 8)) + 3 * Gk ** 3 * 8
     else:
-        spread_bytes = M * nH * 4 + Gk ** 3 * 8 + M * nH * (4 + 8 + 2) + Gr ** 3 * 16
+        spread_bytes = (M * nH * ((16 if tensor_form(1) else 4) + (20 if tensor_form(2) else 4 + 8 + 2))
+                        + Gk ** 3 * 8 + Gr ** 3 * 16)
     hbm_peak = None
     try:
         hbm_peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"])
@@ -882,7 +903,7 @@ def main():
     cufft = cufft_comparison(rec, N, dev, stream, toep_s * 1e6, stages.get("fft_ker", 0.0))
     spread_hbm = {"algorithmic_bytes": int(spread_bytes), "achieved_gbs": spread_bytes / (spread_ms * 1e-3) / 1e9,
                   "hbm_frac": spread_bytes / (spread_ms * 1e-3) / 1e9 / hbm_peak, "peak_source": hbm_src,
-                  "note": "not the binding bound: the spreading is bound by shared-memory atomic issue"}
+                  "note": "not the binding bound: the spreading is bound by instruction issue (see roofline)"}
 
     # the forward projector A of the solution (type-2 NUFFT at every half-disc sample)
     # and the data term |b - A x|^2 / |b|^2, device buffers, CUDA events

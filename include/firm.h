@@ -152,11 +152,12 @@ int firm_backproject(firm_plan_t plan, int M, const void* images, const double* 
 /* FIRM steps 1-3 in one call, the two spreading channels fused (Section 3.4; eq.
  * measurement, eq. backprojection, eq. kernel, eq. embedding_circulant, eq. circ1).
  * Both sums run over the same slice points xi_{m,k} with the same window, so the
- * points are binned once on the 4N^3 grid (poses only: this runs while a staged image
- * upload, firm_stage_images, is still landing), the images are transformed to h b on
- * the disc, the h b of every point is gathered into the binning's order, and one
- * spreading pass adds h^2 phi to the Ker grid and h b phi to the A*b grid (complex,
- * 4N^3); Ker (on [-N, N)^3), K-hat, lam_eff and A*b (on N^3, from the
+ * points are binned once on the 4N^3 grid (poses only: their counting runs while a staged
+ * image upload, firm_stage_images, is still landing; where bricks hold few points, so does
+ * their placement), the images are transformed to h b on the disc, the points are placed
+ * with their weights (few points a brick: the h b of every point is gathered into the
+ * binning's order), and one spreading pass adds h^2 phi to the Ker grid and h b phi to the
+ * A*b grid (complex, 4N^3); Ker (on [-N, N)^3), K-hat, lam_eff and A*b (on N^3, from the
  * 4N grid: oversampling 4 for its N modes) follow as in firm_kernel and
  * firm_backproject, whose results it replaces.  Arguments as those two calls;
  * khat_out and rhs_out are nullable.  FIRM_EINVAL unless the plan was made with
@@ -408,7 +409,8 @@ int firm_bin_info(firm_plan_t plan, int* n_work, int* n_points, int* bricks_per_
  *   4 geometry + image DFT                  5 binning (A*b channel)
  *   6 spreading (A*b channel)               7 2N^3 transform + deconvolution (A*b)
  *   8 CG total                              9 CG iterations of the last solve
- *  10 the fused form's weight gather (firm_kernel_backproject; its spreading is slot 1)
+ *  10 the fused form's placement of the points with their weights, or its weight gather
+ *     (firm_kernel_backproject; its spreading is slot 1)
  * firm_stage_times waits for the recorded events and fills out[0..n-1]. */
 int firm_set_timing(firm_plan_t plan, int on);
 int firm_stage_times(firm_plan_t plan, double* out, int n);

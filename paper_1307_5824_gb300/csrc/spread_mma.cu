@@ -23,9 +23,9 @@
 // arithmetic is 12 and the fragments 14; the fp16 tensor pipe of mma.sync (measured 961
 // products per clock and SM) is a quarter busy.  mma.sync and not tcgen05, because both
 // operands are made by the threads that use them, already in registers.
-// Measured at N = 128, 50,000 images, W = 6 (3.2e8 points), sort and spread together
-// against bank-class sort, weight gather and spread: both channels 46.5 -> 23 ms, kernel
-// channel 19.5 -> 14 ms, A*b 27.7 -> 15 ms.
+// Measured at N = 128, 50,000 images, W = 6 (3.2e8 points), binning and spreading together
+// against the bank-class form (with its weight gather): both channels 50.8 -> 26.9 ms, of
+// which the contraction takes 15.1, kernel channel 23.8 -> 16.5 ms, A*b 34.0 -> 18.0 ms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
