@@ -815,7 +815,7 @@ def main():
     def tensor_form(ch):
         """Whether the spreading of channel form ch (1 Ker, 2 A*b, 3 both) runs on the tensor
         cores: the library's rule on the points per brick of the ball (spread.cu, mma_rule)."""
-        least = {6: {1: 600, 2: 220, 3: 235}, 7: {1: 600, 2: 230}}.get(W, {}).get(ch)
+        least = {6: {1: 600, 2: 400, 3: 235}, 7: {1: 600, 2: 400}}.get(W, {}).get(ch)
         bricks = 0.5236 * ((2 if ch == 2 else 4) * N / 8) ** 3
         return least is not None and M * nH >= least * bricks
 

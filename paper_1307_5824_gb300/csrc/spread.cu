@@ -502,7 +502,11 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 // 0.78 / 0.85 at 469, 1.01 / 0.99 at 657; A*b 0.158 / 0.154 at 226, 0.21 / 0.16 at 450,
 // 0.61 / 0.25 at 1,100; both in one pass 0.80 / 0.99 at 141, 0.91 / 1.02 at 188, 1.22 / 1.11
 // at 281.  W = 7: kernel channel 0.93 / 1.08 at 375, 1.24 / 1.28 at 562, 1.77 / 1.53 at 844;
-// A*b 0.12 / 0.17 at 112, 0.19 / 0.19 at 225, 0.31 / 0.24 at 450.  Both channels in one pass
+// A*b 0.12 / 0.17 at 112, 0.19 / 0.19 at 225, 0.31 / 0.24 at 450.  A*b alone
+// stays in the bank-class form up to 400: the two are level near 225, and the few hundred
+// images of such bricks leave A*A so ill-conditioned without lambda that its white rounding
+// errors keep the CG volume nearer to the exact one (N = 32, 200 images, 10 iterations: median
+// 4e-5, 1e-4 in the tensor-core form, at equal errors of A*b).  Both channels in one pass
 // at W = 7 would need 96 accumulators a thread, and W = 8 windows leave one first tap a
 // class: neither is built.
 // The points and their records take up to 48 bytes a point where ids take 15.  At W = 7 (1.1 to
@@ -512,8 +516,8 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 constexpr double kMmaMostW7 = 4.294967296e9 / 48;
 bool mma_rule(const firm_params& p, size_t points, int nb, int ch) {
     double least;
-    if (p.W == 6) least = ch == 1 ? 600.0 : ch == 2 ? 220.0 : 235.0;
-    else if (p.W == 7 && ch < 3 && (double)p.M * p.N * p.N * 0.3927 <= kMmaMostW7) least = ch == 1 ? 600.0 : 230.0;
+    if (p.W == 6) least = ch == 1 ? 600.0 : ch == 2 ? 400.0 : 235.0;
+    else if (p.W == 7 && ch < 3 && (double)p.M * p.N * p.N * 0.3927 <= kMmaMostW7) least = ch == 1 ? 600.0 : 400.0;
     else return false;
     return (double)points >= least * 0.5236 * nb * nb * (double)nb;
 }

@@ -23,7 +23,7 @@ def rel(a, b):
 
 
 @pytest.mark.parametrize("N,M,cfg,fused,W", [
-    (16, 118, "C2", False, 6), (16, 1641, "C5", False, 6), (16, 6001, "C3", False, 6), (32, 3301, "C5", False, 6),
+    (16, 141, "C2", False, 6), (16, 1641, "C5", False, 6), (16, 6001, "C3", False, 6), (32, 3301, "C5", False, 6),
     (16, 641, "C3", True, 6), (16, 2003, "C5", True, 6), (32, 1301, "C2", True, 6),
     (16, 1641, "C5", False, 7), (16, 6001, "C3", False, 7), (32, 1001, "C2", False, 7)])
 def test_tensor_core_spreading_matches_oracle(N, M, cfg, fused, W):
