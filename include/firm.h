@@ -16,8 +16,9 @@
  *   - Images are M x N x N, [m][i2][i1], float32 or bfloat16 (firm_params.img_dtype),
  *     starting at a 16-byte aligned address (each image is moved into shared memory by
  *     one bulk copy); a misaligned image array is rejected with FIRM_EINVAL.
- *   - R is M x 9 float64, each rotation row-major (columns of its first two rows longer
- *     than 1.3, which no rotation has, may be dropped).  The slice of image m samples
+ *   - R is M x 9 float64, each rotation row-major.  Columns (R_1d, R_2d) of its first two
+ *     rows, of length at most 1 in a rotation, are taken below 3; a longer or NaN one is
+ *     reported as FIRM_EINVAL in the way of FIRM_EINTERNAL.  The slice of image m samples
  *     the points xi = R_m^T (2 pi k1 / N, 2 pi k2 / N, 0) for |k| <= N/2
  *     (eq. forward-projector, eq. truncation: the symmetric disc).
  *   - shifts is M x 2 float64 (x, y) in pixels; the samples of image m are

@@ -331,8 +331,8 @@ struct StageTimer {
         if ((x) != cudaSuccess) { return FIRM_ECUDA; } \
     } while (0)
 
-// The spreading and interpolation kernels set counters[2] when a binned point falls
-// outside its brick (an internal invariant; never expected).  Entry points do not wait
+// Kernels set counters[2] when a binned point falls outside its brick (an internal
+// invariant; never expected) or an input cannot be used.  Entry points do not wait
 // for it: it is read, and cleared, where the host waits for the stream anyway (a host
 // output, the end of a CG solve, a query of device scalars).
 static int take_device_flag(Plan& P) {
@@ -341,7 +341,7 @@ static int take_device_flag(Plan& P) {
     FIRM_CK(cudaStreamSynchronize(P.stream));
     if (!flag) return FIRM_OK;
     FIRM_CK(cudaMemsetAsync(P.ws.counters + 2, 0, sizeof(int), P.stream));
-    return FIRM_EINTERNAL;
+    return flag_status(flag);
 }
 
 // An output to dst: device memory is written in stream order; host memory waits for
@@ -628,8 +628,7 @@ int firm_kernel(firm_plan_t plan, int M, const double* R, const int32_t* group, 
     FIRM_CK(start_stage(P));                   // a staged image upload runs beside the kernel channel
     P.bin_M = -1;
     tm.start(0);
-    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
-    P.launches += M > 0 ? 1 : 0;
+    FIRM_CK(launch_geom(P, P.cur_R, M));
     FIRM_CK(launch_bin(P, M, true, BinFor::spread));
     tm.stop();
     tm.start(1);
@@ -683,8 +682,7 @@ int firm_backproject(firm_plan_t plan, int M, const void* images, const double* 
     }
     P.bin_M = -1;
     tm.start(4);
-    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
-    P.launches += M > 0 ? 1 : 0;
+    FIRM_CK(launch_geom(P, P.cur_R, M));
     FIRM_CK(launch_image_dft(P, M, P.cur_images, P.cur_shifts, P.cur_gid));
     if (from_stage) FIRM_CK(cudaEventRecord(P.ev_stage_read, P.stream));   // staging free again
     tm.stop();
@@ -725,8 +723,7 @@ int firm_kernel_backproject(firm_plan_t plan, int M, const void* images, const d
     const bool host_copy = M > 0 && !staged && !is_device(images);
     if (staged) FIRM_CK(start_stage(P));
     P.bin_M = -1;
-    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
-    P.launches += M > 0 ? 1 : 0;
+    FIRM_CK(launch_geom(P, P.cur_R, M));
     tm.start(0);
     FIRM_CK(launch_bin_count(P, M, 3, BinFor::spread));
     const bool place_first = !host_copy && !P.bin_mma;
@@ -844,8 +841,7 @@ int firm_forward(firm_plan_t plan, int M, const float* V, const double* R, const
     if (M == 0) return FIRM_OK;
     const float* Vd = nullptr;
     FIRM_CK(stage_forward_inputs(P, M, V, R, group, Vd));
-    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
-    P.launches += 1;
+    FIRM_CK(launch_geom(P, P.cur_R, M));
     FIRM_CK(launch_bin(P, M, false, BinFor::interp));
     float2* ghat = reinterpret_cast<float2*>(w.grid);
     FIRM_CK(launch_fwd_transform(P, Vd, ghat));
@@ -880,8 +876,7 @@ int firm_data_residual(firm_plan_t plan, int M, const float* V, const void* imag
         FIRM_CK(cudaMemcpyAsync(w.images, images, (size_t)M * P.N * P.N * esz, cudaMemcpyHostToDevice, P.stream));
         img = w.images;
     }
-    FIRM_CK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
-    P.launches += 1;
+    FIRM_CK(launch_geom(P, P.cur_R, M));
     FIRM_CK(launch_image_dft(P, M, img, sh, P.cur_gid, true));    // b itself into samples
     FIRM_CK(launch_bin(P, M, false, BinFor::interp));                                // b copied in scatter order
     float2* ghat = reinterpret_cast<float2*>(w.grid);
@@ -1171,8 +1166,7 @@ int firm_bin(firm_plan_t plan, int M, const double* R, int channel) {
     cudaError_t e = cudaSuccess;
     const double* Rd = stage(R, w.R, (size_t)M * 9, P.stream, e);
     FIRM_CK(e);
-    FIRM_CK(launch_geom(Rd, M, P.N, w.geom, P.stream));
-    P.launches += M > 0 ? 1 : 0;
+    FIRM_CK(launch_geom(P, Rd, M));
     FIRM_CK(launch_bin(P, M, channel == 0, BinFor::inspect));
     P.bin_M = M;
     P.bin_kc = channel == 0;

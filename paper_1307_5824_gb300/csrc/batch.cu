@@ -128,8 +128,7 @@ cudaError_t plan_front(Plan& P, const firm_batch_item& it, bool spread_here) {
     if (it.shifts) P.cur_shifts = it.shifts;
     else { BCK(cudaMemsetAsync(w.shifts, 0, sizeof(double) * 2 * (M > 0 ? M : 1), P.stream)); P.cur_shifts = w.shifts; }
     BCK(cudaMemsetAsync(w.counters + 2, 0, sizeof(int), P.stream));
-    BCK(launch_geom(P.cur_R, M, P.N, w.geom, P.stream));
-    P.launches += M > 0 ? 1 : 0;
+    BCK(launch_geom(P, P.cur_R, M));
     BCK(launch_bin(P, M, true, BinFor::spread));
     BCK(launch_spread_clear(P, true));
     if (spread_here) BCK(launch_spread_only(P, M, true));
@@ -628,7 +627,7 @@ int firm_batch_wait(firm_batch_t b, int* status, int* iters) {
             cudaMemcpy(&flag, P.ws.counters + 2, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
             return FIRM_ECUDA;
         if (flag && cudaMemset(P.ws.counters + 2, 0, sizeof(int)) != cudaSuccess) return FIRM_ECUDA;
-        int sti = flag ? FIRM_EINTERNAL : s.status;
+        int sti = flag ? flag_status(flag) : s.status;
         if (sti == FIRM_OK && b->last_tol > 0.0 && !(s.rr >= 0.0 && std::sqrt(s.rr) <= s.tol)) sti = FIRM_ENOTCONV;
         P.have_kernel = P.have_rhs = true;
         P.pc_ready = false;

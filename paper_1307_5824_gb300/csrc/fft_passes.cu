@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kThreads) k_image_dft(const ImgArgs a) {
     if (threadIdx.x == 0)
         bulk_g2s(const_cast<T*>(img), reinterpret_cast<const T*>(a.images) + img0, kImgBytes, &s_bar);
     if (!mbar_wait(&s_bar, 0)) {
-        if (threadIdx.x == 0) atomicOr(a.err, 4);
+        if (threadIdx.x == 0) atomicOr(a.err, kFlagCopy);
         mbar_wait(&s_bar, 0);                      // the copy in flight, then leave
         return;
     }

@@ -42,6 +42,14 @@ struct __align__(16) ImgGeom {
     int32_t uh[3], vh[3], ul[3], vl[3];
 };
 constexpr int kGeomBits = 41;
+constexpr int kGeomWide = 1 << 16;    // in ul[0], above the low part: positions of this image need 64 bits
+
+// Bits of the device flag, counters[2]: an internal invariant (a point outside its brick, an
+// image copy that did not land), or an input that cannot be used (a matrix beyond the limit).
+constexpr int kFlagPoint = 1, kFlagCopy = 4, kFlagInput = 8;
+inline int flag_status(int flag) {
+    return flag & (kFlagPoint | kFlagCopy) ? FIRM_EINTERNAL : flag ? FIRM_EINVAL : FIRM_OK;
+}
 
 // CG state on the device (FP64 scalars; Section 3.3).
 struct CgState {
@@ -196,7 +204,7 @@ double wavelength_A(double kV);
 double ctf_value(const firm_ctf_group& g, double r_invA);
 
 // ---- launchers (spread.cu) ----
-cudaError_t launch_geom(const double* R, int M, int N, ImgGeom* geom, cudaStream_t s);
+cudaError_t launch_geom(Plan& P, const double* R, int M);
 // Binning in two steps: the count of points per brick and the work items (poses only),
 // then the points in the items' order.  ch: 1 kernel channel, 2 A*b, 3 both on the 4N
 // grid.  Points to be spread are ordered for the tensor-core form where spread_uses_mma

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kFeatThreads) k_pc_features(const ImgGeom* __r
         const ImgGeom g = geom[m];
         constexpr float unit = 1.0f / (float)(1ll << kGeomBits);
         auto f = [](int h, int l) { return __ll2float_rn(((long long)h << 16) + l) * unit; };
-        const float ua = f(g.uh[0], g.ul[0]) * a1 + f(g.uh[1], g.ul[1]) * a2 + f(g.uh[2], g.ul[2]) * a3;
+        const float ua = f(g.uh[0], g.ul[0] & 0xffff) * a1 + f(g.uh[1], g.ul[1]) * a2 + f(g.uh[2], g.ul[2]) * a3;
         const float va = f(g.vh[0], g.vl[0]) * a1 + f(g.vh[1], g.vl[1]) * a2 + f(g.vh[2], g.vl[2]) * a3;
         const float* h2g = h2 + (size_t)min(max(gid[m], 0), n_ctf - 1) * nH;
         for (int t = t0 + q; t < t1; t += kFeatThreads / kFeatImgs) {

@@ -35,20 +35,27 @@ namespace firm {
 // ---------------------------------------------------------------------------
 // Geometry
 // ---------------------------------------------------------------------------
-// Pairs (R_1d, R_2d) longer than `longest` are dropped (NaN too), so that no point leaves the
-// bricks.  Rotations have at most 1; scaled matrices are taken up to 2.9 (one wrap of the grid)
-// where 4N divides the 512 cells of a 32-bit position, else up to its +-256 cells: 2.66, 1.59
-// and 1.33 at N = 48, 80 and 96.
-__global__ void k_geom(const double* __restrict__ R, int M, double longest, ImgGeom* __restrict__ g) {
+// Rotations have pairs (R_1d, R_2d) of length at most 1; scaled matrices are taken below 3, where
+// one wrap of the grid brings every sample back (point_pos).  A matrix with a longer pair or a
+// NaN is put on the origin, so that no point leaves the bricks, and reported.
+// wide: the length beyond which positions need 64 bits (axis_pos).
+__global__ void k_geom(const double* __restrict__ R, int M, double wide, ImgGeom* __restrict__ g, int* err) {
     pdl_wait();
     pdl_launch();
     int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
     const double* r = R + 9 * (size_t)m;
     ImgGeom o;
+    bool ok = true, in32 = true;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const bool ok = r[d] * r[d] + r[3 + d] * r[3 + d] <= longest * longest;
+        const double len2 = r[d] * r[d] + r[3 + d] * r[3 + d];
+        ok = ok && len2 <= 9.0 * (1.0 - 1e-9);
+        in32 = in32 && len2 <= wide * wide;
+    }
+    if (!ok) atomicOr(err, kFlagInput);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
         const long long u = ok ? __double2ll_rn(r[d] * (double)(1ll << kGeomBits)) : 0;
         const long long v = ok ? __double2ll_rn(r[3 + d] * (double)(1ll << kGeomBits)) : 0;
         o.uh[d] = (int)(u >> 16);
@@ -56,13 +63,15 @@ __global__ void k_geom(const double* __restrict__ R, int M, double longest, ImgG
         o.vh[d] = (int)(v >> 16);
         o.vl[d] = (int)(v & 0xffff);
     }
+    if (!in32) o.ul[0] |= kGeomWide;
     g[m] = o;
 }
 
-cudaError_t launch_geom(const double* R, int M, int N, ImgGeom* geom, cudaStream_t s) {
+cudaError_t launch_geom(Plan& P, const double* R, int M) {
     if (M <= 0) return cudaSuccess;
-    const double longest = 512 % (4 * N) == 0 ? 2.9 : std::min(2.9, 127.8 / N);
-    launch_pdl(k_geom, (M + 255) / 256, 256, 0, s, R, M, longest, geom);
+    const double wide = 512 % P.Gk == 0 ? 3.0 : 127.8 / P.N;      // 2.66, 1.59 and 1.33 at N = 48, 80, 96
+    launch_pdl(k_geom, (M + 255) / 256, 256, 0, P.stream, R, M, wide, P.ws.geom, P.ws.counters + 2);
+    P.launches += 1;
     return cudaGetLastError();
 }
 
@@ -738,7 +747,7 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
                 p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.ls, a.halfG,
                               a.G);
                 base = region_base<W, BZ>(p, lo0, lo1, lo2);
-                if (base < 0) atomicOr(&a.counters[2], 1);   // point outside its brick: reported, never written
+                if (base < 0) atomicOr(&a.counters[2], kFlagPoint);   // point outside its brick: reported, never written
             }
             // rank among the lanes of this step with the same bank class (base mod 32):
             // a point of rank s starts at window plane s (mod W), so points of one class
@@ -957,7 +966,7 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
                 p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.ls, a.halfG,
                               a.G);
                 base = region_base<W, BZ>(p, lo0, lo1, lo2);
-                if (base < 0) atomicOr(&a.counters[2], 1);   // point outside its brick: reported, never written
+                if (base < 0) atomicOr(&a.counters[2], kFlagPoint);   // point outside its brick: reported, never written
             }
             // repeated bank classes in a warp step start at different window planes, as
             // in spread_piece
@@ -1322,7 +1331,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
             const PointPos p = point_pos(a.geom[m], __ldg(&a.htab[t]), a.ls, a.halfG, a.G);
             const int base = region_base<W, BZ>(p, lo0, lo1, lo2);
             if (base < 0) {
-                atomicOr(&a.counters[2], 1);   // point outside its brick: reported, never read
+                atomicOr(&a.counters[2], kFlagPoint);   // point outside its brick: reported, never read
                 continue;
             }
             float wx[W], wy[W], wz[W];

@@ -10,14 +10,18 @@ namespace firm {
 
 // Position of sample k of an image along one axis of the fine grid, relative to the grid's
 // centre, (G/N)(k1 u + k2 v) in units of 2^-23 cells rounded to nearest (6e-8 cells, below
-// the FP32 rounding of the taps formed from it), modulo 512 cells.  Integer arithmetic
-// only: every kernel that calls this (binning, spreading, interpolation) gets identical
-// cells.  ls = log2(G / N) <= 2; exact, since u = uh 2^16 + ul to the last bit.
+// the FP32 rounding of the taps formed from it).  Integer arithmetic only: every kernel that
+// calls this (binning, spreading, interpolation) gets identical cells.  ls = log2(G / N) <= 2;
+// exact, since u = uh 2^16 + ul to the last bit.  In 32 bits (T = unsigned) the sum wraps at 512
+// cells of the 4N grid (256 of the 2N grid): a multiple of the grid's period where G is a power
+// of two, and on the other grids out of reach of every rotation; longer matrices there
+// carry kGeomWide and take 64 bits.
 constexpr int kFracBits = 23;
-__device__ __forceinline__ int axis_pos(const ImgGeom& g, int d, int k1, int k2, int ls) {
-    const unsigned p = (unsigned)k1 * (unsigned)g.uh[d] + (unsigned)k2 * (unsigned)g.vh[d];   // wraps
-    const int q = k1 * g.ul[d] + k2 * g.vl[d] + (1 << (17 - ls));
-    return (int)(p + (unsigned)(q >> 16)) >> (2 - ls);
+template <class T>
+__device__ __forceinline__ T axis_pos(const ImgGeom& g, int d, int k1, int k2, int ls) {
+    const T p = (T)k1 * (T)g.uh[d] + (T)k2 * (T)g.vh[d];
+    const int q = k1 * (d == 0 ? g.ul[0] & 0xffff : g.ul[d]) + k2 * g.vl[d] + (1 << (17 - ls));
+    return p + (T)(q >> 16);
 }
 
 // A cell I in [0, G) (periodic) and a fraction of q / 2^23 cells per axis.
@@ -32,15 +36,22 @@ __device__ __forceinline__ PointPos point_pos(const ImgGeom& g, int32_t kk, int 
     PointPos p;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const int t = axis_pos(g, d, k1, k2, ls);
+        const int t = (int)axis_pos<unsigned>(g, d, k1, k2, ls) >> (2 - ls);
+        p.I[d] = (t >> kFracBits) + halfG;
+        p.q[d] = (uint32_t)t & ((1u << kFracBits) - 1u);
+    }
+    if (g.ul[0] & kGeomWide) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            p.I[d] = (int)(axis_pos<long long>(g, d, k1, k2, ls) >> (2 - ls + kFracBits)) + halfG;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
         // |k1 u + k2 v| <= |k| <= N/2 (u, v: parts of a unit column of R) puts the cell in
         // [-1, G], and k_geom keeps longer ones within [-G, 2G): one wrap either way is the
         // periodic index
-        int I = (t >> kFracBits) + halfG;
-        if (I >= G) I -= G;
-        else if (I < 0) I += G;
-        p.I[d] = I;
-        p.q[d] = (uint32_t)t & ((1u << kFracBits) - 1u);
+        if (p.I[d] >= G) p.I[d] -= G;
+        else if (p.I[d] < 0) p.I[d] += G;
     }
     return p;
 }

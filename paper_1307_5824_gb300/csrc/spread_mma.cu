@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
             pt[u].z -= (k[2] * BASES) << 28;
             cr[u] |= atomicAdd(&s_hist[cr[u]], 1) << 8;
         }
-        if (!in) atomicOr(&a.counters[2], 1);      // a point outside its brick: never expected, reported
+        if (!in) atomicOr(&a.counters[2], kFlagPoint);      // a point outside its brick: never expected, reported
         if (CH >= 2) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) wmax = fmaxf(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
         }
         const int base = s_base;
         if (tid == 0) {
-            if (!fits) atomicOr(&a.counters[2], 1);
+            if (!fits) atomicOr(&a.counters[2], kFlagPoint);
             a.rec_item[item] = make_int4(wk.x, base, fits ? total / 16 : 0, lgn | (ek + 128) << 8 | (eb + 128) << 16);
         }
         __syncthreads();
