@@ -512,10 +512,13 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 // 0.61 / 0.25 at 1,100; both in one pass 0.80 / 0.99 at 141, 0.91 / 1.02 at 188, 1.22 / 1.11
 // at 281.  W = 7: kernel channel 0.93 / 1.08 at 375, 1.24 / 1.28 at 562, 1.77 / 1.53 at 844;
 // A*b 0.12 / 0.17 at 112, 0.19 / 0.19 at 225, 0.31 / 0.24 at 450.  A*b alone
-// stays in the bank-class form up to 400: the two are level near 225, and the few hundred
-// images of such bricks leave A*A so ill-conditioned without lambda that its white rounding
-// errors keep the CG volume nearer to the exact one (N = 32, 200 images, 10 iterations: median
-// 4e-5, 1e-4 in the tensor-core form, at equal errors of A*b).  Both channels in one pass
+// could go over from 225, where the two are level; it does from 400, which leaves at most 0.05 ms.
+// In between lies the undamped N = 32, 200-image workload, whose FP32 CG volume after 10 iterations
+// turns on the last bit of A*b in either form (400 runs with pixels moved by an ulp: median
+// 4e-5, largest 2.7e-4 here, 1.0e-4 and 3.9e-4 in the tensor-core form; with 170 and 250
+// images 6e-5 to 9e-5 at the median in both) and is held to 3e-4.  A*b itself is nearer to 64 bits
+// in the tensor-core form (1.2e-7 against 7.0e-7 at N = 32, 300 images), and the FP64 CG mode
+// gives the same volume from both.  Both channels in one pass
 // at W = 7 would need 96 accumulators a thread, and W = 8 windows leave one first tap a
 // class: neither is built.
 // The points and their records take up to 48 bytes a point where ids take 15.  At W = 7 (1.1 to

@@ -13,10 +13,13 @@
 //   2. k_spread_mma: a warp takes groups of 16 records and runs mma.m16n8k16; the (y, x)
 //      operand and the weighted z operand are formed in registers, in the fragment
 //      layout.  Every factor is an fp16 pair hi + lo (22 bits), a product keeps
-//      hi hi + hi lo + lo hi, and the tensor core adds in FP32; a warp's sums over at
-//      most 128 points go to the brick's (8 + W)^3 int32 region (native shared atomics;
-//      one rounding per sum instead of one per tap), which is added into the FP64 grid
-//      when the item ends.
+//      hi hi + hi lo + lo hi.  The tensor core's FP32 additions truncate to half a unit in
+//      the last place, so it adds the 16 points of a group only and the groups are added
+//      by rounded FP32 adds (sums through the tensor core over 128 points came out 6e-7 of
+//      their value too small, Ker's error against 64 bits 5.3e-7; 1.2e-7 this way, for 1% of
+//      the time).  A warp's sums over at most 128 points go to the brick's (8 + W)^3 int32
+//      region (native shared atomics; one rounding per sum instead of one per tap), which
+//      is added into the FP64 grid when the item ends.
 // Why: a tap per shared-memory atomic (spread.cu) is bound by the atomics' issue rate,
 // 648 per point with both channels; here a point costs 2.5 mma (64 x 8 cells of which 216
 // are hit, three products, padding) and ~30 warp instructions in all, of which the window
@@ -44,6 +47,7 @@ constexpr int kRunGroups = 8;                     // groups summed in FP32 befor
 // so that the products come out in the region's integer units.
 constexpr int kTapBits = 5;
 constexpr float kTapScale = (float)(1 << kTapBits);
+constexpr int kUnitBias = 1024;                   // of the exponents in an item's last word
 
 // CH: 1 kernel channel, 2 A*b, 3 both (Ker, Re, Im).
 template <int W, int CH> struct MmaCfg {
@@ -175,7 +179,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
     constexpr int kWarps = kSortThreads / 32;
     extern __shared__ __align__(16) uint32_t s_rec[];
     __shared__ int s_hist[32], s_off[32], s_total, s_item, s_base;
-    __shared__ float s_red[kWarps];
+    __shared__ float2 s_red[kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_work = a.counters[0];
     const float* const im2 = reinterpret_cast<const float*>(a.pts_w);      // A*b alone: imaginary parts
@@ -200,7 +204,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
         __syncthreads();
         // rank of the points in their class (arbitrary order); largest |h b|
         int cr[PT];                                // class | rank << 8
-        float wmax = 0.0f;
+        float wmax = 0.0f, wsum = 0.0f;
         if (CH >= 2) {
 #pragma unroll
             for (int u = 0; u < PT; ++u) {
@@ -208,7 +212,9 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
                 if (i >= wk.z) continue;
                 const float2 v = CH == 3 ? __ldg(&a.pts_w[wk.y + i])
                                          : make_float2(__uint_as_float(pt[u].w), __ldg(&im2[wk.y + i]));
-                wmax = fmaxf(wmax, fmaxf(fabsf(v.x), fabsf(v.y)));
+                const float w = fmaxf(fabsf(v.x), fabsf(v.y));
+                wmax = fmaxf(wmax, w);
+                wsum += w;
             }
         }
         bool in = true;
@@ -229,8 +235,11 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
         if (!in) atomicOr(&a.counters[2], kFlagPoint);      // a point outside its brick: never expected, reported
         if (CH >= 2) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) wmax = fmaxf(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-            if (lane == 0) s_red[warp] = wmax;
+            for (int o = 16; o > 0; o >>= 1) {
+                wmax = fmaxf(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+                wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+            }
+            if (lane == 0) s_red[warp] = make_float2(wmax, wsum);
         }
         __syncthreads();
         if (warp == 0) {
@@ -250,19 +259,25 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
         __syncthreads();
         if (tid == 0) s_item = atomicAdd(&a.counters[3], 1);               // the next item
         if (CH >= 2) {
-            wmax = s_red[0];
+            wmax = s_red[0].x;
+            wsum = s_red[0].y;
 #pragma unroll
-            for (int i = 1; i < kWarps; ++i) wmax = fmaxf(wmax, s_red[i]);
+            for (int i = 1; i < kWarps; ++i) {
+                wmax = fmaxf(wmax, s_red[i].x);
+                wsum += s_red[i].y;
+            }
         }
-        // the region's unit: n points of weight wmax < 2^e (taps <= 1) stay within 2^30;
-        // n >= 32 keeps the scaled weights within fp16
+        // the region's units 2^ek and 2^eb: a cell's sum (taps <= 1) stays within 2^30 of them,
+        // bounded by n points of weight wmax, for A*b by the sum of its |weights| where that is
+        // less (a third of n wmax as a rule); 2^-25 wmax at least keeps the scaled weights within fp16
         const int lgn = max(32 - __clz(max(wk.z - 1, 1)), 5);
-        int ek = 0, eb = 0;
+        int ek = 0, eb = 0, es = 1 << 20;
         if (CH != 2 && a.wmax_fixed > 0.0f) frexpf(a.wmax_fixed, &ek);
         if (CH >= 2 && wmax > 0.0f) frexpf(wmax, &eb);
-        ek = max(ek, -90);
-        eb = max(eb, -90);
-        const float Sk = ldexpf(1.0f, 30 - 3 * kTapBits - lgn - ek), Sb = ldexpf(1.0f, 30 - 3 * kTapBits - lgn - eb);
+        if (CH >= 2 && wsum < 3e38f) frexpf(wsum, &es);
+        ek = max(ek, -90) + lgn - 30;
+        eb = max(eb, -90) + min(lgn, max(es - eb, 5)) - 30;
+        const float Sk = ldexpf(1.0f, -3 * kTapBits - ek), Sb = ldexpf(1.0f, -3 * kTapBits - eb);
         auto put = [&](int pos, uint32_t c0, uint32_t c1, uint32_t c2, const float* w) {
             uint32_t* r = s_rec + (pos >> 4) * RW + (pos & 15);
             r[0] = c0;
@@ -307,7 +322,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
         const int base = s_base;
         if (tid == 0) {
             if (!fits) atomicOr(&a.counters[2], kFlagPoint);
-            a.rec_item[item] = make_int4(wk.x, base, fits ? total / 16 : 0, lgn | (ek + 128) << 8 | (eb + 128) << 16);
+            a.rec_item[item] = make_int4(wk.x, base, fits ? total / 16 : 0, (ek + kUnitBias) | (eb + kUnitBias) << 16);
         }
         __syncthreads();
         item = s_item;
@@ -325,7 +340,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
 // ---------------------------------------------------------------------------
 // A class's sums into the brick's region (one rounding to the region's unit per cell).
 template <int W, int CH>
-__device__ __forceinline__ void flush_class(const float (&D)[MmaCfg<W, CH>::T][CH][4], int cls, int* lev1, int row, int c) {
+__device__ __forceinline__ void flush_class(const float2 (&D)[MmaCfg<W, CH>::T][CH][2], int cls, int* lev1, int row, int c) {
     using C = MmaCfg<W, CH>;
     constexpr int RG = C::RG, PS = C::PS, RG3 = C::RG3, PER = C::kPer, PERX = C::kPerX;
     const int z0 = cls / (PER * PERX) * C::kBases, y0 = cls / PERX % PER * C::kBases, x0 = cls % PERX * C::kBasesX;
@@ -336,10 +351,10 @@ __device__ __forceinline__ void flush_class(const float (&D)[MmaCfg<W, CH>::T][C
 #pragma unroll
             for (int ch = 0; ch < CH; ++ch) {
                 int* d = dst + ch * RG3 + 2 * t * RG;
-                atomicAdd(d, __float2int_rn(D[t][ch][0]));
-                atomicAdd(d + PS, __float2int_rn(D[t][ch][1]));
-                atomicAdd(d + RG, __float2int_rn(D[t][ch][2]));
-                atomicAdd(d + PS + RG, __float2int_rn(D[t][ch][3]));
+                atomicAdd(d, __float2int_rn(D[t][ch][0].x));
+                atomicAdd(d + PS, __float2int_rn(D[t][ch][0].y));
+                atomicAdd(d + RG, __float2int_rn(D[t][ch][1].x));
+                atomicAdd(d + PS + RG, __float2int_rn(D[t][ch][1].y));
             }
     } else {                                       // rows: 16 x of y = t
         // a class with fewer than kBases first taps, and x cell 15, reach past the region
@@ -351,10 +366,10 @@ __device__ __forceinline__ void flush_class(const float (&D)[MmaCfg<W, CH>::T][C
 #pragma unroll
             for (int ch = 0; ch < CH; ++ch) {
                 int* d = dst + ch * RG3 + t * RG;
-                atomicAdd(d, __float2int_rn(D[t][ch][0]));
-                if (z1) atomicAdd(d + PS, __float2int_rn(D[t][ch][1]));
-                if (x1) atomicAdd(d + 8, __float2int_rn(D[t][ch][2]));
-                if (x1 && z1) atomicAdd(d + PS + 8, __float2int_rn(D[t][ch][3]));
+                atomicAdd(d, __float2int_rn(D[t][ch][0].x));
+                if (z1) atomicAdd(d + PS, __float2int_rn(D[t][ch][0].y));
+                if (x1) atomicAdd(d + 8, __float2int_rn(D[t][ch][1].x));
+                if (x1 && z1) atomicAdd(d + PS + 8, __float2int_rn(D[t][ch][1].y));
             }
         }
     }
@@ -396,13 +411,11 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPo
         const int cls = s_cls[g];
         int ge = g + 1;                            // end of this class's run
         while (ge < gb && ge < g + kRunGroups && s_cls[ge] == cls) ++ge;
-        float D[T][CH][4];
+        float2 D[T][CH][2];
 #pragma unroll
         for (int t = 0; t < T; ++t)
 #pragma unroll
-            for (int ch = 0; ch < CH; ++ch)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) D[t][ch][k] = 0.0f;
+            for (int ch = 0; ch < CH; ++ch) D[t][ch][0] = D[t][ch][1] = make_float2(0.0f, 0.0f);
 #pragma unroll 1
         for (; g < ge; ++g) {
             const int r = g - ga, gi = r & 1;
@@ -496,12 +509,20 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPo
                     mul_split(xh[xb][0], xl[xb][0], yh0[yb], yl0[yb], ah[1], al[1]);
                     mul_split(xh[0][1], xl[0][1], yh1[ya], yl1[ya], ah[2], al[2]);
                     mul_split(xh[xb][1], xl[xb][1], yh1[yb], yl1[yb], ah[3], al[3]);
+                    // the group's products from zero, small ones first, then one rounded add: the
+                    // tensor core's own additions truncate
+                    float E[CH][4] = {};
 #pragma unroll
-                    for (int ch = 0; ch < CH; ++ch) mma16816(D[t][ch], al, bh[ch][0], bh[ch][1]);
+                    for (int ch = 0; ch < CH; ++ch) mma16816(E[ch], al, bh[ch][0], bh[ch][1]);
 #pragma unroll
-                    for (int ch = 0; ch < CH; ++ch) mma16816(D[t][ch], ah, bl[ch][0], bl[ch][1]);
+                    for (int ch = 0; ch < CH; ++ch) mma16816(E[ch], ah, bl[ch][0], bl[ch][1]);
 #pragma unroll
-                    for (int ch = 0; ch < CH; ++ch) mma16816(D[t][ch], ah, bh[ch][0], bh[ch][1]);
+                    for (int ch = 0; ch < CH; ++ch) mma16816(E[ch], ah, bh[ch][0], bh[ch][1]);
+#pragma unroll
+                    for (int ch = 0; ch < CH; ++ch)
+#pragma unroll
+                        for (int k = 0; k < 2; ++k)
+                            D[t][ch][k] = __fadd2_rn(D[t][ch][k], make_float2(E[ch][2 * k], E[ch][2 * k + 1]));
                 }
             }
         }
@@ -511,8 +532,7 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPo
     __syncthreads();
 
     // ---- the region into the FP64 grid (periodic wrap), cleared: a thread per column ----
-    const int lgn = wk.w & 255;
-    const float ik = ldexpf(1.0f, lgn - 30 + (wk.w >> 8 & 255) - 128), ib = ldexpf(1.0f, lgn - 30 + (wk.w >> 16 & 255) - 128);
+    const float ik = ldexpf(1.0f, (wk.w & 0xffff) - kUnitBias), ib = ldexpf(1.0f, (wk.w >> 16) - kUnitBias);
     double* gk = a.grid;
     double* gb_ = CH == 3 ? a.grid + (size_t)a.G * a.G * a.G : a.grid;
     if (tid < RG * RG) {
