@@ -78,23 +78,23 @@ __device__ __forceinline__ float2 dw_warp_sum(float2 v) {
     return v;
 }
 
-// Conversions between float and double by their bits, on host and device: the conversion
-// instructions run at this part's FP64 rate (1/64 of FP32), which bounds a pass over an FP64
-// grid.  The same results as the casts; what is rare there (subnormals, infinities, NaN) takes
-// the cast itself.
-__host__ __device__ __forceinline__ double widen(float v) {
-    const uint32_t b = __builtin_bit_cast(uint32_t, v), m = b & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u) return (double)v;
-    return __builtin_bit_cast(double, (uint64_t)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)) << 32 | (uint32_t)(b << 29));
+// Conversions between float and double by their bits: the conversion instructions run at
+// this part's FP64 rate (1/64 of FP32), which bounds a pass over an FP64 grid.
+// widen: exact for normal numbers (others become some number below 2^-126 in size).
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t b = __float_as_uint(v);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
-// narrow: rounded to nearest even; zeros (most of a grid's corners) stay on the fast path.
-__host__ __device__ __forceinline__ float narrow(double d) {
-    const uint64_t u = __builtin_bit_cast(uint64_t, d);
-    const uint32_t hi = (uint32_t)(u >> 32), s = hi & 0x80000000u, r = (uint32_t)u & 0x1fffffffu;
-    if ((hi & 0x7fffffffu) - 0x38100000u >= 0x47f00000u - 0x38100000u)
-        return u << 1 == 0 ? __builtin_bit_cast(float, s) : (float)d;
-    const uint32_t f = ((uint32_t)(u >> 29) - (896u << 23)) & 0x7fffffffu;      // exponent and 23 bits
-    return __builtin_bit_cast(float, s | (f + ((r + 0x0fffffffu + (f & 1u)) >> 29)));
+// narrow: rounded to nearest (halves away from zero); below 2^-126 it gives 0, and
+// infinities and NaN stay what they are.
+__device__ __forceinline__ float narrow(double d) {
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t e = hi & 0x7ff00000u;
+    const uint32_t m = __funnelshift_l(lo, hi, 3) - (896u << 23);     // exponent and 23 bits (sign lost)
+    uint32_t f = e >= 0x38100000u ? (m & 0x7fffffffu) + ((lo >> 28) & 1u) : 0u;
+    if (e >= 0x47f00000u)                          // 2^128 and above, infinities; NaN
+        f = e == 0x7ff00000u && ((hi & 0xfffffu) | lo) ? 0x7fc00000u : 0x7f800000u;
+    return __uint_as_float((hi & 0x80000000u) | f);
 }
 
 }  // namespace firm
