@@ -88,6 +88,13 @@ __host__ __device__ __forceinline__ double widen(float v) {
     const uint32_t e = m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
     return __builtin_bit_cast(double, (uint64_t)((b & 0x80000000u) | ((m >> 3) + e)) << 32 | (uint32_t)(b << 29));
 }
+// v 2^e, |v| in [1, 2^31], |e| < 800: the exponent added in place, so no FP32 product can overflow
+// or become subnormal.
+__host__ __device__ __forceinline__ double widen_scaled(float v, int e) {
+    const uint32_t b = __builtin_bit_cast(uint32_t, v);
+    const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u + ((uint32_t)e << 20));
+    return __builtin_bit_cast(double, (uint64_t)hi << 32 | (uint32_t)(b << 29));
+}
 // narrow: rounded to nearest (halves away from zero); below 2^-126 it gives 0, and
 // infinities and NaN stay what they are.
 __host__ __device__ __forceinline__ float narrow(double d) {

@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
         if (CH != 2 && a.wmax_fixed > 0.0f) frexpf(a.wmax_fixed, &ek);
         if (CH >= 2 && wmax > 0.0f) frexpf(wmax, &eb);
         if (CH >= 2 && wsum < 3e38f) frexpf(wsum, &es);
-        ek = max(ek, -90) + lgn - 30;
-        eb = max(eb, -90) + min(lgn, max(es - eb, 5)) - 30;
+        ek = max(ek, -112) + lgn - 30;             // the scales stay within FP32
+        eb = max(eb, -112) + min(lgn, max(es - eb, 5)) - 30;
         const float Sk = ldexpf(1.0f, -3 * kTapBits - ek), Sb = ldexpf(1.0f, -3 * kTapBits - eb);
         auto put = [&](int pos, uint32_t c0, uint32_t c1, uint32_t c2, const float* w) {
             uint32_t* r = s_rec + (pos >> 4) * RW + (pos & 15);
@@ -532,7 +532,7 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPo
     __syncthreads();
 
     // ---- the region into the FP64 grid (periodic wrap), cleared: a thread per column ----
-    const float ik = ldexpf(1.0f, (wk.w & 0xffff) - kUnitBias), ib = ldexpf(1.0f, (wk.w >> 16) - kUnitBias);
+    const int ek = (wk.w & 0xffff) - kUnitBias, eb = (wk.w >> 16) - kUnitBias;
     double* gk = a.grid;
     double* gb_ = CH == 3 ? a.grid + (size_t)a.G * a.G * a.G : a.grid;
     if (tid < RG * RG) {
@@ -553,8 +553,8 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPo
                 const int v = *p;
                 if (v == 0) continue;
                 *p = 0;
-                if (CH != 2 && ch == 0) atomicAdd(&gk[cell], widen((float)v * ik));
-                else atomicAdd(&gb_[2 * (size_t)cell + (CH == 3 ? ch - 1 : ch)], widen((float)v * ib));
+                if (CH != 2 && ch == 0) atomicAdd(&gk[cell], widen_scaled((float)v, ek));
+                else atomicAdd(&gb_[2 * (size_t)cell + (CH == 3 ? ch - 1 : ch)], widen_scaled((float)v, eb));
             }
         }
     }

@@ -32,6 +32,11 @@ static void w(uint32_t b) {
     bad += fabsf(v) < least ? !(fabs(d) <= (double)least) : !same(d, (double)v);
 }
 int main() {
+    for (int i = 0; i < 1000000; ++i) {                 // integers of either sign at any unit
+        const float v = (float)(int)((rnd() & 1 ? 1 : -1) * (1 + (int64_t)(rnd() >> (33 + rnd() % 31))));
+        const int e = (int)(rnd() % 400) - 200;
+        bad += !same(firm::widen_scaled(v, e), ldexp((double)v, e));
+    }
     for (uint64_t e = 0; e < 2048; ++e)                 // every exponent, around the ends and ties of the mantissa
         for (uint64_t m : {0ull, 1ull, 0xfffffffull, 0x10000000ull, 0x10000001ull, 0x1fffffffull, 0x2fffffffull,
                            0x30000000ull, 0x30000001ull, 0xfffffe0000000ull, 0xfffffefffffffull, 0xffffff0000000ull,
