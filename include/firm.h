@@ -15,7 +15,9 @@
  *     i_j <-> centred coordinate n_j = i_j - N/2 (Section 3.1).
  *   - Images are M x N x N, [m][i2][i1], float32 or bfloat16 (firm_params.img_dtype),
  *     starting at a 16-byte aligned address (each image is moved into shared memory by
- *     one bulk copy); a misaligned image array is rejected with FIRM_EINVAL.
+ *     one bulk copy); a misaligned image array is rejected with FIRM_EINVAL.  Values are
+ *     finite: a NaN or an infinity leaves A*b unspecified, and where points are dense enough for
+ *     the tensor cores it is reported as FIRM_EINVAL in the way of FIRM_EINTERNAL.
  *   - R is M x 9 float64, each rotation row-major.  Columns (R_1d, R_2d) of its first two
  *     rows, of length at most 1 in a rotation, are taken below 3; a longer or NaN one is
  *     reported as FIRM_EINVAL in the way of FIRM_EINTERNAL.  The slice of image m samples

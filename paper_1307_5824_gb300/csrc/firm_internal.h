@@ -45,7 +45,8 @@ constexpr int kGeomBits = 41;
 constexpr int kGeomWide = 1 << 16;    // in ul[0], above the low part: positions of this image need 64 bits
 
 // Bits of the device flag, counters[2]: an internal invariant (a point outside its brick, an
-// image copy that did not land), or an input that cannot be used (a matrix beyond the limit).
+// image copy that did not land), or an input that cannot be used (a matrix beyond the limit, a
+// NaN or infinite A*b weight in the tensor-core form).
 constexpr int kFlagPoint = 1, kFlagCopy = 4, kFlagInput = 8;
 inline int flag_status(int flag) {
     return flag & (kFlagPoint | kFlagCopy) ? FIRM_EINTERNAL : flag ? FIRM_EINVAL : FIRM_OK;

@@ -270,6 +270,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
         // the region's units 2^ek and 2^eb: a cell's sum (taps <= 1) stays within 2^30 of them,
         // bounded by n points of weight wmax, for A*b by the sum of its |weights| where that is
         // less (a third of n wmax as a rule); 2^-25 wmax at least keeps the scaled weights within fp16
+        // (fmaxf passes over a NaN, the sum keeps it)
+        if (CH >= 2 && tid == 0 && (wsum != wsum || isinf(wmax))) atomicOr(&a.counters[2], kFlagInput);
         const int lgn = max(32 - __clz(max(wk.z - 1, 1)), 5);
         int ek = 0, eb = 0, es = 1 << 20;
         if (CH != 2 && a.wmax_fixed > 0.0f) frexpf(a.wmax_fixed, &ek);

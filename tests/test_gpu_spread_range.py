@@ -55,3 +55,20 @@ def test_small_images_scale(F, M, fused):
     print(f"M={M} fused={fused}: {err:.2e}")
     assert err <= 1e-6
     rec.close()
+
+
+@pytest.mark.parametrize("M,fused", DENSE)
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_non_finite_images_are_reported(F, M, fused, value):
+    """One bad pixel spoils the sums of every class of cells its image crosses: reported by the
+    next call that waits, and the plan takes the next images."""
+    rec, images, rhs = setup(F, M, fused)
+    want = rhs(images)
+    bad = images.copy()
+    bad[M // 2, 3, 5] = value
+    with pytest.raises(F._lib.FirmError) as e:
+        rhs(bad)
+    assert e.value.code == F._lib.FIRM_EINVAL
+    got = rhs(images)
+    assert np.linalg.norm(got - want) <= 1e-6 * np.linalg.norm(want)
+    rec.close()
