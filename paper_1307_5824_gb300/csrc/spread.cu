@@ -1324,8 +1324,9 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
             s_g[i] = __ldg(&a.ghat[((size_t)gz * a.G + gy) * a.G + gx]);
         }
         __syncthreads();
-        // sums of a thread's points in double-words: 48 bits, at the FP32 rate
-        float2 acc_r = make_float2(0.0f, 0.0f), acc_b = make_float2(0.0f, 0.0f);
+        // residuals and sums in FP64 (as double-words they would be 48 bits within FP32's
+        // range, and no faster: the shared loads of the taps bound the loop)
+        double acc_r = 0.0, acc_b = 0.0;
         for (int i = threadIdx.x; i < wk.z; i += blockDim.x) {
             const uint32_t pos = (uint32_t)wk.y + i;
             const uint32_t id = __ldg(&a.payload[pos]);
@@ -1360,25 +1361,22 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
                 a.out[(size_t)m * a.nH + t] = make_float2(h * f.x, h * f.y);
             } else {
                 const float2 bv = __ldg(&a.samples_b[wk.y + __ldg(&a.perm[pos])]);
-                const float2 one = make_float2(h, 0.0f);
-                const float2 dr = dw_sub_mul(make_float2(bv.x, 0.0f), one, f.x);
-                const float2 di = dw_sub_mul(make_float2(bv.y, 0.0f), one, f.y);
-                // c = 2 off the origin: the conjugate half; the origin counts once
-                float2 pr = dw_acc_sq(make_float2(0.0f, 0.0f), dr), pb = make_float2(0.0f, 0.0f);
-                pr = dw_acc_sq(pr, di);
-                pb = dw_acc_prod(pb, bv.x, bv.x);
-                pb = dw_acc_prod(pb, bv.y, bv.y);
-                const float c = t == 0 ? 1.0f : 2.0f;
-                acc_r = dw_add(acc_r, c * pr.x, c * pr.y);
-                acc_b = dw_add(acc_b, c * pb.x, c * pb.y);
+                const double bx = bv.x, by = bv.y, hd = h;
+                const double dr = bx - hd * f.x, di = by - hd * f.y;
+                const double c = t == 0 ? 1.0 : 2.0;       // off the origin: the conjugate half too
+                acc_r += c * (dr * dr + di * di);
+                acc_b += c * (bx * bx + by * by);
             }
         }
         if (RESID) {
-            acc_r = dw_warp_sum(acc_r);
-            acc_b = dw_warp_sum(acc_b);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                acc_r += __shfl_xor_sync(0xffffffffu, acc_r, o);
+                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, o);
+            }
             if (lane == 0) {
-                s_red[0][warp] = dw_to_double(acc_r);
-                s_red[1][warp] = dw_to_double(acc_b);
+                s_red[0][warp] = acc_r;
+                s_red[1][warp] = acc_b;
             }
             __syncthreads();
             if (threadIdx.x == 0) {
