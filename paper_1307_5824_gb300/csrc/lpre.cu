@@ -161,9 +161,11 @@ __global__ void __launch_bounds__(256) k_pc_from_table(const float* __restrict__
 // ---------------------------------------------------------------------------
 // Principal axis of the symmetric 3x3 moment, on the device (one thread), so that
 // firm_kernel needs no host round trip: Jacobi eigenvalue iterations in FP32, then the
-// eigenvector corrected in FP64 by first-order perturbation steps, each of which takes its
-// error e to about 1e-7 e + e^2 / gap.  (Jacobi in FP64 throughout took 45 us: this part's
-// FP64 sine, cosine and division are long chains of slow operations.)
+// eigenvector corrected in FP64 by first-order perturbation steps, each of which takes its error
+// to about 1e-7 / gap of it (gap: to the next eigenvalue, trace 1).  From gaps of 1e-4 down the FP64
+// work is Jacobi rotations by square roots from the FP32 basis, which resolve any gap and take
+// 12 us more.  (In FP64 throughout, with sine and cosine, it took 45 us: long chains of slow
+// operations on this part.)
 // ---------------------------------------------------------------------------
 __device__ static void principal_axis(const double* S, float* a) {     // S: xx, xy, xz, yy, yz, zz
     const double B[3][3] = {{S[0], S[1], S[2]}, {S[1], S[3], S[4]}, {S[2], S[4], S[5]}};
@@ -205,27 +207,81 @@ __device__ static void principal_axis(const double* S, float* a) {     // S: xx,
     int best = 0;
     for (int i = 1; i < 3; ++i)
         if (A[i][i] > A[best][best]) best = i;
-    double v[3] = {V[0][best], V[1][best], V[2][best]};
-    for (int it = 0; it < 3; ++it) {
-        double w[3], lam = 0.0, n2 = 0.0;
-        for (int i = 0; i < 3; ++i) {
-            w[i] = D[i][0] * v[0] + D[i][1] * v[1] + D[i][2] * v[2];
-            lam += w[i] * v[i];
-            n2 += v[i] * v[i];
+    const int j1 = best == 0 ? 1 : 0, j2 = best == 2 ? 1 : 2;
+    const float gap1 = A[best][best] - A[j1][j1], gap2 = A[best][best] - A[j2][j2];
+    if (gap1 > 1e-4f && gap2 > 1e-4f) {
+        double v[3] = {V[0][best], V[1][best], V[2][best]};
+        const double inv[2] = {(double)(1.0f / gap1), (double)(1.0f / gap2)};
+        for (int it = 0; it < 3; ++it) {
+            double w[3], lam = 0.0, n2 = 0.0;
+            for (int i = 0; i < 3; ++i) {
+                w[i] = D[i][0] * v[0] + D[i][1] * v[1] + D[i][2] * v[2];
+                lam += w[i] * v[i];
+                n2 += v[i] * v[i];
+            }
+            lam *= 2.0 - n2;                        // Rayleigh quotient, |v| = 1 to 1e-6
+            for (int i = 0; i < 3; ++i) w[i] -= lam * v[i];
+            for (int k = 0; k < 2; ++k) {
+                const int j = k ? j2 : j1;
+                const double c = (w[0] * V[0][j] + w[1] * V[1][j] + w[2] * V[2][j]) * inv[k];
+                for (int i = 0; i < 3; ++i) v[i] += c * V[i][j];
+            }
+            n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+            const double r = 1.5 - 0.5 * n2;        // 1 / |v| to (n2 - 1)^2
+            for (int i = 0; i < 3; ++i) v[i] *= r;
         }
-        lam *= 2.0 - n2;                            // Rayleigh quotient, |v| = 1 to 1e-6
-        for (int i = 0; i < 3; ++i) w[i] -= lam * v[i];
-        for (int j = 0; j < 3; ++j) {
-            const float gap = A[best][best] - A[j][j];
-            if (j == best || !(gap > 1e-6f)) continue;         // (nearly) equal eigenvalues: any axis of them
-            const double c = (w[0] * V[0][j] + w[1] * V[1][j] + w[2] * V[2][j]) * (double)(1.0f / gap);
-            for (int i = 0; i < 3; ++i) v[i] += c * V[i][j];
-        }
-        n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-        const double r = 1.5 - 0.5 * n2;            // 1 / |v| to (n2 - 1)^2
-        for (int i = 0; i < 3; ++i) v[i] *= r;
+        for (int i = 0; i < 3; ++i) a[i] = (float)v[i];
+        return;
     }
-    for (int i = 0; i < 3; ++i) a[i] = (float)v[i];
+    double U[3][3], B2[3][3];
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) U[i][j] = V[i][j];
+    for (int it = 0; it < 2; ++it) {                // U <- U (3 I - U^T U) / 2: orthonormal to 1e-7, then 1e-14, 1e-28
+        double G[3][3], T[3][3];
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j)
+                G[i][j] = (i == j ? 1.5 : 0.0) - 0.5 * (U[0][i] * U[0][j] + U[1][i] * U[1][j] + U[2][i] * U[2][j]);
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) T[i][j] = U[i][0] * G[0][j] + U[i][1] * G[1][j] + U[i][2] * G[2][j];
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) U[i][j] = T[i][j];
+    }
+    {                                               // B2 = U^T D U
+        double T[3][3];
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) T[i][j] = D[i][0] * U[0][j] + D[i][1] * U[1][j] + D[i][2] * U[2][j];
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) B2[i][j] = U[0][i] * T[0][j] + U[1][i] * T[1][j] + U[2][i] * T[2][j];
+    }
+    for (int sweep = 0; sweep < 8; ++sweep) {
+        if (fabs(B2[0][1]) + fabs(B2[0][2]) + fabs(B2[1][2]) < 1e-15) break;       // of a trace of 1
+        for (int p = 0; p < 2; ++p)
+            for (int q = p + 1; q < 3; ++q) {
+                if (B2[p][q] == 0.0) continue;
+                const double th = (B2[q][q] - B2[p][p]) / (2.0 * B2[p][q]);
+                const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
+                const double c = rsqrt(1.0 + t * t), s = t * c;
+                for (int k = 0; k < 3; ++k) {
+                    const double akp = B2[k][p], akq = B2[k][q];
+                    B2[k][p] = c * akp - s * akq;
+                    B2[k][q] = s * akp + c * akq;
+                }
+                for (int k = 0; k < 3; ++k) {
+                    const double apk = B2[p][k], aqk = B2[q][k];
+                    B2[p][k] = c * apk - s * aqk;
+                    B2[q][k] = s * apk + c * aqk;
+                }
+                for (int k = 0; k < 3; ++k) {
+                    const double ukp = U[k][p], ukq = U[k][q];
+                    U[k][p] = c * ukp - s * ukq;
+                    U[k][q] = s * ukp + c * ukq;
+                }
+            }
+    }
+    best = 0;
+    for (int i = 1; i < 3; ++i)
+        if (B2[i][i] > B2[best][best]) best = i;
+    for (int i = 0; i < 3; ++i) a[i] = (float)U[i][best];
 }
 
 __global__ void k_view_axis(const double* __restrict__ part, int n, float* __restrict__ axis) {
