@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_init(const float* __restrict_
 
 // alpha from the Toeplitz apply's n_pq partial sums of <p, q> (every block forms it), then
 // x += alpha p, r -= alpha q, <r, r> and the next beta.
-__global__ void __launch_bounds__(kCgThreads) k_cg_update(float* __restrict__ x, float2* __restrict__ r,
-                                                          const float* __restrict__ p, const float* __restrict__ q,
+__global__ void __launch_bounds__(kCgThreads) k_cg_update(float* x, float2* r,
+                                                          const float* p, const float* q,
                                                           size_t n4, CgState* cg, double* red, double* hist,
                                                           const double* red_pq, int n_pq) {
     __shared__ double s_warp[kCgThreads / 32];

@@ -135,7 +135,7 @@ struct NoFinish {
 struct KerRowsOp : NoFinish {
     const double* grid; float2* out; const float2* tw; int n_rows, G, N;
     __device__ __forceinline__ float2 load(int row, int n) const {
-        return make_float2(narrow(__ldg(&grid[(size_t)row * G + n])), 0.0f);
+        return make_float2(narrow(grid[(size_t)row * G + n]), 0.0f);
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
         if (k <= N) out[(size_t)row * (N + 1) + k] = v;
@@ -144,7 +144,7 @@ struct KerRowsOp : NoFinish {
 struct KerColsYOp {
     const float2* in; float2* out; const float2* tw; int n_outer, n_inner, G, N;
     __device__ __forceinline__ float2 load(int o, int n, int i) const {
-        return __ldg(&in[((size_t)o * G + n) * (N + 1) + i]);
+        return in[((size_t)o * G + n) * (N + 1) + i];
     }
     __device__ __forceinline__ void store(int o, int k, int i, float2 v) const {
         const int n2 = k < N ? k : (k >= G - N ? k - G : G);
@@ -153,7 +153,7 @@ struct KerColsYOp {
 };
 struct KerColsZOp {
     const float2* in; float* ker; const float* dec; const float2* tw; int n_outer, n_inner, G, N;
-    __device__ __forceinline__ float2 load(int, int n, int i) const { return __ldg(&in[(size_t)n * n_inner + i]); }
+    __device__ __forceinline__ float2 load(int, int n, int i) const { return in[(size_t)n * n_inner + i]; }
     __device__ __forceinline__ void store(int, int k, int i, float2 v) const {
         const int n3 = k < N ? k : (k >= G - N ? k - G : G);
         if (n3 == G) return;
@@ -193,7 +193,7 @@ struct KhatRowsOp : NoFinish {
         size_t idx;
         if (d1 >= 0) idx = ((size_t)(d3 + N) * N2 + (d2 + N)) * (N + 1) + d1;
         else idx = ((size_t)(N - d3) * N2 + (N - d2)) * (N + 1) + (-d1);
-        return make_float2(__ldg(&ker[idx]), 0.0f);
+        return make_float2(ker[idx], 0.0f);
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
         if (k <= N) out[(size_t)row * (N + 1) + k] = v;
@@ -202,7 +202,7 @@ struct KhatRowsOp : NoFinish {
 struct KhatColsYOp {
     const float2* in; float2* out; const float2* tw; int n_outer, n_inner, L;
     __device__ __forceinline__ float2 load(int o, int n, int i) const {
-        return __ldg(&in[((size_t)o * L + n) * n_inner + i]);
+        return in[((size_t)o * L + n) * n_inner + i];
     }
     __device__ __forceinline__ void store(int o, int k, int i, float2 v) const {
         out[((size_t)o * L + k) * n_inner + i] = v;
@@ -210,7 +210,7 @@ struct KhatColsYOp {
 };
 struct KhatColsZOp {
     const float2* in; float* khat; const float2* tw; int n_outer, n_inner;
-    __device__ __forceinline__ float2 load(int, int n, int i) const { return __ldg(&in[(size_t)n * n_inner + i]); }
+    __device__ __forceinline__ float2 load(int, int n, int i) const { return in[(size_t)n * n_inner + i]; }
     __device__ __forceinline__ void store(int, int k, int i, float2 v) const { khat[(size_t)k * n_inner + i] = v.x; }
 };
 
@@ -232,7 +232,7 @@ cudaError_t launch_khat(Plan& P) {
 
 // lam_eff = lambda Ker(0) (relative reading) or lambda (absolute), on the device, so that
 // the Toeplitz apply needs no host round trip; Ker(0) sits at (j3, j2, j1) = (N, N, 0).
-__global__ void k_lam_eff(const float* __restrict__ ker, size_t i0, double lambda, int relative, float* lam) {
+__global__ void k_lam_eff(const float* ker, size_t i0, double lambda, int relative, float* lam) {
     pdl_wait();
     pdl_launch();
     const float k0 = ker[i0];
@@ -291,7 +291,7 @@ cudaError_t launch_damping(Plan& P) {
 struct RhsRowsOp : NoFinish {
     const double* grid; float2* out; const float2* tw; int n_rows, G, N;
     __device__ __forceinline__ float2 load(int row, int n) const {
-        const double2 g = __ldg(reinterpret_cast<const double2*>(grid) + (size_t)row * G + n);
+        const double2 g = reinterpret_cast<const double2*>(grid)[(size_t)row * G + n];
         return make_float2(narrow(g.x), narrow(g.y));
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
@@ -303,7 +303,7 @@ struct RhsRowsOp : NoFinish {
 struct RhsColsYOp {
     const float2* in; float2* out; const float2* tw; int n_outer, n_inner, G, N;
     __device__ __forceinline__ float2 load(int o, int n, int i) const {
-        return __ldg(&in[((size_t)o * G + n) * N + i]);
+        return in[((size_t)o * G + n) * N + i];
     }
     __device__ __forceinline__ void store(int o, int k, int i, float2 v) const {
         const int h = N / 2;
@@ -313,7 +313,7 @@ struct RhsColsYOp {
 };
 struct RhsColsZOp {
     const float2* in; float* rhs; const float* dec; const float2* tw; int n_outer, n_inner, G, N;
-    __device__ __forceinline__ float2 load(int, int n, int i) const { return __ldg(&in[(size_t)n * n_inner + i]); }
+    __device__ __forceinline__ float2 load(int, int n, int i) const { return in[(size_t)n * n_inner + i]; }
     __device__ __forceinline__ void store(int, int k, int i, float2 v) const {
         const int h = N / 2;
         const int n3 = k < h ? k : (k >= G - h ? k - G : G);
@@ -600,7 +600,7 @@ cudaError_t launch_image_dft(Plan& P, int M, const void* images, const double* s
 struct TRowsFwdOp : NoFinish {
     const float* x; float2* out; const float2* tw; int n_rows, N;
     __device__ __forceinline__ float2 load(int row, int n) const {
-        return make_float2(n < N ? __ldg(&x[(size_t)row * N + n]) : 0.0f, 0.0f);
+        return make_float2(n < N ? x[(size_t)row * N + n] : 0.0f, 0.0f);
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
         if (k <= N) out[(size_t)row * (N + 1) + k] = v;
@@ -609,7 +609,7 @@ struct TRowsFwdOp : NoFinish {
 struct TColsYFwdOp {
     const float2* in; float2* out; const float2* tw; int n_outer, n_inner, N;
     __device__ __forceinline__ float2 load(int o, int n, int i) const {
-        return n < N ? __ldg(&in[((size_t)o * N + n) * (N + 1) + i]) : make_float2(0.0f, 0.0f);
+        return n < N ? in[((size_t)o * N + n) * (N + 1) + i] : make_float2(0.0f, 0.0f);
     }
     __device__ __forceinline__ void store(int o, int k, int i, float2 v) const {
         out[((size_t)o * 2 * N + k) * (N + 1) + i] = v;
@@ -618,7 +618,7 @@ struct TColsYFwdOp {
 struct TColsYInvOp {
     const float2* in; float2* out; const float2* tw; int n_outer, n_inner, N;
     __device__ __forceinline__ float2 load(int o, int n, int i) const {
-        return __ldg(&in[((size_t)o * 2 * N + n) * (N + 1) + i]);
+        return in[((size_t)o * 2 * N + n) * (N + 1) + i];
     }
     __device__ __forceinline__ void store(int o, int k, int i, float2 v) const {
         if (k < N) out[((size_t)o * N + k) * (N + 1) + i] = v;
@@ -628,18 +628,18 @@ struct TRowsInvOp : NoFinish {
     const float2* in; const float* x; float* y; const float2* tw; int n_rows, N; float scale, lam;
     __device__ __forceinline__ float2 load(int row, int n) const {
         const float2* rr = in + (size_t)row * (N + 1);
-        return n <= N ? __ldg(&rr[n]) : c_conj(__ldg(&rr[2 * N - n]));
+        return n <= N ? rr[n] : c_conj(rr[2 * N - n]);
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
         if (k >= N) return;
         const size_t i = (size_t)row * N + k;
-        y[i] = fmaf(v.x, scale, lam * __ldg(&x[i]));
+        y[i] = fmaf(v.x, scale, lam * x[i]);
     }
 };
 
 // The z pass: forward, times K-hat, inverse; tile of TX<L>() adjacent (j2, j1) columns.
 template <int L>
-__global__ void __launch_bounds__(kThreads) k_toep_z(float2* __restrict__ t2, const float* __restrict__ khat,
+__global__ void __launch_bounds__(kThreads) k_toep_z(float2* t2, const float* __restrict__ khat,
                                                      const float2* __restrict__ tw, int n_inner, int N,
                                                      const CgState* cg) {
     extern __shared__ float2 S[];
@@ -665,11 +665,11 @@ template <int N> struct ToepFwdOp {
     float bh, bl;               // beta as a double-word
     size_t base;                // first voxel of the plane
     __device__ __forceinline__ float one(size_t i) const {
-        if (!cg) return __ldg(&x[i]);
+        if (!cg) return x[i];
         const float pv = p[i];
         float ah, al;
-        if (z) { ah = __ldg(&z[i]); al = 0.0f; }
-        else { const float2 rv = __ldg(&r[i]); ah = rv.x; al = rv.y; }
+        if (z) { ah = z[i]; al = 0.0f; }
+        else { const float2 rv = r[i]; ah = rv.x; al = rv.y; }
         return fmaf(bh, pv, ah) + fmaf(bl, pv, al);
     }
     __device__ __forceinline__ float2 load(int pair, int n) const {
@@ -739,7 +739,7 @@ template <int N> struct ToepInvOp {
     __device__ __forceinline__ float2 pre(int pair, int n) const {
         if (n >= N) return make_float2(0.0f, 0.0f);
         const size_t i = base + (size_t)(2 * pair) * N + n;
-        return make_float2(__ldg(&x[i]), __ldg(&x[i + N]));
+        return make_float2(x[i], x[i + N]);
     }
     __device__ __forceinline__ void store(int pair, int n, float2 v, float2 xv) {
         if (n >= N) return;
@@ -765,7 +765,7 @@ __global__ void __launch_bounds__(PlaneCfg<L, L / 2>::kThreads) k_toep_plane_inv
     pdl_launch();
     if (cg && cg->done) return;
     const int plane = blockIdx.x;
-    ToepInvOp<N> op{x, y, scale, __ldg(lam_p), cg != nullptr, make_float2(0.0f, 0.0f), (size_t)plane * N * N};
+    ToepInvOp<N> op{x, y, scale, *lam_p, cg != nullptr, make_float2(0.0f, 0.0f), (size_t)plane * N * N};
     plane_inverse<L, N>(op, t2 + (size_t)plane * L * (N + 1), tw, S);
     if (!cg) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -859,7 +859,7 @@ cudaError_t launch_toeplitz(Plan& P, const float* x, float* y, const float2* cg_
 struct PRowsFwdOp : NoFinish {
     const float2* r; float2* u; const float2* tw; int n_rows, N;     // r: double-words
     __device__ __forceinline__ float2 load(int row, int n) const {
-        const float2 v = __ldg(&r[(size_t)row * N + n]);
+        const float2 v = r[(size_t)row * N + n];
         return make_float2(v.x + v.y, 0.0f);
     }
     __device__ __forceinline__ void store(int row, int k, float2 v) const {
@@ -873,7 +873,7 @@ struct PColsYOp {
 };
 
 template <int L>
-__global__ void __launch_bounds__(kThreads) k_pc_z(float2* __restrict__ u, const float* __restrict__ d,
+__global__ void __launch_bounds__(kThreads) k_pc_z(float2* u, const float* __restrict__ d,
                                                    const float2* __restrict__ tw, int n_inner, const CgState* cg) {
     extern __shared__ float2 S[];
     pdl_wait();
@@ -891,7 +891,7 @@ __global__ void __launch_bounds__(kThreads) k_pc_z(float2* __restrict__ u, const
 template <int N> struct PcFwdOp {
     const float2* r;
     __device__ __forceinline__ float2 load(int pair, int n) const {
-        const float2 a = __ldg(&r[(size_t)(2 * pair) * N + n]), b = __ldg(&r[(size_t)(2 * pair + 1) * N + n]);
+        const float2 a = r[(size_t)(2 * pair) * N + n], b = r[(size_t)(2 * pair + 1) * N + n];
         return make_float2(a.x + a.y, b.x + b.y);
     }
     __device__ __forceinline__ void post(int, int, float2) const {}
@@ -919,7 +919,7 @@ template <int N> struct PcInvOp {
     float2 acc, acc_old;
     __device__ __forceinline__ Pre pre(int pair, int n) const {
         const size_t i = (size_t)(2 * pair) * N + n;
-        return Pre{__ldg(&r[i]), __ldg(&r[i + N]), z[i], z[i + N]};
+        return Pre{r[i], r[i + N], z[i], z[i + N]};
     }
     __device__ __forceinline__ void store(int pair, int n, float2 v, const Pre& p) {
         const size_t i = (size_t)(2 * pair) * N + n;
@@ -1006,7 +1006,7 @@ __global__ void k_chan_column(const float* __restrict__ ker, float2* __restrict_
                     const double w3 = w2 * (double)(N - abs(n3)) / N;
                     const size_t idx = n1 >= 0 ? ((size_t)(n3 + N) * N2 + (n2 + N)) * (N + 1) + n1
                                                : ((size_t)(N - n3) * N2 + (N - n2)) * (N + 1) + (-n1);
-                    acc += w3 * (double)__ldg(&ker[idx]);
+                    acc += w3 * (double)ker[idx];
                 }
             }
         }

@@ -52,7 +52,7 @@ template <int L, int N> struct PlaneCfg {
 // Forward: row pairs (op.load(p, n) gives sample n of rows 2p and 2p + 1, op.post(p, n, v)
 // runs after a pair's loads), then columns into out[k2][k1].  S: kSmem bytes.
 template <int L, int N, class Op>
-__device__ __forceinline__ void plane_forward(Op& op, float2* __restrict__ out, const float2* __restrict__ tw, float2* S) {
+__device__ __forceinline__ void plane_forward(Op& op, float2* out, const float2* __restrict__ tw, float2* S) {
     using P = PlaneCfg<L, N>;
     constexpr int H = P::H, NP = P::NP, M = NP * H;
     float2* plane = S;                       // [pair][k1], k1 < H; then [pair][L - k1]
@@ -86,7 +86,7 @@ __device__ __forceinline__ void plane_forward(Op& op, float2* __restrict__ out, 
 // Inverse: columns of in[k2][k1], outputs y < N kept, then row pairs; op.pre(p, n) is
 // fetched ahead of op.store(p, n, (row 2p, row 2p + 1), pre).
 template <int L, int N, class Op>
-__device__ __forceinline__ void plane_inverse(Op& op, const float2* __restrict__ in, const float2* __restrict__ tw,
+__device__ __forceinline__ void plane_inverse(Op& op, const float2* in, const float2* __restrict__ tw,
                                               float2* S) {
     using P = PlaneCfg<L, N>;
     constexpr int H = P::H, NP = P::NP;
@@ -94,7 +94,7 @@ __device__ __forceinline__ void plane_inverse(Op& op, const float2* __restrict__
     float2* X = S + P::kPlane;
     for (int b0 = 0; b0 < H; b0 += P::CB) {
         const int nl = min(P::CB, H - b0);
-        auto ld = [&](int line, int n) { return __ldg(&in[(size_t)n * H + b0 + line]); };
+        auto ld = [&](int line, int n) { return in[(size_t)n * H + b0 + line]; };
         auto st = [&](int line, int k, float2 v) {
             if (k < N) plane[k * H + b0 + line] = v;
         };

@@ -36,7 +36,7 @@ __device__ __forceinline__ int freq_bin(float q1, float q2, float q3, float half
 // second moment of the viewing directions d = third row of R_m (sum of d d^T)
 constexpr int kMomentBlocks = 64, kMomentThreads = 256;
 __global__ void __launch_bounds__(kMomentThreads) k_view_moment(const double* __restrict__ R, int M,
-                                                               double* __restrict__ part) {
+                                                               double* part) {
     pdl_wait();
     pdl_launch();
     __shared__ double s[kMomentThreads / 32][6];
@@ -284,7 +284,7 @@ __device__ static void principal_axis(const double* S, float* a) {     // S: xx,
     for (int i = 0; i < 3; ++i) a[i] = (float)U[i][best];
 }
 
-__global__ void k_view_axis(const double* __restrict__ part, int n, float* __restrict__ axis) {
+__global__ void k_view_axis(const double* part, int n, float* axis) {
     pdl_wait();
     pdl_launch();
     __shared__ double s[6];

@@ -1,5 +1,11 @@
 // pdl.cuh -- programmatic dependent launch.  Kernels of a chain that start with pdl_wait()
 // and are launched with launch_pdl need no drained SM between them: 1 to 2 us a launch.
+//
+// Such a kernel is resident while the one before it still writes, so what that one writes is
+// read by plain loads only: __ldg and const __restrict__ (loads for data that is read-only for
+// the kernel's whole life, which the compiler may also move above pdl_wait) are for tables that
+// are complete two launches earlier -- the plan's tables, the caller's inputs, K-hat and the
+// preconditioner's diagonal.
 #pragma once
 #include <cuda_runtime.h>
 

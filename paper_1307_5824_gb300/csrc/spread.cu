@@ -39,7 +39,7 @@ namespace firm {
 // one wrap of the grid brings every sample back (point_pos).  A matrix with a longer pair or a
 // NaN is put on the origin, so that no point leaves the bricks, and reported.
 // wide: the length beyond which positions need 64 bits (axis_pos).
-__global__ void k_geom(const double* __restrict__ R, int M, double wide, ImgGeom* __restrict__ g, int* err) {
+__global__ void k_geom(const double* __restrict__ R, int M, double wide, ImgGeom* g, int* err) {
     pdl_wait();
     pdl_launch();
     int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256) k_bin(BinArgs a, int M) {
                 const uint32_t slot = base + (uint32_t)(lane - my_head);
                 a.payload[slot] = ((uint32_t)m << kTBits) | (uint32_t)t;
                 a.cls[slot] = (uint8_t)c;
-                if (a.samples) a.samples_b[slot] = __ldg(&a.samples[(size_t)m * a.nH + t]);
+                if (a.samples) a.samples_b[slot] = a.samples[(size_t)m * a.nH + t];
             }
         }
     }
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN,
                         const int g = min(max(__ldg(&a.gid[m]), 0), a.n_ctf - 1);
                         pt[j].w = __float_as_uint(__ldg(&a.h2[(size_t)g * a.nH + t]));
                     }
-                    if (CH >= 2) wv[j] = __ldg(&a.samples[(size_t)m * a.nH + t]);
+                    if (CH >= 2) wv[j] = a.samples[(size_t)m * a.nH + t];
                 } else {
                     c[j] = region_base<W, BZ>(p, bx * kBrick, by * kBrick, bz * BZ) & 31;
                 }
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(256) k_bin_scatter2d(BinArgs a, int M, int hN,
             } else {
                 a.payload[slot] = ((uint32_t)(m0 + j) << kTBits) | (uint32_t)t;
                 a.cls[slot] = (uint8_t)c[j];
-                if (a.samples) a.samples_b[slot] = __ldg(&a.samples[(size_t)(m0 + j) * a.nH + t]);
+                if (a.samples) a.samples_b[slot] = a.samples[(size_t)(m0 + j) * a.nH + t];
             }
         }
     }
@@ -268,10 +268,10 @@ __device__ __forceinline__ void block_scan2(unsigned long long& ip, long long& i
 }
 
 template <bool WRITE>
-__global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* __restrict__ count,
-                                                              uint32_t* __restrict__ cursor, int nbricks,
-                                                              ScanPart* __restrict__ part, int4* __restrict__ work,
-                                                              int* __restrict__ counters, int max_work, int chunk) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* count,
+                                                              uint32_t* cursor, int nbricks,
+                                                              ScanPart* part, int4* work,
+                                                              int* counters, int max_work, int chunk) {
     pdl_wait();
     pdl_launch();
     __shared__ ScanPart s_w[32], s_tot;
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* __
 }
 
 // Exclusive scan of the per-block totals in place (one block; n <= 32 * kScanThreads).
-__global__ void __launch_bounds__(kScanThreads) k_scan_parts(ScanPart* __restrict__ part, int n) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_parts(ScanPart* part, int n) {
     pdl_wait();
     pdl_launch();
     __shared__ ScanPart s_w[32], s_tot;
@@ -367,10 +367,10 @@ constexpr int kSortSmem = kChunk * (4 + 1) + kSortLevels * (4 + 4);   // ids, cl
 // to payload; inv_perm != nullptr receives, at each point's scatter position, its
 // position in the sorted piece (the fused form's weight gather walks the points in
 // scatter order, where the points of one image sit together).
-__global__ void __launch_bounds__(256) k_class_sort(uint32_t* __restrict__ payload, const uint8_t* __restrict__ cls,
-                                                    const int4* __restrict__ work, const int* __restrict__ counters,
-                                                    uint16_t* __restrict__ perm, const uint32_t* __restrict__ in,
-                                                    uint16_t* __restrict__ inv_perm) {
+__global__ void __launch_bounds__(256) k_class_sort(uint32_t* payload, const uint8_t* cls,
+                                                    const int4* work, const int* counters,
+                                                    uint16_t* perm, const uint32_t* in,
+                                                    uint16_t* inv_perm) {
     pdl_wait();
     pdl_launch();
     extern __shared__ uint32_t sm_u[];
@@ -633,7 +633,7 @@ constexpr int kSpreadWarps = kSpreadThreads / 32;
 // starting at p0.
 __device__ __forceinline__ float2 point_weight(const SpreadArgs& a, bool cplx, int m, int t, uint32_t p0,
                                                uint32_t pos) {
-    if (cplx) return __ldg(&a.samples_b[p0 + __ldg(&a.perm[pos])]);
+    if (cplx) return a.samples_b[p0 + a.perm[pos]];
     const int g = min(max(__ldg(&a.gid[m]), 0), a.n_ctf - 1);
     return make_float2(__ldg(&a.h2[(size_t)g * a.nH + t]), 0.0f);
 }
@@ -712,12 +712,12 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
             // the piece's A*b weights sit in its own window of samples_b (scatter order):
             // read it straight, coalesced, instead of through the ids and permutation
             for (int j = threadIdx.x; j < wk.z; j += kSpreadThreads) {
-                const float2 wv = __ldg(&a.samples_b[wk.y + j]);
+                const float2 wv = a.samples_b[wk.y + j];
                 wmax = fmaxf(wmax, fmaxf(fabsf(wv.x), fabsf(wv.y)));
             }
         } else {
             for (int i = 0; i < my_n; ++i) {
-                const uint32_t id = __ldg(&a.payload[s0 + kSpreadThreads * i]);
+                const uint32_t id = a.payload[s0 + kSpreadThreads * i];
                 const float2 wv = point_weight(a, CPLX, (int)(id >> kTBits), (int)(id & ((1u << kTBits) - 1u)),
                                                (uint32_t)wk.y, s0 + kSpreadThreads * i);
                 wmax = fmaxf(wmax, fmaxf(fabsf(wv.x), fabsf(wv.y)));
@@ -746,7 +746,7 @@ __device__ __forceinline__ void spread_piece(const SpreadArgs& a, const KbPoly& 
             PointPos p{};
             int base = -1;
             if (live) {
-                id = __ldg(&a.payload[s0 + kSpreadThreads * i]);
+                id = a.payload[s0 + kSpreadThreads * i];
                 p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.ls, a.halfG,
                               a.G);
                 base = region_base<W, BZ>(p, lo0, lo1, lo2);
@@ -868,7 +868,7 @@ __global__ void __launch_bounds__(kSpreadThreads, CPLX ? 5 : 6) k_spread_batch(c
             int lo = 0, hi = n;                        // last p with item_off[p] <= g
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (__ldg(&item_off[mid]) <= g) lo = mid; else hi = mid;
+                if (item_off[mid] <= g) lo = mid; else hi = mid;
             }
             s_item = g;
             s_prob = lo;
@@ -878,7 +878,7 @@ __global__ void __launch_bounds__(kSpreadThreads, CPLX ? 5 : 6) k_spread_batch(c
         if (g >= total) break;
         const int pi = s_prob;
         const SpreadArgs a = desc[pi];
-        spread_piece<W, CPLX>(a, poly, a.work[g - __ldg(&item_off[pi])], lev1, lev2, s_red);
+        spread_piece<W, CPLX>(a, poly, a.work[g - item_off[pi]], lev1, lev2, s_red);
     }
 }
 
@@ -948,7 +948,7 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
     const uint32_t s0 = (uint32_t)wk.y + threadIdx.x;
     const int my_n = wk.z > (int)threadIdx.x ? (wk.z - (int)threadIdx.x + T - 1) / T : 0;
     // largest |h b| of the piece (the A*b scale), found by the gather pass
-    const float wmax = __ldg(&a.wmax_item[item]);
+    const float wmax = a.wmax_item[item];
     constexpr int PPR = FusedRound<T>::PPR, SB = FusedRound<T>::kScaleBits;
     const int rounds = (((wk.z + T - 1) / T) + PPR - 1) / PPR;
     int ek = 0, eb = 0;
@@ -965,7 +965,7 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
             PointPos p{};
             int base = -1;
             if (live) {
-                id = __ldg(&a.payload[s0 + T * i]);
+                id = a.payload[s0 + T * i];
                 p = point_pos(a.geom[id >> kTBits], __ldg(&a.htab[id & ((1u << kTBits) - 1u)]), a.ls, a.halfG,
                               a.G);
                 base = region_base<W, BZ>(p, lo0, lo1, lo2);
@@ -979,7 +979,7 @@ __device__ __forceinline__ void spread_piece_fused(const SpreadArgs& a, const Kb
             const int t = (int)(id & ((1u << kTBits) - 1u));
             const int g = min(max(__ldg(&a.gid[m]), 0), a.n_ctf - 1);
             const float wk2 = __ldg(&a.h2[(size_t)g * a.nH + t]) * Sk;
-            const float2 wv = __ldg(&a.samples_b[s0 + T * i]);     // gathered in payload order
+            const float2 wv = a.samples_b[s0 + T * i];     // gathered in payload order
             const float2 w2 = make_float2(wv.x * Sb, wv.y * Sb);
             const float dth = point_dither(id);
             float wx[W], wy[W], wz[W];
@@ -1062,11 +1062,11 @@ __global__ void __launch_bounds__(kFusedThreads) k_spread_fused(const SpreadArgs
 // The fused pass's A*b weights in payload order (samples_b[pos] = h b of the point at
 // pos, one gathered 8-byte read per point) and each work item's largest |h b| (its
 // fixed-point scale), so the spreading pass reads both coalesced.
-__global__ void __launch_bounds__(256) k_fused_gather(const uint32_t* __restrict__ scat,
-                                                      const uint16_t* __restrict__ inv_perm,
-                                                      const int4* __restrict__ work, const int* __restrict__ counters,
-                                                      const float2* __restrict__ samples, int nH,
-                                                      float2* __restrict__ samples_b, float* __restrict__ wmax_item) {
+__global__ void __launch_bounds__(256) k_fused_gather(const uint32_t* scat,
+                                                      const uint16_t* inv_perm,
+                                                      const int4* work, const int* counters,
+                                                      const float2* samples, int nH,
+                                                      float2* samples_b, float* wmax_item) {
     pdl_wait();
     pdl_launch();
     __shared__ float s_red[8];
@@ -1078,9 +1078,9 @@ __global__ void __launch_bounds__(256) k_fused_gather(const uint32_t* __restrict
         // the points in scatter order (an image's points of this brick together: their
         // weights share sectors), each written to its sorted position
         for (int i = threadIdx.x; i < wk.z; i += blockDim.x) {
-            const uint32_t id = __ldg(&scat[wk.y + i]);
-            const float2 v = __ldg(&samples[(size_t)(id >> kTBits) * nH + (id & ((1u << kTBits) - 1u))]);
-            samples_b[wk.y + __ldg(&inv_perm[wk.y + i])] = v;
+            const uint32_t id = scat[wk.y + i];
+            const float2 v = samples[(size_t)(id >> kTBits) * nH + (id & ((1u << kTBits) - 1u))];
+            samples_b[wk.y + inv_perm[wk.y + i]] = v;
             wmax = fmaxf(wmax, fmaxf(fabsf(v.x), fabsf(v.y)));
         }
 #pragma unroll
@@ -1321,7 +1321,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
             gy -= (gy >= a.G) ? a.G : 0;
             gz += (gz < 0) ? a.G : 0;
             gz -= (gz >= a.G) ? a.G : 0;
-            s_g[i] = __ldg(&a.ghat[((size_t)gz * a.G + gy) * a.G + gx]);
+            s_g[i] = a.ghat[((size_t)gz * a.G + gy) * a.G + gx];
         }
         __syncthreads();
         // residuals and sums in FP64 (as double-words they would be 48 bits within FP32's
@@ -1329,7 +1329,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
         double acc_r = 0.0, acc_b = 0.0;
         for (int i = threadIdx.x; i < wk.z; i += blockDim.x) {
             const uint32_t pos = (uint32_t)wk.y + i;
-            const uint32_t id = __ldg(&a.payload[pos]);
+            const uint32_t id = a.payload[pos];
             const int m = (int)(id >> kTBits);
             const int t = (int)(id & ((1u << kTBits) - 1u));
             const PointPos p = point_pos(a.geom[m], __ldg(&a.htab[t]), a.ls, a.halfG, a.G);
@@ -1360,7 +1360,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
             if (!RESID) {
                 a.out[(size_t)m * a.nH + t] = make_float2(h * f.x, h * f.y);
             } else {
-                const float2 bv = __ldg(&a.samples_b[wk.y + __ldg(&a.perm[pos])]);
+                const float2 bv = a.samples_b[wk.y + a.perm[pos]];
                 const double bx = bv.x, by = bv.y, hd = h;
                 const double dr = bx - hd * f.x, di = by - hd * f.y;
                 const double c = t == 0 ? 1.0 : 2.0;       // off the origin: the conjugate half too
@@ -1390,8 +1390,8 @@ __global__ void __launch_bounds__(kSpreadThreads) k_interp(const InterpArgs a) {
 }
 
 // out[0..1] = sums over the work items, in item order (one CTA: fixed order).
-__global__ void __launch_bounds__(1024) k_item_sum(const double* __restrict__ part, const int* __restrict__ counters,
-                                                   double* __restrict__ out) {
+__global__ void __launch_bounds__(1024) k_item_sum(const double* part, const int* counters,
+                                                   double* out) {
     pdl_wait();
     pdl_launch();
     __shared__ double s[2][1024];

@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
 #pragma unroll
         for (int u = 0; u < PT; ++u) {
             const int i = u * kSortThreads + tid;
-            if (i < wk.z) pt[u] = __ldg(&a.pts[wk.y + i]);
+            if (i < wk.z) pt[u] = a.pts[wk.y + i];
         }
     };
     fetch();
@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
             for (int u = 0; u < PT; ++u) {
                 const int i = u * kSortThreads + tid;
                 if (i >= wk.z) continue;
-                const float2 v = CH == 3 ? __ldg(&a.pts_w[wk.y + i])
-                                         : make_float2(__uint_as_float(pt[u].w), __ldg(&im2[wk.y + i]));
+                const float2 v = CH == 3 ? a.pts_w[wk.y + i]
+                                         : make_float2(__uint_as_float(pt[u].w), im2[wk.y + i]);
                 const float w = fmaxf(fabsf(v.x), fabsf(v.y));
                 wmax = fmaxf(wmax, w);
                 wsum += w;
@@ -301,12 +301,12 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
             const float w0 = __uint_as_float(pt[u].w);
             if (CH == 2) {
                 w[0] = w0 * Sb;
-                w[CH - 1] = __ldg(&im2[wk.y + i]) * Sb;
+                w[CH - 1] = im2[wk.y + i] * Sb;
             } else {
                 w[0] = w0 * Sk;
             }
             if (CH == 3) {
-                const float2 v = __ldg(&a.pts_w[wk.y + i]);
+                const float2 v = a.pts_w[wk.y + i];
                 w[CH - 2] = v.x * Sb;
                 w[CH - 1] = v.y * Sb;
             }
@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma_batch(const Sprea
             int lo = 0, hi = n;                        // last p with item_off[p] <= g
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (__ldg(&item_off[mid]) <= g) lo = mid; else hi = mid;
+                if (item_off[mid] <= g) lo = mid; else hi = mid;
             }
             s_item = g;
             s_prob = lo;
@@ -613,7 +613,7 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma_batch(const Sprea
         if (g >= total) break;
         const int pi = s_prob;
         const SpreadArgs& a = desc[pi];
-        spread_item_mma<W, CH>(a, poly, a.rec_item[g - __ldg(&item_off[pi])], lev1, wbuf);
+        spread_item_mma<W, CH>(a, poly, a.rec_item[g - item_off[pi]], lev1, wbuf);
     }
 }
 
