@@ -172,6 +172,7 @@ size_t layout_workspace(const firm_params& p, char* base, Workspace& w) {
     w.work = c.take<int4>(max_work);
     w.wmax_item = c.take<float>(max_work);
     w.rec_item = c.take<int4>(max_work);
+    w.pass = c.take<int4>(kMmaMaxPasses + 1);
     w.scan_part = c.take<unsigned long long>(2 * (nb3 / kScanSpan + 1));
     w.item_part = c.take<double>(2 * max_work);
     w.counters = c.take<int>(8);
@@ -182,8 +183,10 @@ size_t layout_workspace(const firm_params& p, char* base, Workspace& w) {
                                        Gr * Gr * Gr * 2 * sizeof(double));
     w.grid = c.take<double>(grid_bytes / sizeof(double));
     // fused plans keep the kernel channel's ids in scatter order for the weight gather
-    w.payload_scat = fused ? c.take<uint32_t>(M * nH) : nullptr;
-    w.inv_perm = fused ? c.take<uint16_t>(M * nH) : nullptr;
+    // (up to where the tensor-core form takes over)
+    const size_t scat = (size_t)std::min((double)(M * nH), mma_least(p, (int)nbk, 3));
+    w.payload_scat = fused ? c.take<uint32_t>(scat) : nullptr;
+    w.inv_perm = fused ? c.take<uint16_t>(scat) : nullptr;
     // union: staged images | point ids | FFT intermediates (never live together)
     const size_t fx1 = std::max({Gk * Gk * (N + 1), Gr * Gr * N, H3});
     const size_t fx2 = std::max({Gk * 2 * N * (N + 1), Gr * N * N, H3});
@@ -194,9 +197,9 @@ size_t layout_workspace(const firm_params& p, char* base, Workspace& w) {
     const size_t pay_bytes = (ids_bytes + cls_bytes + smp_bytes + M * nH * sizeof(uint16_t) + 255) & ~(size_t)255;
     // tensor-core spreading: 4 words a record slot for the kernel channel, 5 for A*b, 6 fused
     const int nb_k = (int)nbk, nb_r = (int)(Gr / kBrick);
-    const bool mma_k = mma_rule(p, M * nH, nb_k, 1) || (fused && mma_rule(p, M * nH, nb_k, 3));
-    const size_t slots_k = mma_k ? mma_slots(M * nH, nb_k) : 0;
-    const size_t slots_r = mma_rule(p, M * nH, nb_r, 2) ? mma_slots(M * nH, nb_r) : 0;
+    auto mma = [&](int nb, int ch) { return (double)(M * nH) >= mma_least(p, nb, ch); };
+    const size_t slots_k = mma(nb_k, 1) || (fused && mma(nb_k, 3)) ? mma_slots(M * nH, nb_k) : 0;
+    const size_t slots_r = mma(nb_r, 2) ? mma_slots(M * nH, nb_r) : 0;
     const size_t rec_words = std::max(slots_k * (fused ? 6 : 4), slots_r * 5);
     // points: 16 B, and with A*b the imaginary part, or fused both parts of its weight
     const size_t pts_each = sizeof(uint4) + (fused ? sizeof(float2) : slots_r ? sizeof(float) : 0);
@@ -726,7 +729,7 @@ int firm_kernel_backproject(firm_plan_t plan, int M, const void* images, const d
     FIRM_CK(launch_geom(P, P.cur_R, M));
     tm.start(0);
     FIRM_CK(launch_bin_count(P, M, 3, BinFor::spread));
-    const bool place_first = !host_copy && !P.bin_mma;
+    const bool place_first = !host_copy && !P.bin_passes;
     if (place_first) FIRM_CK(launch_bin_place(P, M, 3));
     tm.stop();
     if (staged) {

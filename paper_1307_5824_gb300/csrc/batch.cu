@@ -110,11 +110,19 @@ bool same_items(const std::vector<firm_batch_item>& a, const firm_batch_item* b,
         if (e_ != cudaSuccess) return e_;         \
     } while (0)
 
-// Plans of the batch whose points are spread in the tensor-core form.
-int count_mma(const firm_batch_s& b, const firm_batch_item* items, bool kc) {
-    int c = 0;
-    for (int i = 0; i < b.n; ++i) c += spread_uses_mma(b.plans[i]->P, items[i].M, kc ? 1 : 2) ? 1 : 0;
-    return c;
+// Plans of the batch by the form their points are spread in: bank classes, or one pass of the
+// tensor-core form (plans of several passes spread on their own).
+struct Forms {
+    int bank = 0, mma = 0;
+};
+Forms count_forms(const firm_batch_s& b, const firm_batch_item* items, bool kc) {
+    Forms f;
+    for (int i = 0; i < b.n; ++i) {
+        const int passes = spread_passes(b.plans[i]->P, items[i].M, kc ? 1 : 2);
+        f.bank += passes == 0;
+        f.mma += passes == 1;
+    }
+    return f;
 }
 
 // Everything up to (not including) the kernel-channel spreading, for one plan.
@@ -131,7 +139,7 @@ cudaError_t plan_front(Plan& P, const firm_batch_item& it, bool spread_here) {
     BCK(launch_geom(P, P.cur_R, M));
     BCK(launch_bin(P, M, true, BinFor::spread));
     BCK(launch_spread_clear(P, true));
-    if (spread_here) BCK(launch_spread_only(P, M, true));
+    if (spread_here || P.bin_passes > 1) BCK(launch_spread_only(P, M, true));
     P.last_M = M;
     if (M > 0) BCK(launch_view_axis(P, P.cur_R, M));     // the preconditioners' cone axis
     return cudaSuccess;
@@ -147,7 +155,7 @@ cudaError_t plan_middle(Plan& P, const firm_batch_item& it, bool spread_here) {
     BCK(launch_image_dft(P, M, P.cur_images, P.cur_shifts, P.cur_gid));
     BCK(launch_bin(P, M, false, BinFor::spread));
     BCK(launch_spread_clear(P, false));
-    if (spread_here) BCK(launch_spread_only(P, M, false));
+    if (spread_here || P.bin_passes > 1) BCK(launch_spread_only(P, M, false));
     return cudaSuccess;
 }
 
@@ -251,18 +259,19 @@ cudaError_t enqueue_body(firm_batch_s& b, const firm_batch_item* items, int iter
     }
     if (persistent) {
         BCK(join(b));
-        const int mk = count_mma(b, items, true), mr = count_mma(b, items, false);
-        BCK(launch_spread_batch(b.n, mk, true, b.W, b.poly, b.desc_k, b.item_off, b.queue, b.num_sms, b.main));
-        own += 2 * ((mk > 0) + (mk < b.n));
+        const Forms fk = count_forms(b, items, true), fr = count_forms(b, items, false);
+        BCK(launch_spread_batch(fk.bank, fk.mma, b.n, true, b.W, b.poly, b.desc_k, b.item_off, b.queue, b.num_sms,
+                                b.main));
+        own += 2 * ((fk.mma > 0) + (fk.bank > 0));
         BCK(fork(b));
         for (int k = 0; k < b.n; ++k) {
             const int i = b.order[k];
             BCK(plan_middle(b.plans[i]->P, items[i], false));
         }
         BCK(join(b));
-        BCK(launch_spread_batch(b.n, mr, false, b.W, b.poly, b.desc_r, b.item_off + 2 * (b.n + 1), b.queue + 2,
-                                b.num_sms, b.main));
-        own += 2 * ((mr > 0) + (mr < b.n));
+        BCK(launch_spread_batch(fr.bank, fr.mma, b.n, false, b.W, b.poly, b.desc_r, b.item_off + 2 * (b.n + 1),
+                                b.queue + 2, b.num_sms, b.main));
+        own += 2 * ((fr.mma > 0) + (fr.bank > 0));
         BCK(fork(b));
     }
     if (!solve) {

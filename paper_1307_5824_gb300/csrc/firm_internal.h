@@ -23,6 +23,12 @@ constexpr int kMinChunk = 1024;       // smallest work-item size a plan may be t
 // 27 classes, an item's records starting at a multiple of 16 slots.
 constexpr int kMmaChunk = 4096;
 constexpr int kMmaPad = 27 * 15 + 15;
+// The records are made and spread in passes over the work items, of this many slots each, so
+// that their buffer (20 to 24 bytes a slot) does not grow with the images: 1.6 GB at most.  A pass
+// costs two kernels' tails (both channels at N = 128, 50,000 images: 32.0 ms in 7 passes, 31.9 in 4
+// of twice the size, 31.8 in one of 11 GB).
+constexpr unsigned kMmaPassSlots = 1u << 26;
+constexpr int kMmaMaxPasses = 40;     // 37 at the limit of 2^31 points
 constexpr int kMaxBatch = 1024;       // most plans one batch holds
 constexpr int kTBits = 13;            // point id = m << kTBits | t (t < 8192)
 constexpr int kMaxHist = 20001;       // residual history capacity (iterations + 1)
@@ -108,11 +114,11 @@ struct Workspace {
     float2* pts_w = nullptr;        //   (h^2; A*b: its real part), and the other weights
     uint32_t* rec = nullptr;        //   sorted, padded point records
     uint8_t* rec_cls = nullptr;     //   the class of every 16 slots
+    int4* pass = nullptr;           //   per pass: (first item, items sorted, record groups taken, items spread)
     int4* rec_item = nullptr;       //   per work item: (brick, first slot, groups, scales)
     unsigned long long* scan_part = nullptr;   // brick scan: per-block (points, items) totals
     double* item_part = nullptr;    // per work item: two FP64 partial sums (data residual)
-    int* counters = nullptr;        // [0] work items, [1] work cursor, [2] error flag, [3] sort cursor,
-                                    // [4] record slots taken (in 16s)
+    int* counters = nullptr;        // [0] work items, [1] work cursor, [2] error flag
     double* grid = nullptr;         // fine grid, FP64 (real for Ker, complex for A*b)
     float2* fx1 = nullptr;          // FFT intermediates
     float2* fx2 = nullptr;
@@ -173,7 +179,7 @@ struct Plan {
     long long launches = 0;         // kernels launched by this plan
     int pc_mode = 0;                // FIRM_PRECOND_*
     bool pc_ready = false;          // pc_diag built for the current K-hat and mode
-    bool bin_mma = false;           // the binned points are ordered for the tensor-core form
+    int bin_passes = 0;             // passes of the tensor-core form the points are binned for; 0: bank classes
     int last_M = 0;                 // images of the last firm_kernel
     int bin_M = -1;                 // images of the last firm_bin (its ids and items still held); -1 none
     bool bin_kc = true;             // channel of the last firm_bin (true: kernel, 4N grid)
@@ -219,11 +225,11 @@ inline cudaError_t launch_bin(Plan& P, int M, bool kernel_channel, BinFor use) {
     const cudaError_t e = launch_bin_count(P, M, kernel_channel ? 1 : 2, use);
     return e != cudaSuccess ? e : launch_bin_place(P, M, kernel_channel ? 1 : 2);
 }
-// Whether M images of a plan are spread in the tensor-core form (points: all of them, on a
-// grid of nb bricks per axis), and the record slots that can take.
-bool mma_rule(const firm_params& p, size_t points, int nb, int ch);
-size_t mma_slots(size_t points, int nb);
-bool spread_uses_mma(const Plan& P, int M, int ch);
+// The tensor-core form's rule on the number of points (on a grid of nb bricks per axis), its
+// record slots, and the passes that M images of a plan take in it.
+double mma_least(const firm_params& p, int nb, int ch);       // points from which it is taken
+size_t mma_slots(size_t points, int nb);                       // of the buffer: one pass
+int spread_passes(const Plan& P, int M, int ch);              // 0: bank classes
 cudaError_t launch_spread(Plan& P, int M, bool kernel_channel);        // clear + spread
 cudaError_t launch_spread_clear(Plan& P, bool kernel_channel);          // zero the fine grid
 cudaError_t launch_spread_only(Plan& P, int M, bool kernel_channel);    // spread (grid cleared)
@@ -239,9 +245,9 @@ cudaError_t launch_fused_gather(Plan& P, int M);
 // array of n per-plan descriptors; item_off: device (n + 1) ints; queue: device int.
 size_t spread_batch_desc_bytes();
 void spread_batch_fill_desc(Plan& P, int M, bool kernel_channel, void* host_desc);
-// n_mma of the plans are binned for the tensor-core form: their items go in a launch of
-// their own.  item_off: 2 (n + 1) ints, queue: 2 ints.
-cudaError_t launch_spread_batch(int n, int n_mma, bool kernel_channel, int W, const KbPoly& poly, const void* dev_desc,
+// n_bank of the n plans are binned for bank classes and n_mma for one pass of the tensor-core
+// form: a launch each.  Plans of several passes spread on their own.  item_off: 2 (n + 1) ints, queue: 2 ints.
+cudaError_t launch_spread_batch(int n_bank, int n_mma, int n, bool kernel_channel, int W, const KbPoly& poly, const void* dev_desc,
                                 int* item_off, int* queue, int num_sms, cudaStream_t s);
 
 // ---- launchers (fft_passes.cu) ----

@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "dw.cuh"
 #include "firm_internal.h"
@@ -271,7 +272,7 @@ template <bool WRITE>
 __global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* count,
                                                               uint32_t* cursor, int nbricks,
                                                               ScanPart* part, int4* work,
-                                                              int* counters, int max_work, int chunk) {
+                                                              int* counters, int4* pass, int max_work, int chunk) {
     pdl_wait();
     pdl_launch();
     __shared__ ScanPart s_w[32], s_tot;
@@ -309,8 +310,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_bricks(const uint32_t* co
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) {
         counters[0] = (int)min(woff, (long long)max_work);
         counters[1] = 0;
-        counters[3] = 0;
-        counters[4] = 0;
+        pass[0] = make_int4(0, 0, 0, 0);               // one pass over all items (else k_mma_passes)
+        pass[1] = make_int4(counters[0], 0, 0, 0);
     }
 }
 
@@ -342,10 +343,10 @@ static void launch_scan(Plan& P, int nbricks, int chunk) {
     const int nblk = (nbricks + kScanSpan - 1) / kScanSpan;
     ScanPart* part = reinterpret_cast<ScanPart*>(w.scan_part);
     launch_pdl(k_scan_bricks<false>, nblk, kScanThreads, 0, P.stream, w.count, w.cursor, nbricks, part, w.work,
-                                                               w.counters, (int)P.max_work, chunk);
+                                                               w.counters, w.pass, (int)P.max_work, chunk);
     launch_pdl(k_scan_parts, 1, kScanThreads, 0, P.stream, part, nblk);
     launch_pdl(k_scan_bricks<true>, nblk, kScanThreads, 0, P.stream, w.count, w.cursor, nbricks, part, w.work,
-                                                              w.counters, (int)P.max_work, chunk);
+                                                              w.counters, w.pass, (int)P.max_work, chunk);
     P.launches += 3;
 }
 
@@ -467,12 +468,12 @@ __global__ void __launch_bounds__(256) k_class_sort(uint32_t* payload, const uin
 }
 
 // The class sort of a plan's binned points (not the tensor-core form, which sorts its own).
-static void launch_class_sort(Plan& P, bool kc) {
+static void launch_class_sort(Plan& P, int ch) {
     Workspace& w = P.ws;
     cudaFuncSetAttribute(k_class_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, kSortSmem);
-    const bool keep = kc && w.payload_scat;       // fused plans keep the scatter order
+    const bool keep = ch == 3;                    // the fused form's weight gather walks the scatter order
     launch_pdl(k_class_sort, P.num_sms * 4, 256, kSortSmem, P.stream, w.payload, w.cls, w.work, w.counters,
-                                                               kc ? nullptr : w.perm, keep ? w.payload_scat : nullptr,
+                                                               ch != 2 ? nullptr : w.perm, keep ? w.payload_scat : nullptr,
                                                                keep ? w.inv_perm : nullptr);
     P.launches += 1;
 }
@@ -492,7 +493,7 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
     const dim3 g((n_tiles + 7) / 8, (unsigned)(mb < 65535 ? mb : 65535));
     const int4* col = P.ws.colinfo;
     const bool sm = a.samples != nullptr;
-    if (P.bin_mma) {
+    if (P.bin_passes) {
         if (kc && sm) launch_pdl(k_bin_scatter2d<W, true, 3>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
         else if (kc) launch_pdl(k_bin_scatter2d<W, true, 1>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
         else launch_pdl(k_bin_scatter2d<W, false, 2>, g, 256, 0, P.stream, a, M, hN, col, tiles_x, n_tiles);
@@ -521,35 +522,46 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 // gives the same volume from both.  Both channels in one pass
 // at W = 7 would need 96 accumulators a thread, and W = 8 windows leave one first tap a
 // class: neither is built.
-// The points and their records take up to 48 bytes a point where ids take 15.  At W = 7 (1.1 to
-// 1.6 times the bank-class form's rate, 2 at W = 6) that is taken up to 4 GiB, which keeps the
-// workspace of any plan of up to 50,000 images below 10 GiB.  By the plan's number of images,
-// not the call's: a plan laid out without records never takes a call that needs them.
-constexpr double kMmaMostW7 = 4.294967296e9 / 48;
-bool mma_rule(const firm_params& p, size_t points, int nb, int ch) {
+// The points take 16 bytes, 20 with A*b and 24 with both channels, where ids and what goes
+// with them take 15, and the records of a pass up to 1.6 GB.  At W = 7 (1.1 to 1.6 times the
+// bank-class form's rate, 2 at W = 6) that is taken up to 9e7 points, 13,907 images at N = 128,
+// which keeps the workspace of separate-channel plans of up to 50,000 images below 10 GiB.  By the
+// plan's number of images, not the call's: a plan laid out without records never takes a call
+// that needs them.
+constexpr double kMmaMostW7 = 8.948e7;
+double mma_least(const firm_params& p, int nb, int ch) {
     double least;
     if (p.W == 6) least = ch == 1 ? 600.0 : ch == 2 ? 400.0 : 235.0;
     else if (p.W == 7 && ch < 3 && (double)p.M * p.N * p.N * 0.3927 <= kMmaMostW7) least = ch == 1 ? 600.0 : 400.0;
-    else return false;
-    return (double)points >= least * 0.5236 * nb * nb * (double)nb;
+    else return 1e300;
+    return std::ceil(least * 0.5236 * nb * nb * (double)nb);
 }
 
-size_t mma_slots(size_t points, int nb) {
+// Slots of all items, each with the most padding.
+static size_t all_slots(size_t points, int nb) {
     const size_t items = std::min((size_t)nb * nb * nb, points) + points / kMmaChunk;
     return points + items * kMmaPad;
 }
 
-bool spread_uses_mma(const Plan& P, int M, int ch) {
-    return mma_rule(P.p, (size_t)M * P.nH, ch == 2 ? P.nbr : P.nbk, ch);
+size_t mma_slots(size_t points, int nb) {
+    return std::min<size_t>(all_slots(points, nb), (size_t)kMmaPassSlots + kMmaChunk + kMmaPad);
 }
 
-static BinArgs bin_args(Plan& P, int M, bool kc) {
+int spread_passes(const Plan& P, int M, int ch) {
+    const int nb = ch == 2 ? P.nbr : P.nbk;
+    const size_t points = (size_t)M * P.nH;
+    if ((double)points < mma_least(P.p, nb, ch)) return 0;
+    return (int)((all_slots(points, nb) + kMmaPassSlots - 1) / kMmaPassSlots);
+}
+
+static BinArgs bin_args(Plan& P, int M, int ch) {
+    const bool kc = ch != 2;
     Workspace& w = P.ws;
     BinArgs a;
     a.geom = w.geom;
     a.htab = w.htab;
     a.count = w.count;
-    a.payload = kc && w.payload_scat && !P.bin_mma ? w.payload_scat : w.payload;
+    a.payload = ch == 3 && !P.bin_passes ? w.payload_scat : w.payload;
     a.cls = w.cls;
     a.samples = kc ? nullptr : w.samples;
     a.samples_b = w.samples_b;
@@ -581,11 +593,11 @@ cudaError_t launch_bin_count(Plan& P, int M, int ch, BinFor use) {
     const bool kc = ch != 2;
     const int nb = kc ? P.nbk : P.nbr;
     const int nbricks = nb * nb * (kc ? P.nbkz : P.nbr);
-    P.bin_mma = spread && spread_uses_mma(P, M, ch);
+    P.bin_passes = spread ? spread_passes(P, M, ch) : 0;
     cudaError_t e = cudaMemsetAsync(P.ws.count, 0, sizeof(uint32_t) * nbricks, P.stream);
     if (e != cudaSuccess) return e;
     if (M > 0) {
-        const BinArgs a = bin_args(P, M, kc);
+        const BinArgs a = bin_args(P, M, ch);
         switch (P.p.W) {
             case 6: bin_count_w<6>(P, a, M, kc); break;
             case 7: bin_count_w<7>(P, a, M, kc); break;
@@ -593,7 +605,7 @@ cudaError_t launch_bin_count(Plan& P, int M, int ch, BinFor use) {
             default: return cudaErrorInvalidValue;
         }
     }
-    launch_scan(P, nbricks, P.bin_mma ? kMmaChunk : use == BinFor::interp ? interp_chunk(P, M) : P.chunk);
+    launch_scan(P, nbricks, P.bin_passes ? kMmaChunk : use == BinFor::interp ? interp_chunk(P, M) : P.chunk);
     return cudaGetLastError();
 }
 
@@ -601,17 +613,19 @@ static SpreadArgs spread_args(Plan& P, bool kc);
 cudaError_t launch_bin_place(Plan& P, int M, int ch) {
     const bool kc = ch != 2;
     if (M <= 0) return cudaSuccess;
-    BinArgs a = bin_args(P, M, kc);
+    if (ch == 3 && !P.ws.payload_scat) return cudaErrorInvalidValue;      // fused plans only
+    BinArgs a = bin_args(P, M, ch);
     a.count = P.ws.cursor;
-    if (ch == 3 && P.bin_mma) a.samples = P.ws.samples;      // the A*b weights go with the points
+    if (ch == 3 && P.bin_passes) a.samples = P.ws.samples;      // the A*b weights go with the points
     switch (P.p.W) {
         case 6: bin_place_w<6>(P, a, M, kc); break;
         case 7: bin_place_w<7>(P, a, M, kc); break;
         case 8: bin_place_w<8>(P, a, M, kc); break;
         default: return cudaErrorInvalidValue;
     }
-    if (P.bin_mma) return launch_mma_sort(P, spread_args(P, kc), ch);
-    launch_class_sort(P, kc);
+    if (P.bin_passes == 1) return launch_mma_sort(P, spread_args(P, kc), ch, 0);
+    if (P.bin_passes) return launch_mma_passes(P);           // each pass sorts its items as it comes
+    launch_class_sort(P, ch);
     return cudaGetLastError();
 }
 
@@ -883,7 +897,7 @@ __global__ void __launch_bounds__(kSpreadThreads, CPLX ? 5 : 6) k_spread_batch(c
 }
 
 // item_off = exclusive prefix of the work-item counts of the plans of one form (mma 0 or
-// 1; the others count 0); queue = 0.  One warp.
+// 1; the others count 0, also those of several passes, 2, which spread on their own); queue = 0.  One warp.
 __global__ void k_batch_items(const SpreadArgs* __restrict__ desc, int n, int mma, int* __restrict__ item_off,
                               int* queue) {
     const int lane = threadIdx.x;
@@ -1156,7 +1170,7 @@ static SpreadArgs spread_args(Plan& P, bool kc) {
     a.rec = w.rec;
     a.rec_cls = w.rec_cls;
     a.rec_item = w.rec_item;
-    a.rec_slots = (uint32_t)std::min<size_t>(mma_slots((size_t)P.p.M * P.nH, kc ? P.nbk : P.nbr), 0xffffffffu);
+    a.rec_slots = (uint32_t)mma_slots((size_t)P.p.M * P.nH, kc ? P.nbk : P.nbr);
     a.work = w.work;
     a.counters = w.counters;
     a.geom = w.geom;
@@ -1173,7 +1187,8 @@ static SpreadArgs spread_args(Plan& P, bool kc) {
     a.nH = P.nH;
     a.n_ctf = P.n_ctf;
     a.ls = kc ? 2 : 1;
-    a.mma = P.bin_mma ? 1 : 0;
+    a.pass = w.pass;
+    a.mma = P.bin_passes ? 1 : 0;
     a.wmax_fixed = kc ? P.h2_max : 0.0f;
     a.wmax_item = nullptr;
     a.poly = P.poly;
@@ -1189,7 +1204,7 @@ cudaError_t launch_spread_clear(Plan& P, bool kc) {
 cudaError_t launch_spread_only(Plan& P, int M, bool kc) {
     if (M <= 0) return cudaSuccess;
     const SpreadArgs a = spread_args(P, kc);
-    if (P.bin_mma) return launch_spread_mma(P, a, kc ? 1 : 2);
+    if (P.bin_passes) return launch_spread_mma(P, a, kc ? 1 : 2);
     switch (P.p.W) {
         case 6: return kc ? spread_w<6, false>(P, a) : spread_w<6, true>(P, a);
         case 7: return kc ? spread_w<7, false>(P, a) : spread_w<7, true>(P, a);
@@ -1208,7 +1223,7 @@ cudaError_t launch_fused_gather(Plan& P, int M) {
     if (M <= 0) return cudaSuccess;
     Workspace& w = P.ws;
     if (!w.payload_scat) return cudaErrorInvalidValue;      // fused plans only
-    if (P.bin_mma) return cudaSuccess;                       // the spreading kernel gathers its weights itself
+    if (P.bin_passes) return cudaSuccess;                    // placed with the points
     launch_pdl(k_fused_gather, P.num_sms * 8, 256, 0, P.stream, w.payload_scat, w.inv_perm, w.work, w.counters, w.samples,
                                                        P.nH, w.samples_b, w.wmax_item);
     P.launches += 1;
@@ -1222,7 +1237,7 @@ cudaError_t launch_spread_fused(Plan& P, int M) {
     SpreadArgs a = spread_args(P, true);
     a.samples_b = P.ws.samples_b;
     a.wmax_item = P.ws.wmax_item;
-    if (P.bin_mma) return launch_spread_mma(P, a, 3);
+    if (P.bin_passes) return launch_spread_mma(P, a, 3);
     switch (P.p.W) {
         case 6: return spread_fused_w<6>(P, a);
         case 7: return spread_fused_w<7>(P, a);
@@ -1235,18 +1250,19 @@ size_t spread_batch_desc_bytes() { return sizeof(SpreadArgs); }
 
 void spread_batch_fill_desc(Plan& P, int M, bool kc, void* host_desc) {
     SpreadArgs a = spread_args(P, kc);
-    a.mma = spread_uses_mma(P, M, kc ? 1 : 2) ? 1 : 0;
+    a.mma = std::min(spread_passes(P, M, kc ? 1 : 2), 2);
     *reinterpret_cast<SpreadArgs*>(host_desc) = a;
 }
 
-cudaError_t launch_spread_batch(int n, int n_mma, bool kc, int W, const KbPoly& poly, const void* dev_desc,
+cudaError_t launch_spread_batch(int n_bank, int n_mma, int n, bool kc, int W, const KbPoly& poly, const void* dev_desc,
                                 int* item_off, int* queue, int num_sms, cudaStream_t s) {
     const SpreadArgs* d = reinterpret_cast<const SpreadArgs*>(dev_desc);
     if (n_mma > 0) {
         k_batch_items<<<1, 32, 0, s>>>(d, n, 1, item_off + n + 1, queue + 1);
         const cudaError_t e = launch_spread_mma_batch(n, kc, W, d, item_off + n + 1, queue + 1, poly, num_sms, s);
-        if (e != cudaSuccess || n_mma == n) return e;
+        if (e != cudaSuccess) return e;
     }
+    if (n_bank == 0) return cudaSuccess;
     switch (W) {
         case 6: return kc ? spread_batch_w<6, false>(n, d, item_off, queue, poly, num_sms, s)
                           : spread_batch_w<6, true>(n, d, item_off, queue, poly, num_sms, s);

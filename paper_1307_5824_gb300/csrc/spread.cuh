@@ -136,6 +136,7 @@ struct SpreadArgs {
     uint8_t* rec_cls;
     int4* rec_item;
     uint32_t rec_slots;
+    int4* pass;
     const int4* work;
     int* counters;
     const ImgGeom* geom;
@@ -148,7 +149,7 @@ struct SpreadArgs {
     double* grid;             // G^3 real, or G^3 complex interleaved (re, im)
     int G, halfG, nb, nH, n_ctf;
     int ls;                   // log2(G / N)
-    int mma;                  // 1: binned for the tensor-core form (spread_mma.cu)
+    int mma;                  // 1: binned for the tensor-core form (spread_mma.cu); in a batch 2: several passes
     float wmax_fixed;         // > 0: bound on |w| known in advance (no pre-pass)
     const float* wmax_item;   // fused form: per work item, the largest |h b| of its points
     KbPoly poly;
@@ -166,7 +167,8 @@ __device__ __forceinline__ uint32_t coord_word(int cell, uint32_t q) {
 }
 
 // Tensor-core form (spread_mma.cu); ch: 1 kernel channel, 2 A*b, 3 both.
-cudaError_t launch_mma_sort(Plan& P, const SpreadArgs& a, int ch);
+cudaError_t launch_mma_passes(Plan& P);
+cudaError_t launch_mma_sort(Plan& P, const SpreadArgs& a, int ch, int pass);
 cudaError_t launch_spread_mma(Plan& P, const SpreadArgs& a, int ch);
 cudaError_t launch_spread_mma_batch(int n, bool kc, int W, const SpreadArgs* desc, const int* item_off, int* queue,
                                     const KbPoly& poly, int num_sms, cudaStream_t s);

@@ -171,7 +171,7 @@ __device__ __forceinline__ void slot_taps(const MmaPoly& poly, uint2 c, uint32_t
 // Sort
 // ---------------------------------------------------------------------------
 template <int W, int CH>
-__global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a) {
+__global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a, int pass) {
     pdl_wait();
     pdl_launch();
     using C = MmaCfg<W, CH>;
@@ -181,9 +181,10 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
     __shared__ int s_hist[32], s_off[32], s_total, s_item, s_base;
     __shared__ float2 s_red[kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n_work = a.counters[0];
+    int4* const ps = a.pass + pass;
+    const int first = ps[0].x, n_work = ps[1].x;
     const float* const im2 = reinterpret_cast<const float*>(a.pts_w);      // A*b alone: imaginary parts
-    if (tid == 0) s_item = atomicAdd(&a.counters[3], 1);
+    if (tid == 0) s_item = first + atomicAdd(&ps->y, 1);
     __syncthreads();
     int item = s_item;
     int4 wk = make_int4(0, 0, 0, 0);
@@ -253,11 +254,11 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_mma_sort(const SpreadArgs a
             s_off[lane] = v - pad;
             if (lane == 31) {
                 s_total = v;
-                s_base = atomicAdd(&a.counters[4], v / 16);
+                s_base = atomicAdd(&ps->z, v / 16);
             }
         }
         __syncthreads();
-        if (tid == 0) s_item = atomicAdd(&a.counters[3], 1);               // the next item
+        if (tid == 0) s_item = first + atomicAdd(&ps->y, 1);               // the next item
         if (CH >= 2) {
             wmax = s_red[0].x;
             wsum = s_red[0].y;
@@ -563,7 +564,8 @@ __device__ __forceinline__ void spread_item_mma(const SpreadArgs& a, const MmaPo
 }
 
 template <int W, int CH>
-__global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs a, const __grid_constant__ MmaPoly poly) {
+__global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs a, const __grid_constant__ MmaPoly poly,
+                                                                     int pass) {
     pdl_wait();
     pdl_launch();
     using C = MmaCfg<W, CH>;
@@ -572,10 +574,11 @@ __global__ void __launch_bounds__(kMmaThreads, 2) k_spread_mma(const SpreadArgs 
     int* const lev1 = sm_mma + kMmaWarps * (C::kWarpWords + 8 * C::kRecWords);
     uint32_t* const wbuf = reinterpret_cast<uint32_t*>(sm_mma) + (threadIdx.x >> 5) * (C::kWarpWords + 8 * C::kRecWords);
     for (int i = threadIdx.x; i < CH * C::RG3; i += kMmaThreads) lev1[i] = 0;
-    const int n_work = a.counters[0];
+    int4* const ps = a.pass + pass;
+    const int first = ps[0].x, n_work = ps[1].x;
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(&a.counters[1], 1);
+        if (threadIdx.x == 0) s_item = first + atomicAdd(&ps->w, 1);
         __syncthreads();
         const int item = s_item;
         if (item >= n_work) break;
@@ -642,7 +645,7 @@ cudaError_t launch_spread_mma_batch(int n, bool kc, int W, const SpreadArgs* des
 }
 
 template <int W, int CH>
-static cudaError_t spread_mma_w(Plan& P, const SpreadArgs& a) {
+static cudaError_t spread_mma_w(Plan& P, const SpreadArgs& a, int pass) {
     constexpr size_t smem = MmaCfg<W, CH>::kSmem;
     cudaError_t e = cudaFuncSetAttribute(k_spread_mma<W, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -650,41 +653,78 @@ static cudaError_t spread_mma_w(Plan& P, const SpreadArgs& a) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_mma<W, CH>, kMmaThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    launch_pdl(k_spread_mma<W, CH>, P.num_sms * per_sm, kMmaThreads, smem, P.stream, a, mma_poly(a.poly, W));
+    launch_pdl(k_spread_mma<W, CH>, P.num_sms * per_sm, kMmaThreads, smem, P.stream, a, mma_poly(a.poly, W), pass);
     P.launches += 1;
     return cudaGetLastError();
 }
 
 template <int W, int CH>
-static cudaError_t mma_sort_w(Plan& P, const SpreadArgs& a) {
+static cudaError_t mma_sort_w(Plan& P, const SpreadArgs& a, int pass) {
     constexpr size_t smem = MmaCfg<W, CH>::kSortSmem;
     cudaError_t e = cudaFuncSetAttribute(k_mma_sort<W, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    launch_pdl(k_mma_sort<W, CH>, P.num_sms * 2, kSortThreads, smem, P.stream, a);
+    launch_pdl(k_mma_sort<W, CH>, P.num_sms * 2, kSortThreads, smem, P.stream, a, pass);
     P.launches += 1;
     return cudaGetLastError();
 }
 
-cudaError_t launch_mma_sort(Plan& P, const SpreadArgs& a, int ch) {
+// First item of every pass: the item before which `pass` buffers of slots are spoken for, with
+// all padding (an item's points and slots before it follow from its number and start).
+__global__ void k_mma_passes(const int4* work, const int* counters, int4* pass, int n) {
+    pdl_wait();
+    pdl_launch();
+    const int p = threadIdx.x;
+    if (p > n) return;
+    const unsigned at = (unsigned)p * kMmaPassSlots;          // 37 passes at most: below 2^32
+    int lo = 0, hi = counters[0];
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if ((unsigned)work[mid].y + (unsigned)mid * kMmaPad < at) lo = mid + 1;
+        else hi = mid;
+    }
+    pass[p] = make_int4(p == n ? counters[0] : lo, 0, 0, 0);
+}
+
+cudaError_t launch_mma_passes(Plan& P) {
+    static_assert(kMmaMaxPasses < 64 && (unsigned long long)kMmaMaxPasses * kMmaPassSlots < (1ull << 32), "pass offsets");
+    P.launches += 1;
+    return launch_pdl(k_mma_passes, 1, 64, 0, P.stream, P.ws.work, P.ws.counters, P.ws.pass, P.bin_passes);
+}
+
+cudaError_t launch_mma_sort(Plan& P, const SpreadArgs& a, int ch, int pass) {
     if (P.p.W == 7)
-        return ch == 1 ? mma_sort_w<7, 1>(P, a) : ch == 2 ? mma_sort_w<7, 2>(P, a) : cudaErrorInvalidValue;
+        return ch == 1   ? mma_sort_w<7, 1>(P, a, pass)
+               : ch == 2 ? mma_sort_w<7, 2>(P, a, pass)
+                         : cudaErrorInvalidValue;
     switch (ch) {
-        case 1: return mma_sort_w<6, 1>(P, a);
-        case 2: return mma_sort_w<6, 2>(P, a);
-        case 3: return mma_sort_w<6, 3>(P, a);
+        case 1: return mma_sort_w<6, 1>(P, a, pass);
+        case 2: return mma_sort_w<6, 2>(P, a, pass);
+        case 3: return mma_sort_w<6, 3>(P, a, pass);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+static cudaError_t spread_pass(Plan& P, const SpreadArgs& a, int ch, int pass) {
+    if (P.p.W == 7)
+        return ch == 1   ? spread_mma_w<7, 1>(P, a, pass)
+               : ch == 2 ? spread_mma_w<7, 2>(P, a, pass)
+                         : cudaErrorInvalidValue;
+    switch (ch) {
+        case 1: return spread_mma_w<6, 1>(P, a, pass);
+        case 2: return spread_mma_w<6, 2>(P, a, pass);
+        case 3: return spread_mma_w<6, 3>(P, a, pass);
         default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_spread_mma(Plan& P, const SpreadArgs& a, int ch) {
-    if (P.p.W == 7)
-        return ch == 1 ? spread_mma_w<7, 1>(P, a) : ch == 2 ? spread_mma_w<7, 2>(P, a) : cudaErrorInvalidValue;
-    switch (ch) {
-        case 1: return spread_mma_w<6, 1>(P, a);
-        case 2: return spread_mma_w<6, 2>(P, a);
-        case 3: return spread_mma_w<6, 3>(P, a);
-        default: return cudaErrorInvalidValue;
+    if (P.bin_passes == 1) return spread_pass(P, a, ch, 0);      // sorted with the placement
+    for (int p = 0; p < P.bin_passes; ++p) {
+        cudaError_t e = launch_mma_sort(P, a, ch, p);
+        if (e == cudaSuccess) e = spread_pass(P, a, ch, p);
+        if (e != cudaSuccess) return e;
     }
+    return cudaSuccess;
 }
 
 }  // namespace firm
