@@ -780,9 +780,8 @@ __global__ void __launch_bounds__(PlaneCfg<L, L / 2>::kThreads) k_toep_plane_inv
 }
 
 template <int L, class Op>
-__global__ void __launch_bounds__(kThreads) k_rows_cg(Op op, const CgState* cg) {
+__global__ void __launch_bounds__(kThreads) k_rows_post(Op op) {
     extern __shared__ float2 S[];
-    if (cg && cg->done) return;
     constexpr int ROWS = rows_per_block<L>();
     const int r0 = blockIdx.x * ROWS;
     const int nl = min(ROWS, op.n_rows - r0);
@@ -796,9 +795,8 @@ __global__ void __launch_bounds__(kThreads) k_rows_cg(Op op, const CgState* cg) 
 }
 
 template <int L, int SIGN, class Op>
-__global__ void __launch_bounds__(kThreads) k_cols_cg(const Op op, const CgState* cg) {
+__global__ void __launch_bounds__(kThreads) k_cols_plain(const Op op) {
     extern __shared__ float2 S[];
-    if (cg && cg->done) return;
     const int tiles = (op.n_inner + TX<L>() - 1) / TX<L>();
     const int outer = blockIdx.x / tiles;
     const int c0 = (blockIdx.x % tiles) * TX<L>();
@@ -1040,17 +1038,17 @@ static cudaError_t chan_spectrum_l(Plan& P) {
     cudaError_t e;
     k_chan_column<<<P.num_sms * 4, 256, 0, P.stream>>>(w.ker, w.r, N);
     PRowsFwdOp a{{}, w.r, u, w.tw_n, N * N, N};
-    if ((e = cudaFuncSetAttribute(k_rows_cg<L, PRowsFwdOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows)))
+    if ((e = cudaFuncSetAttribute(k_rows_post<L, PRowsFwdOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows)))
         return e;
-    k_rows_cg<L, PRowsFwdOp><<<(N * N + ROWS - 1) / ROWS, kThreads, smem_rows, P.stream>>>(a, nullptr);
+    k_rows_post<L, PRowsFwdOp><<<(N * N + ROWS - 1) / ROWS, kThreads, smem_rows, P.stream>>>(a);
     PColsYOp b{u, w.tw_n, N, H, N};
-    if ((e = cudaFuncSetAttribute(k_cols_cg<L, -1, PColsYOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
+    if ((e = cudaFuncSetAttribute(k_cols_plain<L, -1, PColsYOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
         return e;
-    k_cols_cg<L, -1, PColsYOp><<<N * ((H + TX<L>() - 1) / TX<L>()), kThreads, smem_cols, P.stream>>>(b, nullptr);
+    k_cols_plain<L, -1, PColsYOp><<<N * ((H + TX<L>() - 1) / TX<L>()), kThreads, smem_cols, P.stream>>>(b);
     PColsZOp c{u, w.tw_n, 1, N * H};
-    if ((e = cudaFuncSetAttribute(k_cols_cg<L, -1, PColsZOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
+    if ((e = cudaFuncSetAttribute(k_cols_plain<L, -1, PColsZOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
         return e;
-    k_cols_cg<L, -1, PColsZOp><<<(N * H + TX<L>() - 1) / TX<L>(), kThreads, smem_cols, P.stream>>>(c, nullptr);
+    k_cols_plain<L, -1, PColsZOp><<<(N * H + TX<L>() - 1) / TX<L>(), kThreads, smem_cols, P.stream>>>(c);
     P.launches += 4;
     return cudaGetLastError();
 }
@@ -1130,21 +1128,21 @@ static cudaError_t toeplitz_static_l(float2* scratch, const float* khat, const f
     const size_t smem_rows = sizeof(float2) * smem_elems<L, false>(ROWS);
     const size_t smem_cols = sizeof(float2) * smem_elems<L, true>(TX<L>());
     TRowsFwdOp a{{}, x, t1, tw, N * N, N};
-    if ((e = cudaFuncSetAttribute(k_rows_cg<L, TRowsFwdOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows)))
+    if ((e = cudaFuncSetAttribute(k_rows_post<L, TRowsFwdOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows)))
         return e;
-    k_rows_cg<L, TRowsFwdOp><<<(N * N + ROWS - 1) / ROWS, kThreads, smem_rows, s>>>(a, nullptr);
+    k_rows_post<L, TRowsFwdOp><<<(N * N + ROWS - 1) / ROWS, kThreads, smem_rows, s>>>(a);
     TColsYFwdOp b{t1, t2, tw, N, N + 1, N};
-    if ((e = cudaFuncSetAttribute(k_cols_cg<L, -1, TColsYFwdOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
+    if ((e = cudaFuncSetAttribute(k_cols_plain<L, -1, TColsYFwdOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
         return e;
     const int tiles_b = (N + 1 + TX<L>() - 1) / TX<L>();
-    k_cols_cg<L, -1, TColsYFwdOp><<<N * tiles_b, kThreads, smem_cols, s>>>(b, nullptr);
+    k_cols_plain<L, -1, TColsYFwdOp><<<N * tiles_b, kThreads, smem_cols, s>>>(b);
     const int n_inner = 2 * N * (N + 1);
     if ((e = cudaFuncSetAttribute(k_toep_z<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols))) return e;
     k_toep_z<L><<<(n_inner + TX<L>() - 1) / TX<L>(), kThreads, smem_cols, s>>>(t2, khat, tw, n_inner, N, nullptr);
     TColsYInvOp d{t2, t1, tw, N, N + 1, N};
-    if ((e = cudaFuncSetAttribute(k_cols_cg<L, +1, TColsYInvOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
+    if ((e = cudaFuncSetAttribute(k_cols_plain<L, +1, TColsYInvOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cols)))
         return e;
-    k_cols_cg<L, +1, TColsYInvOp><<<N * tiles_b, kThreads, smem_cols, s>>>(d, nullptr);
+    k_cols_plain<L, +1, TColsYInvOp><<<N * tiles_b, kThreads, smem_cols, s>>>(d);
     const float scale = 1.0f / ((float)L * (float)L * (float)L);
     TRowsInvOp f{{}, t1, x, y, tw, N * N, N, scale, lam};
     if ((e = run_rows<L, +1>(f, s)) != cudaSuccess) return e;

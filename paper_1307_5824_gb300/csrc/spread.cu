@@ -11,7 +11,7 @@
 // h b on G = 2N; or both at once on G = 4N):
 //   1. bin:    count points per 8^3 brick (warp-aggregated atomics), scan, and place the
 //              points in per-brick segments cut into work items.
-//   2. spread, in one of two forms by the points per brick (mma_rule):
+//   2. spread, in one of two forms by the points per brick (mma_least):
 //      - bank classes (few): point ids, every item ordered round-robin over the bank
 //        classes; persistent CTAs accumulate an item into an (8 + W)^3 shared-memory
 //        region in int32 fixed point (one native shared atomic per tap), fold it into
@@ -1178,7 +1178,6 @@ static SpreadArgs spread_args(Plan& P, bool kc) {
     a.gid = P.cur_gid;
     a.h2 = w.h2;
     a.samples_b = w.samples_b;
-    a.samples = w.samples;
     a.perm = w.perm;
     a.grid = w.grid;
     a.G = G;

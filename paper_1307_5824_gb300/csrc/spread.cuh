@@ -144,7 +144,6 @@ struct SpreadArgs {
     const int32_t* gid;
     const float* h2;          // kernel channel weights [group][t]
     const float2* samples_b;  // right-hand-side weights in scatter order
-    const float2* samples;    // fused form: the weights h b at [m][t]
     const uint16_t* perm;     // per payload position: the point's index in scatter order
     double* grid;             // G^3 real, or G^3 complex interleaved (re, im)
     int G, halfG, nb, nH, n_ctf;
