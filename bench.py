@@ -807,17 +807,20 @@ def main():
     pts = M * nK
     W = args.W
     nH = (nK + 1) // 2
-    # Spreading time of this form: the fused pass is stage 1, with the placement of its points
-    # (or, in the bank-class form, the gather of their weights) in stage 10; the separate
-    # channels are stages 1 and 6.
+    # Spreading time of this form: the fused pass is stage 1 (with the sorts of its points where
+    # they take several passes), with the placement of its points (or, in the bank-class form, the
+    # gather of their weights) in stage 10; the separate channels are stages 1 and 6.
     spread_ms = stages["spread_ker"] + stages["spread_rhs"] + stages.get("gather_fused", 0.0)
 
     def tensor_form(ch):
-        """Whether the spreading of channel form ch (1 Ker, 2 A*b, 3 both) runs on the tensor
-        cores: the library's rule on the points per brick of the ball (spread.cu, mma_rule)."""
+        """Passes of the spreading of channel form ch (1 Ker, 2 A*b, 3 both) on the tensor cores, 0
+        for bank classes: the library's rule on the points per brick of the ball (spread.cu,
+        mma_least, spread_passes)."""
         least = {6: {1: 600, 2: 400, 3: 235}, 7: {1: 600, 2: 400}}.get(W, {}).get(ch)
-        bricks = 0.5236 * ((2 if ch == 2 else 4) * N / 8) ** 3
-        return least is not None and M * nH >= least * bricks
+        nb = (2 if ch == 2 else 4) * N // 8
+        if least is None or M * nH < least * 0.5236 * nb ** 3 or (W == 7 and M * N * N * 0.3927 > 8.948e7):
+            return 0
+        return -(-(M * nH + (min(nb ** 3, M * nH) + M * nH // 4096) * 420) // 2 ** 26)
 
     def roofline_of(st, is_fused):
         """Rate of the dominant spreading kernel of one channel form.  Tensor-core form: the
@@ -825,7 +828,8 @@ def main():
         cells, 3 products of the fp16 parts, at W = 6; 128 x 8 at W = 7) against the measured
         mma.sync rate, 961 products per clock and SM.  Bank-class form: one shared-memory atomic
         add per tap and channel against one warp-wide shared atomic per clock and SM (10.07e12
-        / s).  DRAM bytes per launch from an ncu capture of this workload (committed with the
+        / s).  In several passes the sorts of the points' records are in the stage's time too.  DRAM
+        bytes of the stage's kernels from an ncu capture of this workload (committed with the
         hash of the spreading source it was taken on; null once that source changed)."""
         if is_fused:
             dom, ch = "spread_ker", 3
@@ -835,6 +839,8 @@ def main():
         mma = tensor_form(ch)
         if mma:
             kname, src_file = f"k_spread_mma<{W},{ch}>", "spread_mma.cu"
+            if mma > 1:
+                kname = f"k_mma_sort + {kname}, {mma} passes"
             peak = 152 * 961 * 2 * 2.07e9
             achieved = M * nH * ch * 3 * (512 if W == 6 else 1024) * 2 / (st[dom] * 1e-3)
             rate = {"bound": "tensor", "unit": "TFLOP/s",
@@ -869,7 +875,9 @@ def main():
     if fused:   # the points placed, sorted into records and spread; or the weights gathered and spread
         spread_bytes = M * nH * (4 * 24 if tensor_form(3) else (4 + 8 + 8) + (4 + 8)) + 3 * Gk ** 3 * 8
     else:
-        spread_bytes = (M * nH * ((16 if tensor_form(1) else 4) + (20 if tensor_form(2) else 4 + 8 + 2))
+        per_point = lambda n, passes: n * (3 if passes > 1 else 1)       # points read, records written and read
+        spread_bytes = (M * nH * ((per_point(16, tensor_form(1)) if tensor_form(1) else 4) +
+                                  (per_point(20, tensor_form(2)) if tensor_form(2) else 4 + 8 + 2))
                         + Gk ** 3 * 8 + Gr ** 3 * 16)
     hbm_peak = None
     try:
