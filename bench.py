@@ -816,8 +816,10 @@ def main():
         """Passes of the spreading of channel form ch (1 Ker, 2 A*b, 3 both) on the tensor cores, 0
         for bank classes: the library's rule on the points per brick of the ball (spread.cu,
         mma_least, spread_passes)."""
-        least = {6: {1: 600, 2: 400, 3: 235}, 7: {1: 600, 2: 400}}.get(W, {}).get(ch)
         nb = (2 if ch == 2 else 4) * N // 8
+        small = nb <= 24
+        least = {6: {1: 600 if small else 800, 2: 400, 3: 235 if small else 290},
+                 7: {1: 600 if small else 660, 2: 400}}.get(W, {}).get(ch)
         if least is None or M * nH < least * 0.5236 * nb ** 3 or (W == 7 and M * N * N * 0.3927 > 8.948e7):
             return 0
         return -(-(M * nH + (min(nb ** 3, M * nH) + M * nH // 4096) * 420) // 2 ** 26)

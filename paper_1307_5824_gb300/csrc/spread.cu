@@ -507,12 +507,16 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 // Average points per brick of the ball from which the tensor-core form is the faster one
 // (binning and spreading together).  Its cost per brick is high -- 25 or 27 classes padded
 // to 16 points, each flushed to the region -- and its cost per point low, the lower the
-// more channels share the window arithmetic.  Measured at N = 64, in ms, bank-class form
-// against tensor-core form.  W = 6: kernel channel 0.70 / 0.77 at 375 points a brick,
-// 0.78 / 0.85 at 469, 1.01 / 0.99 at 657; A*b 0.158 / 0.154 at 226, 0.21 / 0.16 at 450,
-// 0.61 / 0.25 at 1,100; both in one pass 0.80 / 0.99 at 141, 0.91 / 1.02 at 188, 1.22 / 1.11
-// at 281.  W = 7: kernel channel 0.93 / 1.08 at 375, 1.24 / 1.28 at 562, 1.77 / 1.53 at 844;
-// A*b 0.12 / 0.17 at 112, 0.19 / 0.19 at 225, 0.31 / 0.24 at 450.  A*b alone
+// more channels share the window arithmetic.  Measured in ms,
+// bank-class form / tensor-core form.  Kernel channel, W = 6: N = 128 7.25 / 7.60 at 700 points
+// a brick, 8.06 / 8.14 at 800, 8.90 / 8.67 at 900; N = 64 0.98 / 1.01, 1.12 / 1.09, 1.23 / 1.18.
+// Both channels in one pass: N = 128 8.14 / 8.53 at 265, 8.78 / 8.78 at 300, 9.53 / 9.08 at 340;
+// N = 64 1.06 / 1.08 at 235, 1.18 / 1.12 at 265.  Kernel channel, W = 7: N = 96 4.14 / 4.27 at 625,
+// 4.55 / 4.47 at 700; N = 64 1.29 / 1.32 at 600, 1.47 / 1.43 at 700.  A*b: N = 64, W = 6
+// 0.139 / 0.142 at 225, 0.207 / 0.166 at 400; W = 7 0.192 / 0.199, 0.293 / 0.237.  On the small 4N
+// grids, up to 24 bricks an axis (N = 48), the few bricks at the centre hold many times the
+// average and the bank-class form ends with them: 0.52 / 0.44 at 600 (N = 48), 0.30 / 0.18 (N = 32),
+// both in one pass 0.59 / 0.48 at 235 (N = 48); the form is taken from lower averages there.  A*b alone
 // could go over from 225, where the two are level; it does from 400, which leaves at most 0.05 ms.
 // In between lies the undamped N = 32, 200-image workload, whose FP32 CG volume after 10 iterations
 // turns on the last bit of A*b in either form (400 runs with pixels moved by an ulp: median
@@ -531,9 +535,11 @@ static void bin_place_w(Plan& P, const BinArgs& a, int M, bool kc) {
 constexpr double kMmaMostW7 = 8.948e7;
 double mma_least(const firm_params& p, int nb, int ch) {
     double least;
-    if (p.W == 6) least = ch == 1 ? 600.0 : ch == 2 ? 400.0 : 235.0;
-    else if (p.W == 7 && ch < 3 && (double)p.M * p.N * p.N * 0.3927 <= kMmaMostW7) least = ch == 1 ? 600.0 : 400.0;
-    else return 1e300;
+    const bool small = nb <= 24;
+    if (ch == 2) least = 400.0;
+    else if (p.W == 6) least = ch == 1 ? (small ? 600.0 : 800.0) : small ? 235.0 : 290.0;
+    else least = small ? 600.0 : 660.0;
+    if (p.W == 8 || (p.W == 7 && (ch == 3 || (double)p.M * p.N * p.N * 0.3927 > kMmaMostW7))) return 1e300;
     return std::ceil(least * 0.5236 * nb * nb * (double)nb);
 }
 
