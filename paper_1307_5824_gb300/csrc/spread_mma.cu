@@ -27,8 +27,8 @@
 // products per clock and SM) is a quarter busy.  mma.sync and not tcgen05, because both
 // operands are made by the threads that use them, already in registers.
 // Measured at N = 128, 50,000 images, W = 6 (3.2e8 points), binning and spreading together
-// against the bank-class form (with its weight gather): both channels 50.8 -> 26.9 ms, of
-// which the contraction takes 15.1, kernel channel 23.8 -> 16.5 ms, A*b 34.0 -> 18.0 ms.
+// against the bank-class form (with its weight gather): both channels 50.8 -> 27.4 ms, of
+// which the contraction takes 15.0, kernel channel 23.8 -> 17.0 ms, A*b 34.0 -> 18.6 ms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
