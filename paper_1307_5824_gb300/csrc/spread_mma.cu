@@ -96,7 +96,10 @@ static MmaPoly mma_poly(const KbPoly& P, int W) {
 __device__ __forceinline__ uint32_t h2u(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
 __device__ __forceinline__ __half2 u2h(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 
-// (x, y) = hi + lo, hi and lo fp16 pairs: 22 bits, absolute floor 2^-25.
+// (x, y) = hi + lo, hi and lo fp16 pairs: 22 bits, absolute floor 2^-25.  (Splitting FP32 factors for
+// the tensor cores, and adding their sums outside them because they truncate: Ootomo & Yokota,
+// "Recovering single precision accuracy from Tensor Cores while surpassing the FP32
+// theoretical peak performance", 2022.)
 __device__ __forceinline__ void split2(float2 v, uint32_t& hi, uint32_t& lo) {
     const __half2 h = __float22half2_rn(v);
     const float2 f = __half22float2(h);

@@ -60,7 +60,8 @@ def test_conversions_against_the_casts(tmp_path):
     src, exe = tmp_path / "conv.cu", tmp_path / "conv"
     src.write_text(SRC)
     csrc = os.path.join(ROOT, "paper_1307_5824_gb300", "csrc")
-    subprocess.run(["nvcc", "-std=c++17", "-O1", "-gencode", "arch=compute_103a,code=sm_103a", "-I", csrc, str(src),
+    from paper_1307_5824_gb300.build import nvcc
+    subprocess.run([nvcc(), "-std=c++17", "-O1", "-gencode", "arch=compute_103a,code=sm_103a", "-I", csrc, str(src),
                     "-o", str(exe)], check=True, capture_output=True, text=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True)
     assert out.stdout.strip() == "0"

@@ -72,3 +72,29 @@ def test_non_finite_images_are_reported(F, M, fused, value):
     got = rhs(images)
     assert np.linalg.norm(got - want) <= 1e-6 * np.linalg.norm(want)
     rec.close()
+
+
+@pytest.mark.parametrize("M,fused", DENSE)
+def test_host_images(F, M, fused):
+    """Host images, copied in stream order into the memory the points take afterwards, and staged
+    ahead, against the same images on the device (1e-6: the order of the sums)."""
+    N = 16
+    inp = synth.config_inputs("C5", M=M, N=N)
+    rec = F.Reconstructor(N, M, groups=inp["groups"], lam=1e-3, fused=fused)
+    R, gid, shifts = dev(inp["R"].reshape(M, 9)), dev(inp["group_id"]), dev(inp["shifts"])
+    host = torch.from_numpy(inp["images"].astype(np.float32)).pin_memory()
+    got = []
+    for images, stage in ((host.cuda(), False), (host, False), (host, True)):
+        out = torch.empty((N, N, N), device="cuda")
+        if stage:
+            rec.stage_images(images)
+        if fused:
+            rec.kernel_backproject(images, shifts, R, gid, rhs_out=out)
+        else:
+            rec.kernel(R, gid)
+            rec.backproject(images, shifts, R, gid, rhs_out=out)
+        rec.lambda_eff()
+        got.append(out.cpu().numpy().astype(np.float64))
+    for other in got[1:]:
+        assert np.linalg.norm(other - got[0]) <= 1e-6 * np.linalg.norm(got[0])
+    rec.close()
